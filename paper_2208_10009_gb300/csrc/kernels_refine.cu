@@ -48,6 +48,21 @@ cudaError_t upload_subray_table(cudaStream_t s) {
     return cudaMemcpyToSymbolAsync(c_sub, &t, sizeof(t), 0, cudaMemcpyHostToDevice, s);
 }
 
+// The FP64 pattern in shared memory, for kernels whose lanes read different sub-rays at a
+// time (a constant-bank read with several addresses in a warp is replayed per address).
+struct SubTab64 {
+    double rho[38], cphi[38], sphi[38];
+};
+
+__device__ __forceinline__ void load_sub64(SubTab64 &t) {
+    for (int i = threadIdx.x; i < 38; i += blockDim.x) {
+        t.rho[i] = c_sub.rho_d[i];
+        t.cphi[i] = c_sub.cphi_d[i];
+        t.sphi[i] = c_sub.sphi_d[i];
+    }
+    __syncthreads();
+}
+
 struct PathGeo {
     float3 tx, rx;
     dvec3 txd, rxd;
@@ -321,7 +336,8 @@ __device__ __forceinline__ bool aoa_within32(float3 d, float4 P, float4 Wv, cons
 
 __device__ __forceinline__ bool reached(const RefineArgs &A, const PathGeo &g, const UnfD &ud, dvec3 c, double key,
                                         double dw) {
-    if (!(A.target > 0.0 && key < INFINITY && key <= dw * dw * A.tan2_target)) return false;
+    if (!A.target_on || __double_as_longlong(key) >= __double_as_longlong((double)INFINITY)) return false;
+    if (!(key <= dw * dw * A.tan2_target)) return false;
     if (g.wedge < 0 && g.k == 0) return true;
     const float4 *wp = g.wedge >= 0 ? A.scene.wedges + 4 * (size_t)g.wedge : nullptr;
     return aoa_within64(c, wp ? ud.w : ud.p[g.k - 1], ud.w, wp, g.txd, A.tan2_target);
@@ -334,6 +350,9 @@ __device__ __forceinline__ bool reached(const RefineArgs &A, const PathGeo &g, c
 // margin.)
 __device__ __forceinline__ bool stalled(double key, double dw, double R, double stall) {
     if (!(key < INFINITY)) return true;
+    // the angle is at most |d x W| / (d . W): most paths are seen to be inside without it
+    const float t = (float)dw * (float)(R * stall);
+    if ((float)key < 0.999f * t * t && t > 0.0f) return false;
     return atan2f(sqrtf((float)key), (float)dw) > (float)(R * stall + 1e-6);
 }
 
@@ -347,6 +366,8 @@ __device__ __forceinline__ bool reached32(const RefineArgs &A, const PathGeo &g,
 
 __device__ __forceinline__ bool stalled32(float key, float dw, float Rf, float stall) {
     if (!(key < INFINITY)) return true;
+    const float t = dw * (Rf * stall);   // as in stalled
+    if (key < 0.999f * t * t && t > 0.0f) return false;
     return atan2f(sqrtf(key), dw) > Rf * stall + 1e-6f;
 }
 
@@ -404,23 +425,22 @@ __device__ __forceinline__ int frame_axis32(float3 c) {
     return (ay < ax && ay <= az) ? 1 : ((az < ax && az < ay) ? 2 : 0);
 }
 
+// (magnitudes compared as integers, like key64's sign tests)
 __device__ __forceinline__ int frame_axis64(dvec3 c) {
-    double ax = fabs(c.x), ay = fabs(c.y), az = fabs(c.z);
+    const long long ax = __double_as_longlong(fabs(c.x)), ay = __double_as_longlong(fabs(c.y)),
+                    az = __double_as_longlong(fabs(c.z));
     return (ay < ax && ay <= az) ? 1 : ((az < ax && az < ay) ? 2 : 0);
 }
 
-__device__ __forceinline__ void frame32(float3 c, float3 &u, float3 &v) {
-    const int a = frame_axis32(c);
-    const float3 e = make_float3(a == 0, a == 1, a == 2);
-    u = cross(c, e);
+__device__ __forceinline__ void frame32(float3 c, int a, float3 &u, float3 &v) {
+    u = a == 0 ? make_float3(0.0f, c.z, -c.y) : (a == 1 ? make_float3(-c.z, 0.0f, c.x) : make_float3(c.y, -c.x, 0.0f));
     u = u * (1.0f / sqrtf(dot(u, u)));
     v = cross(c, u);
 }
 
 __device__ __forceinline__ void frame64(dvec3 c, dvec3 &u, dvec3 &v) {
     const int a = frame_axis64(c);
-    const dvec3 e = dv(a == 0, a == 1, a == 2);
-    u = dcross(c, e);
+    u = a == 0 ? dv(0.0, c.z, -c.y) : (a == 1 ? dv(-c.z, 0.0, c.x) : dv(c.y, -c.x, 0.0));
     u = u * (1.0 / dnorm(u));
     v = dcross(c, u);
 }
@@ -434,7 +454,7 @@ __device__ __forceinline__ int8_t choice_entry(int bk, int axis) { return (int8_
 __device__ __forceinline__ int iterate32(const UnfF &uf, int nk, int K, int off, float Rf, float3 &cf, float &key_c,
                                          float &dw_c) {
     float3 u, v;
-    frame32(cf, u, v);
+    frame32(cf, frame_axis32(cf), u, v);
     float best = INFINITY, bdw = 0.0f;
     int bk = -1;
     float3 bd = cf;
@@ -464,28 +484,89 @@ __device__ __forceinline__ int iterate32(const UnfF &uf, int nk, int K, int off,
     return bk;
 }
 
-__device__ __forceinline__ int iterate64(const UnfD &ud, int nk, int K, int off, double R, dvec3 &c, double &key_c,
-                                         double &dw_c) {
+// The FP64 iteration.  GB300's FP64 pipe (1/64 of the FP32 rate, conversions included) bounds
+// it, and K exact sub-rays cost K (5 nk + 24) of its operations where the frame and the
+// normalisation cost about 80.  So the sub-rays are first ranked in FP32: d_k x W is linear in
+// the frame,
+//   e_k = ca (c x W) + sa (cos phi_k (u x W) + sin phi_k (v x W)),
+// and with c x W (the part that cancels) taken in FP64, |e_k| comes out within
+//   delta = 1e-5 (sa |W| + |c x W|) + 4e-15 |W|
+// of the square root of key64's value: the FP32 terms round below 2e-6 of their size, and
+// key64's own rounding (of d_k and of the cross product) stays below 2e-15 |W|.  A sub-ray whose
+// |e_k| exceeds the smallest by more than 2 delta has the larger key64, valid or not, so only
+// the others are evaluated, exactly as before: one as a rule, more within about 1e-14 of the
+// double floor.  Should the smallest be invalid (a face met out of order), all K are.
+// Office tail (942,656 paths, K = 16): 935 -> 302 us, FP64 pipe no longer the bound; large city
+// (17.7k paths, 12 FP64 iterations, K = 9): 590 -> 387 us; 4,026 room paths run to the double
+// floor (60 iterations, K = 6), whose FP64 iterations ran in lane groups: 1452 -> 530 us.
+__device__ __forceinline__ int iterate64(const UnfD &ud, int nk, int K, int off, const SubTab64 &tab, double R,
+                                         dvec3 &c, double &key_c, double &dw_c) {
     dvec3 u, v;
     frame64(c, u, v);
+    const dvec3 W = dv(ud.w.x, ud.w.y, ud.w.z), cw = dcross(c, W);
+    const float3 e0 = make_float3((float)cw.x, (float)cw.y, (float)cw.z);
+    const float3 Wf = make_float3((float)W.x, (float)W.y, (float)W.z);
+    float3 uW, vW;
+    {
+        const float3 cf = make_float3((float)c.x, (float)c.y, (float)c.z);
+        float3 uf, vf;
+        frame32(cf, frame_axis64(c), uf, vf);
+        uW = cross(uf, Wf);
+        vW = cross(vf, Wf);
+    }
+    const float Rf = (float)R, nW = sqrtf(dot(Wf, Wf));
+    float rho = -1.0f, sa = 0.0f, ca = 1.0f, samax = 0.0f, a1 = INFINITY, a2 = INFINITY;
+    auto ranked = [&](int k) {   // |e_k|^2; the patterns' sub-rays come ring by ring
+        if (c_sub.rho[off + k] != rho) {
+            rho = c_sub.rho[off + k];
+            sincos_sub32(rho * Rf, sa, ca);
+        }
+        const float3 e = e0 * ca + (uW * c_sub.cphi[off + k] + vW * c_sub.sphi[off + k]) * sa;
+        return dot(e, e);
+    };
+    int k1 = 0;
+    for (int k = 0; k < K; ++k) {
+        const float a = ranked(k);
+        samax = fmaxf(samax, sa);
+        a2 = fminf(a2, fmaxf(a, a1));
+        if (a < a1) {
+            a1 = a;
+            k1 = k;
+        }
+    }
+    const float delta = 1e-5f * (samax * nW + sqrtf(dot(e0, e0))) + 4e-15f * nW + 1e-18f;
+    const float lim = sqrtf(a1) + 2.0f * delta;
+    const float thr = lim * lim * 1.00001f;   // a sub-ray beyond it cannot win (never so for a NaN)
+    unsigned left = 1u << k1;                 // the sub-rays to evaluate
+    if (!(a2 > thr)) {
+        rho = -1.0f;
+        for (int k = 0; k < K; ++k)
+            if (!(ranked(k) > thr)) left |= 1u << k;
+    }
     double best = INFINITY, bdw = 0.0;
     int bk = -1;
     dvec3 bd = c;
-    double rho = -1.0, sa = 0.0, ca = 1.0;
-    for (int k = 0; k < K; ++k) {
-        if (c_sub.rho_d[off + k] != rho) {
-            rho = c_sub.rho_d[off + k];
-            sincos_sub(rho * R, sa, ca);
-        }
-        dvec3 dk = c * ca + (u * c_sub.cphi_d[off + k] + v * c_sub.sphi_d[off + k]) * sa;
+    for (bool first = true; left;) {   // lowest k first: the plain rule on ties
+        const int k = __ffs(left) - 1;
+        left &= left - 1;
+        double s, co;
+        sincos_sub(tab.rho[off + k] * R, s, co);
+        const dvec3 dk = c * co + (u * tab.cphi[off + k] + v * tab.sphi[off + k]) * s;
         double dw = 0.0;
-        double key = key64(ud, nk, dk, dw);
+        const double key = key64(ud, nk, dk, dw);
         // key < best, both >= 0 (or +inf): their bits order like the values
         if (__double_as_longlong(key) < __double_as_longlong(best)) {
             best = key;
             bdw = dw;
             bk = k;
             bd = dk;
+        }
+        if (first && k == k1 && !(__double_as_longlong(key) < __double_as_longlong((double)INFINITY))) {
+            // the nearest is invalid, so the margin says nothing: take all, from the start
+            first = false;
+            left = (1u << K) - 1u;
+            best = INFINITY;
+            bk = -1;
         }
     }
     if (bk >= 0) {
@@ -816,6 +897,8 @@ __global__ void __launch_bounds__(256) refine_kernel(RefineArgs A) {
     const float shrinkf = c_sub.shrink_f[A.K];
     const double stall = 1.0 / (1.0 - shrink) + 2.0 * shrink;
     const float stallf = (float)stall;
+    __shared__ SubTab64 tab;
+    load_sub64(tab);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         long long pi = A.range ? (long long)A.index[A.range[0] + i] : i;
@@ -882,7 +965,7 @@ __global__ void __launch_bounds__(256) refine_kernel(RefineArgs A) {
                     break;
                 }
                 const int ax = A.choice_log ? frame_axis64(c) : 0;
-                const int bk = iterate64(ud, g.k, A.K, off, R, c, key, dw);
+                const int bk = iterate64(ud, g.k, A.K, off, tab, R, c, key, dw);
                 if (bk < 0) {
                     fail = true;
                     break;
@@ -945,23 +1028,10 @@ __device__ __forceinline__ void group_argmin(float &e, int &k, unsigned gmask) {
 }
 
 template <int G>
-__device__ __forceinline__ void group_argmin64(double &e, int &k, unsigned gmask) {
-#pragma unroll
-    for (int off = G / 2; off > 0; off >>= 1) {
-        double e2 = __shfl_xor_sync(gmask, e, off, G);
-        int k2 = __shfl_xor_sync(gmask, k, off, G);
-        if (e2 < e || (e2 == e && k2 < k)) {
-            e = e2;
-            k = k2;
-        }
-    }
-}
-
-template <int G>
 __device__ __forceinline__ int group_iterate32(const UnfF &uf, int nk, int K, int off, float Rf, float3 &cf,
                                                float &key_c, float &dw_c, int gl, unsigned gmask) {
     float3 u, v;
-    frame32(cf, u, v);
+    frame32(cf, frame_axis32(cf), u, v);
     float best = INFINITY;
     int bk = 0x7fffffff;
     for (int k = gl; k < K; k += G) {
@@ -990,44 +1060,10 @@ __device__ __forceinline__ int group_iterate32(const UnfF &uf, int nk, int K, in
     return bk;
 }
 
-template <int G>
-__device__ __forceinline__ int group_iterate64(const UnfD &ud, int nk, int K, int off, double R, dvec3 &c,
-                                               double &key_c, double &dw_c, int gl, unsigned gmask) {
-    dvec3 u, v;
-    frame64(c, u, v);
-    double best = INFINITY;
-    int bk = 0x7fffffff;
-    for (int k = gl; k < K; k += G) {
-        double sa, ca;
-        sincos_sub(c_sub.rho_d[off + k] * R, sa, ca);
-        dvec3 dk = c * ca + (u * c_sub.cphi_d[off + k] + v * c_sub.sphi_d[off + k]) * sa;
-        double dw;
-        double key = key64(ud, nk, dk, dw);
-        if (key < best) {
-            best = key;
-            bk = k;
-        }
-    }
-    group_argmin64<G>(best, bk, gmask);
-    if (!(best < INFINITY)) return -1;
-    double sa, ca;
-    sincos_sub(c_sub.rho_d[off + bk] * R, sa, ca);
-    dvec3 bd = c * ca + (u * c_sub.cphi_d[off + bk] + v * c_sub.sphi_d[off + bk]) * sa;
-    double dw = 0.0;
-    double key = key64(ud, nk, bd, dw);
-    c = bd * (1.0 / dnorm(bd));
-    key_c = key;
-    dw_c = dw;
-    return bk;
-}
-
 // Validity and outputs with the per-bounce / per-segment queries spread over the group.
-// Lane 0 traces the bounce points once (FP64) and shares them through the group's slot
-// of shared memory (sh.p[j] = (p_j, den_j), sh.w = (direction of the last leg, sum of
-// the segment parameters, or -1 if the trace failed)).
 template <int G>
 __device__ void group_finalize(const RefineArgs &A, const PathGeo &g, dvec3 c, sbr_path_record &p, int gl,
-                               unsigned gmask, double err_bound, UnfD &sh) {
+                               unsigned gmask, double err_bound) {
     const SceneDev &S = A.scene;
     if (g.wedge >= 0) {   // group-uniform: one path per group
         if (gl == 0) wedge_finalize(A, g, c, p, err_bound);
@@ -1080,18 +1116,15 @@ __device__ void group_finalize(const RefineArgs &A, const PathGeo &g, dvec3 c, s
 template <int G>
 __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
     // the unfolded planes of each group's current path (shared by its G lanes)
-    __shared__ UnfD s_ud[G == 1 ? 1 : 256 / G];
     __shared__ UnfF s_uf[256 / G];
-    UnfD &ud = s_ud[G == 1 ? 0 : threadIdx.x / G];   // unused by the one-lane form
     UnfF &uf = s_uf[threadIdx.x / G];
     const long long total = path_count(A);
     // batch_unfold_kernel ran (the one-lane form always runs with it: split_min = 0)
     const bool prebuilt = G == 1 || total >= A.split_min;
     const int off = c_sub.off[A.K];
-    const double shrink = c_sub.shrink[A.K];
     const float shrinkf = c_sub.shrink_f[A.K];
-    const double stall = 1.0 / (1.0 - shrink) + 2.0 * shrink;
-    const float stallf = (float)stall;
+    const double shrink = c_sub.shrink[A.K];
+    const float stallf = (float)(1.0 / (1.0 - shrink) + 2.0 * shrink);
     const int lane = threadIdx.x & 31;
     const int gl = lane % G;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (lane - gl));
@@ -1132,14 +1165,8 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
                 if (j < g.k || j == kMaxOrder) (j < kMaxOrder ? uf.p[j] : uf.w) = A.unf[kUnfStride * pi + j];
             cf = f3(A.unf[kUnfStride * pi + kMaxOrder + 1]);
         } else {
-            for (int j = gl; j < g.k; j += G) {
-                ud.p[j] = unfold_plane(A.scene, g, j);
-                uf.p[j] = unfold_plane32(A.scene, g, j);
-            }
-            if (gl == G - 1) {
-                ud.w = unfold_rx(A.scene, g);
-                uf.w = unfold_rx32(A.scene, g);
-            }
+            for (int j = gl; j < g.k; j += G) uf.p[j] = unfold_plane32(A.scene, g, j);
+            if (gl == G - 1) uf.w = unfold_rx32(A.scene, g);
             cf = make_float3((float)p.dir[0], (float)p.dir[1], (float)p.dir[2]);
         }
         __syncwarp(gmask);
@@ -1172,20 +1199,18 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
                 ++it;
             }
         }
-        dvec3 c;
-        double key = INFINITY, dw = 0.0;
-        if (!fail && Rf < A.fp64_below_f && prebuilt) {
-            // many paths: the FP64 iterations run in batch_refine64_kernel, one thread per
-            // path.  The record keeps the iterations done; the path's unf slot keeps the
-            // cone centre and |d x W|^2 of the FP32 phase, the record's err field d . W.
-            // Listed by order group (group offsets from batch_unfold_kernel's counts), so that
-            // the tail kernel's warps run paths of one order.
+        if (!fail && Rf < A.fp64_below_f) {
+            // the FP64 iterations run in batch_refine64_kernel, one thread per path.  The
+            // record keeps the iterations done; the path's unf slot keeps the cone centre and
+            // |d x W|^2 of the FP32 phase, the record's err field d . W.  With many paths listed
+            // by order group (group offsets from batch_unfold_kernel's counts), so that the
+            // tail kernel's warps run paths of one order; with few in one group.
             if (gl == 0) {
                 sbr_path_record *dst = A.paths + pi;
                 dst->iters = it;
                 dst->err = dwf;
                 A.unf[kUnfStride * pi + kMaxOrder + 1] = make_float4(cf.x, cf.y, cf.z, keyf);
-                const int grp = order_group(g);
+                const int grp = prebuilt ? order_group(g) : 0;
                 unsigned long long at = 0;
                 for (int b = 0; b < grp; ++b) at += A.order_cnt[b];
                 at += atomicAdd(A.order_cnt + 32 + grp, 1ULL);
@@ -1193,79 +1218,52 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
             }
             continue;
         }
-        if (G != 1 && !fail && Rf < A.fp64_below_f) {
-            double R = cone_radius64(A, p.rough_err, it, shrink);
-            if (fp64) {
-                c = dv(p.dir[0], p.dir[1], p.dir[2]);
-                key = key64(ud, g.k, c, dw);
-            } else {
-                c = dv(cf.x, cf.y, cf.z);
-                key = keyf;
-                dw = dwf;
-            }
-            stop = kStopNone;   // the FP64 phase judges the state again
-            while (it < A.max_iters) {
-                if (reached(A, g, ud, c, key, dw)) {
-                    stop = kStopReached;
-                    break;
-                }
-                if (stalled(key, dw, R, stall)) {
-                    stop = kStopStalled;
-                    break;
-                }
-                const int ax = A.choice_log ? frame_axis64(c) : 0;
-                const int bk = group_iterate64<G>(ud, g.k, A.K, off, R, c, key, dw, gl, gmask);
-                if (bk < 0) {
-                    fail = true;
-                    break;
-                }
-                flags |= SBR_PATH_FP64;
-                fp64 = true;
-                if (A.choice_log && gl == 0) A.choice_log[pi * A.max_iters + it] = choice_entry(bk, ax);
-                R *= shrink;
-                ++it;
-            }
-        }
         if (fail) flags |= SBR_PATH_TRACE_FAIL;
         else if (stop == kStopStalled) flags |= SBR_PATH_STALLED;
         if (gl == 0) {
-            if (!fp64) c = dv(cf.x, cf.y, cf.z);
-            p.iters = it;
-            p.flags = flags | (it > 0 ? SBR_PATH_REFINED : 0);
-            p.dir[0] = c.x;
-            p.dir[1] = c.y;
-            p.dir[2] = c.z;
-            p.err = error_angle(key, dw, keyf, dwf, fp64);
+            p.err = error_angle(INFINITY, 0.0, keyf, dwf, false);
             if (prebuilt) list_for_finalize(A, g, pi, p.err, (double)Rf);
             // iteration results; the validity test and outputs follow in batch_finalize_kernel
             sbr_path_record *dst = A.paths + pi;
-            dst->iters = p.iters;
-            dst->dir[0] = p.dir[0];
-            dst->dir[1] = p.dir[1];
-            dst->dir[2] = p.dir[2];
+            dst->iters = it;
+            dst->dir[0] = cf.x;
+            dst->dir[1] = cf.y;
+            dst->dir[2] = cf.z;
             dst->err = p.err;
-            dst->flags = p.flags;
+            dst->flags = flags | (it > 0 ? SBR_PATH_REFINED : 0);
         }
     }
 }
 
-// Batched form, FP64 tail (from split_min paths on), one thread per path: the paths whose
-// cone fell below fp64_below in batch_refine_kernel continue here with the plain form's
-// FP64 iterations (iterate64, all K sub-rays in one thread), so that each instruction of
-// GB300's narrow FP64 pipe serves 32 paths, where a lane group serves one.  The state
-// carried over, and the arithmetic, are those of the in-group FP64 phase: a path that
-// started in FP64 (no iteration done) takes its FP64 rough direction; otherwise the FP32
-// phase's centre with its |d x W|^2 and d . W.  The path is then listed in its order group
-// for batch_finalize_kernel.
-__global__ void __launch_bounds__(128) batch_refine64_kernel(RefineArgs A) {
+// Batched form, FP64 tail, one thread per path: the paths whose cone fell below fp64_below in
+// batch_refine_kernel continue here with the plain form's FP64 iterations (iterate64), so that
+// each instruction of GB300's narrow FP64 pipe serves 32 paths, where a lane group would serve
+// one.  The state carried over: a path that started in FP64 (no iteration done) takes its FP64
+// rough direction; otherwise the FP32 phase's centre with its |d x W|^2 and d . W.  With many
+// paths the path is then listed in its order group for batch_finalize_kernel.  One warp a
+// block: the FP64 pipe belongs to the SM, so a short list (the large city's 17k paths are 535
+// warps) has to spread over as many SMs as it has warps.  A list of at most kTailWide paths an
+// SM takes a warp a path instead: its lanes unfold the planes side by side and then iterate
+// in step, which spares the waits of one thread's chain of mirrors (canyon, 631 paths with one
+// FP64 iteration each: 14 against 20 us a launch) and the divergence of its iterations;
+// with more paths the pipe is full of redundant lanes (8 paths an SM cost what a thread a path does).
+constexpr int kTailBlock = 32, kTailWide = 6;
+__global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A) {
+    const bool many = path_count(A) >= A.split_min;
+    __shared__ SubTab64 tab;
     // the list holds group b's n_b paths from the group's offset (the sizes of groups < b)
     long long n = 0;
     for (int b = 0; b < 10; ++b) n += A.order_cnt[32 + b];
+    if (n == 0) return;
+    load_sub64(tab);
     const int off = c_sub.off[A.K];
     const double shrink = c_sub.shrink[A.K];
     const double stall = 1.0 / (1.0 - shrink) + 2.0 * shrink;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
+    __shared__ UnfD s_ud;
+    const int lane = threadIdx.x;
+    const bool wide = n <= kTailWide * (long long)A.num_sms;
+    const long long per = wide ? 1 : kTailBlock;   // paths a warp
+    for (long long t = blockIdx.x * per + (wide ? 0 : lane); t < n; t += gridDim.x * per) {
         long long slot = t, base = 0;
         for (int b = 0; b < 10; ++b) {
             const long long nb = (long long)A.order_cnt[32 + b];
@@ -1279,8 +1277,17 @@ __global__ void __launch_bounds__(128) batch_refine64_kernel(RefineArgs A) {
         load_path(A, p, g);
         UnfD ud;
         const float4 *u = A.unf + kUnfStride * pi;
-        for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
-        ud.w = unfold_rx(A.scene, g);
+        if (wide) {
+            __syncwarp();
+            if (lane < g.k) s_ud.p[lane] = unfold_plane(A.scene, g, lane);
+            if (lane == kTailBlock - 1) s_ud.w = unfold_rx(A.scene, g);
+            __syncwarp();
+            for (int j = 0; j < g.k; ++j) ud.p[j] = s_ud.p[j];
+            ud.w = s_ud.w;
+        } else {
+            for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
+            ud.w = unfold_rx(A.scene, g);
+        }
         const float4 cu = u[kMaxOrder + 1];
         const float3 cf = f3(cu);
         const float keyf = cu.w, dwf = (float)p.err;
@@ -1308,22 +1315,23 @@ __global__ void __launch_bounds__(128) batch_refine64_kernel(RefineArgs A) {
                 break;
             }
             const int ax = A.choice_log ? frame_axis64(c) : 0;
-            const int bk = iterate64(ud, g.k, A.K, off, R, c, key, dw);
+            const int bk = iterate64(ud, g.k, A.K, off, tab, R, c, key, dw);
             if (bk < 0) {
                 fail = true;
                 break;
             }
             flags |= SBR_PATH_FP64;
             fp64 = true;
-            if (A.choice_log) A.choice_log[pi * A.max_iters + it] = choice_entry(bk, ax);
+            if (A.choice_log && (!wide || lane == 0)) A.choice_log[pi * A.max_iters + it] = choice_entry(bk, ax);
             R *= shrink;
             ++it;
         }
         if (fail) flags |= SBR_PATH_TRACE_FAIL;
         else if (stop == kStopStalled) flags |= SBR_PATH_STALLED;
         if (!fp64) c = dv(cf.x, cf.y, cf.z);
+        if (wide && lane != 0) continue;   // the lanes agree
         const double err = error_angle(key, dw, keyf, dwf, fp64);
-        list_for_finalize(A, g, pi, err, R);
+        if (many) list_for_finalize(A, g, pi, err, R);
         sbr_path_record *dst = A.paths + pi;
         dst->iters = it;
         dst->dir[0] = c.x;
@@ -1374,7 +1382,6 @@ __global__ void __launch_bounds__(128) batch_unfold_kernel(RefineArgs A) {
 // faster than the occlusion queries split into a kernel of their own with a thread per
 // (path, leg) (which walks each path again for every leg).
 __global__ void __launch_bounds__(128, 8) batch_finalize_kernel(RefineArgs A) {
-    __shared__ UnfD s_sh[4];
     const long long total = path_count(A);
     const double shrink = c_sub.shrink[A.K];
     const bool per_thread = total >= A.split_min;
@@ -1399,7 +1406,7 @@ __global__ void __launch_bounds__(128, 8) batch_finalize_kernel(RefineArgs A) {
             store_result(A.paths + pi, p);
         } else {
             const int lane = threadIdx.x & 31;
-            group_finalize<32>(A, g, c, p, lane, 0xffffffffu, converged_bound(p.iters, R), s_sh[threadIdx.x >> 5]);
+            group_finalize<32>(A, g, c, p, lane, 0xffffffffu, converged_bound(p.iters, R));
             if (lane == 0) store_result(A.paths + pi, p);
         }
     }
@@ -1461,12 +1468,12 @@ cudaError_t launch_batch_refine(const RefineArgs &a, int grid, int block, cudaSt
     if (e != cudaSuccess) return e;
     static int tail_blocks = 0;
     if (!tail_blocks) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tail_blocks, batch_refine64_kernel, 128, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tail_blocks, batch_refine64_kernel, kTailBlock, 0);
         if (tail_blocks < 1) tail_blocks = 1;
     }
     {
         Range r("batch refine: FP64 tail");
-        batch_refine64_kernel<<<sms * tail_blocks, 128, 0, s>>>(a);
+        batch_refine64_kernel<<<sms * tail_blocks, kTailBlock, 0, s>>>(a);
     }
     static int fin_blocks = 0;
     if (!fin_blocks) {

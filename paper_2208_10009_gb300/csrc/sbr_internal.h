@@ -340,6 +340,7 @@ struct RefineArgs {
     int chunk;                // lanes per path in the batched kernel (8, 16, 32)
     long long split_min;      // batched form: from this many paths on, validity and outputs run
                               // one thread per path in a second kernel
+    int num_sms;
     int ntx, nrx, nf, nw;     // bounds of the ids a path record may hold
 };
 cudaError_t launch_refine(const RefineArgs &a, int grid, int block, cudaStream_t s);
