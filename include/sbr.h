@@ -199,8 +199,8 @@ typedef struct {
                                    ids stay the lattice's own (position-independent records) */
 #define SBR_LAUNCH_RECORDS_ONLY 16 /* stop after the reception judgment: the container keeps the
                                       reception records (sbr_records_read) and no paths */
-#define SBR_LAUNCH_ID_ORDER 32 /* trace the rays in lattice id order.  By default a launch of a
-                                  whole equiangular lattice takes them in compact tiles of
+#define SBR_LAUNCH_ID_ORDER 32 /* trace the rays in lattice id order.  By default a launch of
+                                  the equiangular lattice takes them in compact tiles of
                                   each face's triangular grid (neighbouring directions together
                                   in a warp); the results are the same either way (§III.A:
                                   rays are independent) */

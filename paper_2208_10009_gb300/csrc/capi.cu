@@ -175,11 +175,11 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher) {
     if (launcher == 0) {
         sbr_status st = ensure_lattice(ctx, n);
         if (st != SBR_OK) return st;
-        SBR_CUDA(launch_raygen(ctx->lattice, static_cast<float4 *>(ctx->dirs), N, ctx->stream));
+        SBR_CUDA(launch_raygen_schedule(ctx->lattice, static_cast<float4 *>(ctx->dirs), ctx->stream));
     } else {
         sbr_status st = ensure_poly(ctx, launcher, n);
         if (st != SBR_OK) return st;
-        SBR_CUDA(launch_raygen_equidistant(ctx->poly, static_cast<float4 *>(ctx->dirs), N, ctx->stream));
+        SBR_CUDA(launch_raygen_equidistant(ctx->poly, static_cast<float4 *>(ctx->dirs), N, true, ctx->stream));
     }
     ctx->dirs_n = n;
     ctx->dirs_launcher = launcher;
@@ -255,7 +255,7 @@ sbr_status sbr_raygen_equidistant(sbr_ctx *ctx, int32_t n, int32_t poly, float *
     DeviceGuard g(ctx->device);
     sbr_status st = ensure_poly(ctx, poly, n);
     if (st != SBR_OK) return st;
-    SBR_CUDA(launch_raygen_equidistant(ctx->poly, reinterpret_cast<float4 *>(dirs), N, ctx->stream));
+    SBR_CUDA(launch_raygen_equidistant(ctx->poly, reinterpret_cast<float4 *>(dirs), N, false, ctx->stream));
     return SBR_OK;
 }
 
@@ -734,6 +734,7 @@ static DedupArgs dedup_args(sbr_ctx *ctx, sbr_paths *paths, int nrx, int rank, i
     d.paths = paths->paths;
     d.path_cap = paths->path_cap;
     d.dirs = static_cast<const float4 *>(ctx->dirs);
+    d.sched_n = paths->launcher == 0 ? paths->n_div : 0;
     d.counters = paths->counters;
     d.nrx = nrx;
     d.shard_rank = rank;
@@ -787,8 +788,20 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     a.dirs = static_cast<const float4 *>(ctx->dirs);
     a.tx = paths->tx;
     a.ntx = ntx;
-    a.nrays_per_tx = ray_count;
-    a.ray_begin = ray_begin;
+    a.ray_begin = (int)ray_begin;
+    a.ray_end = (int)(ray_begin + ray_count);
+    a.id_order_n = prm->launcher == 0 && (prm->flags & SBR_LAUNCH_ID_ORDER) ? prm->n_div : 0;
+    a.first = ray_begin;
+    a.count = ray_count;
+    if (prm->launcher == 0 && !a.id_order_n && ray_count > 0 && ray_count < N) {
+        // a range of ids on the schedule: whole faces, of which the ids outside the range are
+        // passed over (the range cuts at most its first and last face)
+        const int64_t E = 12 + 30LL * (prm->n_div - 1), per = (int64_t)(prm->n_div - 1) * (prm->n_div - 2) / 2;
+        if (ray_begin >= E) a.first = E + (ray_begin - E) / per * per;
+        const int64_t last = a.ray_end - 1;
+        a.count = (last < E ? a.ray_end : E + ((last - E) / per + 1) * per) - a.first;
+    }
+    a.inv_count = a.count > 0 ? 1.0f / (float)a.count : 0.0f;
     a.max_order = prm->max_order;
     double cone = prm->rx_angle_scale * sbr_theta_launch(prm->n_div);
     a.cone = (float)cone;
@@ -801,8 +814,6 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     a.dump_faces = prm->dump_faces;
     a.dump_per_tx = prm->dump_stride > 0 ? (N + prm->dump_stride - 1) / prm->dump_stride : 0;
     a.refill_min = prm->refill_min > 0 ? std::min(prm->refill_min, 32) : 24;
-    a.tiled_n = (prm->launcher == 0 && ray_begin == 0 && ray_count == N && !(prm->flags & SBR_LAUNCH_ID_ORDER))
-                    ? prm->n_div : 0;
     int block = prm->block_threads > 0 ? prm->block_threads : 128;
     if (block % 32 != 0 || block > 128)
         return fail(ctx, SBR_EINVAL, "sbr_launch: block_threads must be a multiple of 32, at most 128");
@@ -819,8 +830,11 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
         df.dirs = a.dirs;
         df.tx = paths->tx;
         df.ntx = ntx;
-        df.nrays_per_tx = ray_count;
-        df.ray_begin = ray_begin;
+        df.first = a.first;
+        df.count = a.count;
+        df.ray_begin = a.ray_begin;
+        df.ray_end = a.ray_end;
+        df.id_order_n = a.id_order_n;
         df.cone = a.cone;
         df.tan_cone = a.tan_cone;
         df.recs = paths->recs;
@@ -829,13 +843,14 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
         // the candidate list borrows the dedup table, which is cleared after this step
         df.cand = reinterpret_cast<float4 *>(paths->table);
         df.cand_cap = paths->table_slots * 5 / 8;
-        df.tiled_n = a.tiled_n;
         Range r("sbr_launch: diffraction");
         SBR_CUDA(launch_diffract(df, ctx->num_sms, ctx->stream));
     }
     if (timing) SBR_CUDA(cudaEventRecord(ctx->ev[4], ctx->stream));
     paths->trace_grid = grid;
     paths->trace_block = block;
+    paths->n_div = prm->n_div;
+    paths->launcher = prm->launcher;
     if (!(prm->flags & SBR_LAUNCH_RECORDS_ONLY)) {
         DedupArgs d = dedup_args(ctx, paths, rx->dev.nrx, 0, 1);
         Range r("sbr_launch: dedup");
@@ -845,8 +860,6 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     paths->timed = timing;
     paths->ntx = ntx;
     paths->nrx = rx->dev.nrx;
-    paths->n_div = prm->n_div;
-    paths->launcher = prm->launcher;
     paths->max_order = prm->max_order;
     paths->rx = rx;
     paths->alpha = prm->rx_angle_scale;

@@ -89,12 +89,12 @@ __device__ __forceinline__ bool cone_box(float lx, float ly, float lz, float hx,
 }
 
 // Pass 1, one thread per (Tx, ray): candidate wedges of the ray (edge point X inside the
-// cone, ahead of Tx, Tx in the exterior), appended to the candidate list as (X, ray) and
+// cone, ahead of Tx, Tx in the exterior), appended to the candidate list as (X, place) and
 // (tx, wedge).  The walk advances one node or one wedge per loop turn, so the lanes of a
 // warp append their candidates together (one atomic per turn).
 __global__ void __launch_bounds__(128) diffract_candidates(DiffractArgs A) {
     const SceneDev &S = A.scene;
-    const long long total = (long long)A.ntx * A.nrays_per_tx;
+    const long long total = (long long)A.ntx * A.count;
     const int lane = threadIdx.x & 31;
     unsigned tests = 0;
     // grid-stride in whole warps so that every lane reaches the warp-wide votes
@@ -102,11 +102,14 @@ __global__ void __launch_bounds__(128) diffract_candidates(DiffractArgs A) {
          base += (long long)gridDim.x * blockDim.x) {
         const long long i = base + lane;
         bool done = i >= total, tail = false;
-        const int txi = done ? 0 : (int)(i / A.nrays_per_tx);
-        const int local = done ? 0 : (int)(i - (long long)txi * A.nrays_per_tx);
-        const int ray = A.tiled_n > 0 ? tiled_ray(local, A.tiled_n) : (int)A.ray_begin + local;
+        const int txi = done ? 0 : (int)(i / A.count);
+        int place = (int)A.first + (done ? 0 : (int)(i - (long long)txi * A.count));
+        if (A.id_order_n > 0) place = schedule_place(place, A.id_order_n);
         const float3 o = f3(__ldg(A.tx + txi));
-        const float3 d = f3(__ldg(A.dirs + ray));
+        const float4 dd = __ldg(A.dirs + place);
+        const float3 d = f3(dd);
+        const int ray = __float_as_int(dd.w);
+        done = done || ray < A.ray_begin || ray >= A.ray_end;
         const RayPre r = make_ray(o, d);
         const float od = dot(o, d);
         int stack[kStackDepth];
@@ -167,7 +170,7 @@ __global__ void __launch_bounds__(128) diffract_candidates(DiffractArgs A) {
                 if (cand >= 0) {
                     const long long slot = (long long)at + __popc(want & ((1u << lane) - 1u));
                     if (slot < A.cand_cap) {
-                        A.cand[2 * slot] = make_float4(X.x, X.y, X.z, __int_as_float(ray));
+                        A.cand[2 * slot] = make_float4(X.x, X.y, X.z, __int_as_float(place));
                         A.cand[2 * slot + 1] = make_float4(__int_as_float(txi), __int_as_float(cand), 0.0f, 0.0f);
                     }
                 }
@@ -218,10 +221,11 @@ __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
                                           __shfl_sync(0xffffffffu, c0.z, src), __shfl_sync(0xffffffffu, c0.w, src));
             const int txi = __float_as_int(__shfl_sync(0xffffffffu, c1.x, src));
             const int id = __float_as_int(__shfl_sync(0xffffffffu, c1.y, src));
-            const int ray = __float_as_int(x0.w);
             const WedgeF w = load_wedge(S, id);
             const float3 o = f3(__ldg(A.tx + txi));
-            const float3 d = f3(__ldg(A.dirs + ray));
+            const float4 dd = __ldg(A.dirs + __float_as_int(x0.w));
+            const float3 d = f3(dd);
+            const int ray = __float_as_int(dd.w);
             const float3 X = f3(x0);
             const float3 eb = w.b - w.a;
             const float3 e = eb * (1.0f / sqrtf(dot(eb, eb)));

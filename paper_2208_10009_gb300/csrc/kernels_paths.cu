@@ -5,6 +5,7 @@
 // (error-angle bits, ray id); a second pass checks every record against its slot's
 // winner so that a hash collision is detected, never silently merged.
 #include "dedup_keys.cuh"
+#include "lattice_order.cuh"
 #include "sbr_device.cuh"
 
 namespace sbr {
@@ -75,7 +76,7 @@ __global__ void dedup_select(DedupArgs a) {
         out.rough_dray = r.dray;
         out.iters = 0;
         out.valid = 0;
-        float4 d = __ldg(a.dirs + r.ray);
+        float4 d = __ldg(a.dirs + (a.sched_n > 0 ? schedule_place(r.ray, a.sched_n) : r.ray));
         out.dir[0] = d.x;
         out.dir[1] = d.y;
         out.dir[2] = d.z;

@@ -61,6 +61,60 @@ __global__ void raygen_kernel(LatticeDev L, float4 *__restrict__ dirs, int N) {
     }
 }
 
+// The same rays at their places of the schedule, with their ids: the trace then reads a
+// refill's rays as they lie, where it used to map each place to an id and a 64-bit work index to
+// a transmitter by division (about 150 of the 560 instructions it spent on a segment besides its
+// tree walk), once per transmitter.  A block takes one block of rows of a face (or 256 of the
+// vertex and edge rays): the layer, side and place of a point follow from its grid coordinates,
+// where the id order needs a quadratic search per ray.  Bound by the two sines and the
+// divisions of arc_point, not by its 16 bytes a ray: n = 2200 (48.4M rays) 395 -> 297 us
+// (2.6 TB/s); with it the large city's trace 37.22 -> 36.19 ms, the canyon's 852 -> 822 us, and a
+// quarter range of the city's rays, in id order before, 16.27 -> 14.55 ms.
+__global__ void __launch_bounds__(256) raygen_schedule_kernel(LatticeDev L, float4 *__restrict__ dirs, int edge_blocks,
+                                                              int row_blocks) {
+    const int n = L.n, E = 12 + 30 * (n - 1);
+    if ((int)blockIdx.x < edge_blocks) {
+        const int id = blockIdx.x * 256 + threadIdx.x;
+        if (id >= E) return;
+        float3 d;
+        if (id < 12) {
+            d = f3(__ldg(L.ico + id));
+        } else {
+            int r = id - 12;
+            int e = r / (n - 1), j = r - e * (n - 1) + 1;
+            int2 ed = __ldg(L.edges + e);
+            d = arc_point(f3(__ldg(L.ico + ed.x)), f3(__ldg(L.ico + ed.y)), L.edge_angle, j, n);
+        }
+        dirs[id] = make_float4(d.x, d.y, d.z, __int_as_float(id));
+        return;
+    }
+    const int item = blockIdx.x - edge_blocks, f = item / row_blocks;
+    const RowBlock b = row_block(n, item - f * row_blocks);
+    const int base = E + f * ((n - 1) * (n - 2) / 2), points = b.full + b.stair;
+    float4 *out = dirs + base + b.first;
+    for (int q = threadIdx.x; q < points; q += 256) {
+        int p0, p1;
+        block_point(n, b, q, p0, p1);
+        const GridPoint g = grid_point(n, p0, p1);
+        float3 d;
+        if (g.m == 0) {
+            d = f3(__ldg(L.centre + f));   // n = 0 mod 3: the face centre ray
+        } else {
+            const float4 *W = L.layers + ((size_t)f * L.nl + g.a) * 3;
+            const float4 w0 = __ldg(W + g.e), w1 = __ldg(W + (g.e == 2 ? 0 : g.e + 1));
+            d = arc_point(f3(w0), f3(w1), w0.w, g.j, g.m);
+        }
+        out[q] = make_float4(d.x, d.y, d.z, __int_as_float(grid_ray(n, base, g)));
+    }
+}
+
+cudaError_t launch_raygen_schedule(const LatticeDev &lat, float4 *dirs, cudaStream_t s) {
+    const int edge_blocks = (12 + 30 * (lat.n - 1) + 255) / 256;
+    const int row_blocks = lat.n > 2 ? (lat.n - 2 + kTileRows - 1) / kTileRows : 0;
+    raygen_schedule_kernel<<<edge_blocks + 20 * row_blocks, 256, 0, s>>>(lat, dirs, edge_blocks, row_blocks);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_raygen(const LatticeDev &lat, float4 *dirs, int64_t N, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -76,7 +130,7 @@ cudaError_t launch_raygen(const LatticeDev &lat, float4 *dirs, int64_t N, cudaSt
 // interior rows before row i of a face: sum_{i'=1}^{i-1} (n - 1 - i')
 __device__ __forceinline__ long long row_prefix(int n, long long i) { return (i - 1) * (n - 1) - (i - 1) * i / 2; }
 
-__global__ void raygen_equidistant_kernel(PolyDev P, float4 *__restrict__ dirs, long long N) {
+__global__ void raygen_equidistant_kernel(PolyDev P, float4 *__restrict__ dirs, long long N, bool tagged) {
     const int n = P.n;
     const long long n_edge = (long long)P.ne * (n - 1);
     const long long per_face = (long long)(n - 1) * (n - 2) / 2;
@@ -109,18 +163,18 @@ __global__ void raygen_equidistant_kernel(PolyDev P, float4 *__restrict__ dirs, 
             p = A + (Bv - A) * ((float)i / (float)n) + (C - A) * ((float)j / (float)n);
         }
         float inv = 1.0f / sqrtf(dot(p, p));
-        dirs[id] = make_float4(p.x * inv, p.y * inv, p.z * inv, 0.0f);
+        dirs[id] = make_float4(p.x * inv, p.y * inv, p.z * inv, tagged ? __int_as_float((int)id) : 0.0f);
     }
 }
 
-cudaError_t launch_raygen_equidistant(const PolyDev &P, float4 *dirs, int64_t N, cudaStream_t s) {
+cudaError_t launch_raygen_equidistant(const PolyDev &P, float4 *dirs, int64_t N, bool tagged, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     long long want = (N + 255) / 256;
     int grid = (int)(want < (long long)sms * 16 ? want : (long long)sms * 16);
     if (grid < 1) grid = 1;
-    raygen_equidistant_kernel<<<grid, 256, 0, s>>>(P, dirs, (long long)N);
+    raygen_equidistant_kernel<<<grid, 256, 0, s>>>(P, dirs, (long long)N, tagged);
     return cudaGetLastError();
 }
 
@@ -300,7 +354,7 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
 
 // Persistent trace kernel.  Each warp keeps 32 rays in registers; after a segment, once at
 // least refill_min lanes hold a finished ray (miss or order cap), those lanes take fresh,
-// consecutive places of the schedule (tiled_ray, or lattice ids) from a global counter with
+// consecutive places of the schedule from a global counter with
 // one warp-aggregated atomic (ballot + popc).  Waiting for several idle lanes keeps a warp's
 // rays neighbours on the sphere (coherent traversal) while still keeping warps mostly full
 // until the pool drains.  After
@@ -320,7 +374,7 @@ __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
     pd.n = 0;
     const unsigned lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
-    const long long total = (long long)a.ntx * a.nrays_per_tx;
+    const long long total = (long long)a.ntx * a.count;
     unsigned seg = 0, nodes = 0, tris = 0, rxt = 0;
     bool alive = false, pool_empty = false;
     LaneRay st;
@@ -338,16 +392,22 @@ __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
             if (!alive) {
                 long long gid = (long long)base + __popc(need & lt_mask);
                 if (gid < total) {
-                    st.txi = (int)(gid / a.nrays_per_tx);
-                    const int local = (int)(gid - (long long)st.txi * a.nrays_per_tx);
-                    st.ray = a.tiled_n > 0 ? tiled_ray(local, a.tiled_n) : (int)a.ray_begin + local;
+                    // its transmitter, by a product instead of a 64-bit division, then fixed
+                    st.txi = a.ntx == 1 ? 0 : (int)((float)gid * a.inv_count);
+                    long long local = gid - (long long)st.txi * a.count;
+                    while (local < 0) local += a.count, --st.txi;
+                    while (local >= a.count) local -= a.count, ++st.txi;
+                    int place = (int)(a.first + local);
+                    if (a.id_order_n > 0) place = schedule_place(place, a.id_order_n);
+                    const float4 dd = __ldg(a.dirs + place);
                     st.o = f3(__ldg(a.tx + st.txi));
-                    st.d = f3(__ldg(a.dirs + st.ray));
+                    st.d = f3(dd);
+                    st.ray = __float_as_int(dd.w);
                     st.L = 0.0f;
                     st.k = 0;
                     st.prev = -1;
-                    alive = true;
-                    if (a.dump_stride > 0 && st.ray % a.dump_stride == 0) {
+                    alive = st.ray >= a.ray_begin && st.ray < a.ray_end;
+                    if (alive && a.dump_stride > 0 && st.ray % a.dump_stride == 0) {
                         int *df = a.dump_faces + ((size_t)st.txi * a.dump_per_tx + st.ray / a.dump_stride) *
                                                      (a.max_order + 1);
                         for (int j = 0; j <= a.max_order; ++j) df[j] = -2;
@@ -355,7 +415,10 @@ __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
                 }
             }
         }
-        if (__ballot_sync(0xffffffffu, alive) == 0) break;
+        if (__ballot_sync(0xffffffffu, alive) == 0) {
+            if (pool_empty) break;
+            continue;   // a range passed over every place taken
+        }
         if (alive) {
             RayPre r = make_ray(st.o, st.d);
             float th;

@@ -23,6 +23,7 @@
 #include <string>
 
 #include "dedup_keys.cuh"
+#include "lattice_order.cuh"
 
 namespace {
 
@@ -45,7 +46,8 @@ struct NaArgs {
     const sbr::RecDev *recs;         // input records
     const long long *rec_count;      // device: records emitted by the launch
     int64_t rec_cap;
-    const float4 *dirs;              // lattice directions of the launch
+    const float4 *dirs;              // directions of the launch
+    int sched_n;                     // as DedupArgs::sched_n
     sbr_path_record *out;            // output paths
     int64_t cap;
 };
@@ -120,7 +122,7 @@ __global__ void na_select(NaArgs a) {
         o.rough_dray = r.dray;
         o.iters = 0;
         o.valid = 0;
-        float4 d = a.dirs[r.ray];
+        float4 d = a.dirs[a.sched_n > 0 ? sbr::schedule_place(r.ray, a.sched_n) : r.ray];
         o.dir[0] = d.x;
         o.dir[1] = d.y;
         o.dir[2] = d.z;
@@ -217,6 +219,7 @@ extern "C" sbr_status sbr_dedup_noalloc(sbr_ctx *ctx, const sbr_paths *src, sbr_
     a.rec_count = src->counters + sbr::kRecords;
     a.rec_cap = src->record_cap;
     a.dirs = static_cast<const float4 *>(ctx->dirs);
+    a.sched_n = src->launcher == 0 ? src->n_div : 0;
     a.out = out;
     a.cap = cap;
     int grid = std::max(1, ctx->num_sms * 2);

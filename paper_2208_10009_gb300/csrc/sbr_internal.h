@@ -142,7 +142,9 @@ struct sbr_ctx {
     std::string last_error;
     int num_sms = 0;
     int max_threads_per_sm = 0;
-    // ray-generation workspace (directions for the last division level)
+    // ray-generation workspace (directions of the last division level: the equiangular
+    // lattice's at their places of the schedule, an equidistant launcher's at their ray ids;
+    // the ray id's bits in w)
     void *dirs = nullptr;
     size_t dirs_bytes = 0;
     int dirs_n = 0;
@@ -243,7 +245,10 @@ bool build_polyhedron(int poly, std::vector<float4> &v, std::vector<int2> &e, st
 
 // kernels (kernels_*.cu)
 cudaError_t launch_raygen(const LatticeDev &lat, float4 *dirs, int64_t N, cudaStream_t s);
-cudaError_t launch_raygen_equidistant(const PolyDev &p, float4 *dirs, int64_t N, cudaStream_t s);
+// the same directions in the schedule's order (lattice_order.cuh), each with its ray id's bits in w
+cudaError_t launch_raygen_schedule(const LatticeDev &lat, float4 *dirs, cudaStream_t s);
+// tagged: the ray id's bits in w
+cudaError_t launch_raygen_equidistant(const PolyDev &p, float4 *dirs, int64_t N, bool tagged, cudaStream_t s);
 
 struct TraceArgs {
     SceneDev scene;
@@ -251,8 +256,10 @@ struct TraceArgs {
     const float4 *dirs;
     const float4 *tx;
     int ntx;
-    int64_t nrays_per_tx;     // rays traced per transmitter: ids ray_begin .. ray_begin + nrays_per_tx
-    int64_t ray_begin;
+    int64_t first, count;     // places of dirs taken per transmitter: first .. first + count, of which
+    int ray_begin, ray_end;   // the ray ids in [ray_begin, ray_end) are traced
+    float inv_count;          // 1 / count (transmitter of a work index, then fixed)
+    int id_order_n;           // > 0: ray ids in turn (a place is an id) on the schedule of this n
     int max_order;
     float cone;               // reception cone half-angle (rad)
     float tan_cone;
@@ -265,8 +272,6 @@ struct TraceArgs {
     int *dump_faces;
     int64_t dump_per_tx;
     int refill_min;           // a warp takes new rays once at least this many lanes are idle
-    int tiled_n;              // > 0: the launch traces the whole equiangular lattice of this
-                              // division level, in the order of tiled_ray; 0: lattice id order
 };
 cudaError_t launch_trace(const TraceArgs &a, int grid, int block, cudaStream_t s);
 
@@ -276,15 +281,15 @@ struct DiffractArgs {
     const float4 *dirs;
     const float4 *tx;
     int ntx;
-    int64_t nrays_per_tx;     // rays searched per transmitter: ids ray_begin .. ray_begin + nrays_per_tx
-    int64_t ray_begin;
+    int64_t first, count;     // places and ray ids as in TraceArgs
+    int ray_begin, ray_end;
+    int id_order_n;
     float cone, tan_cone;
     RecDev *recs;
     int64_t rec_cap;
     long long *counters;
     float4 *cand;             // candidate (ray, wedge) list, 2 float4 each (scratch)
     int64_t cand_cap;
-    int tiled_n;              // as TraceArgs::tiled_n: the rays in the order of tiled_ray
 };
 cudaError_t launch_diffract(const DiffractArgs &a, int num_sms, cudaStream_t s);
 
@@ -295,7 +300,8 @@ struct DedupArgs {
     int64_t slots;            // power of two
     sbr_path_record *paths;
     int64_t path_cap;
-    const float4 *dirs;       // lattice directions (rough launch direction)
+    const float4 *dirs;       // launch directions (rough launch direction), at their places of
+    int sched_n;              // the schedule of this division level; 0: at their ray ids
     long long *counters;
     int nrx;                  // paths of pair (tx, rx) are emitted iff (tx * nrx + rx) % shard_world
     int shard_rank, shard_world;   // == shard_rank
