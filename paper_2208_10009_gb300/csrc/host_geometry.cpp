@@ -288,6 +288,21 @@ void put_child(float4 *n, int slot, const Box &b) {
 
 }  // namespace
 
+// the smallest FP16 value >= x (x >= 0; +inf beyond 65504)
+static unsigned short half_up(double x) {
+    if (x > 65504.0) return 0x7C00;
+    if (x < 6.103515625e-05) {                            // subnormal: units of 2^-24
+        const double q = x * 16777216.0;
+        const int i = (int)q;
+        return (unsigned short)(i + ((double)i < q));
+    }
+    float f = (float)x;
+    if ((double)f < x) f = std::nextafter(f, INFINITY);
+    unsigned u;
+    std::memcpy(&u, &f, sizeof(u));
+    return (unsigned short)(((u + 0x1FFF) >> 13) - (112u << 10));
+}
+
 bool build_bvh(const std::vector<float> &lo, const std::vector<float> &hi, int leaf_max, BvhOut &out,
                std::string &err) {
     size_t n = lo.size() / 3;
@@ -400,14 +415,18 @@ bool build_bvh(const std::vector<float> &lo, const std::vector<float> &hi, int l
             float *f = reinterpret_cast<float *>(nd);
             bool empty = !(bx.hi[0] >= bx.lo[0]);
             for (int a = 0; a < 3; ++a) {
-                f[(2 * a) * 4 + slot] = empty ? 1e30f : bx.lo[a];
-                f[(2 * a + 1) * 4 + slot] = empty ? 1e30f : bx.hi[a];
+                // centre and half extent, the latter rounded up so that the pair covers the box
+                // (FP16: at most 2^-10 of the half extent larger)
+                const float c = empty ? 1e30f : (float)(0.5 * ((double)bx.lo[a] + (double)bx.hi[a]));
+                const double need = empty ? 0.0 : std::max((double)bx.hi[a] - (double)c, (double)c - (double)bx.lo[a]);
+                f[4 * a + slot] = c;
+                reinterpret_cast<unsigned short *>(f + 12)[4 * a + slot] = half_up(need);
             }
         };
         if (order4.empty()) {
             Box empty;
             for (int i = 0; i < 4; ++i) put4(&out.nodes4[0], i, empty);
-            int *ref = reinterpret_cast<int *>(&out.nodes4[6]);
+            int *ref = reinterpret_cast<int *>(&out.nodes4[5]);
             for (int i = 0; i < 4; ++i) ref[i] = leaf_ref(0, 0);
         }
         // worst-case stack: along a root-to-leaf path every node pushes up to nkids - 1
@@ -426,7 +445,7 @@ bool build_bvh(const std::vector<float> &lo, const std::vector<float> &hi, int l
         }
         for (size_t w = 0; w < order4.size(); ++w) {
             float4 *nd = &out.nodes4[8 * w];
-            int *ref = reinterpret_cast<int *>(&nd[6]);
+            int *ref = reinterpret_cast<int *>(&nd[5]);
             Box empty;
             for (int i = 0; i < 4; ++i) {
                 int c = i < nkids[w] ? kids[w][i] : -1;

@@ -254,6 +254,15 @@ __device__ __forceinline__ void flush_records(const TraceArgs &a, const LaneRay 
     pd.n = 0;
 }
 
+// slab4 for boxes grown by the radius: cn and cf are o / d with the growth taken off and added
+__device__ __forceinline__ Slab4 slab4_grown(const NodeAxis &v, float inv, float cn, float cf, float ai) {
+    const float2 n01 = fma2(v.h01, -ai, fma2s(v.c01.x, v.c01.y, inv, -cn));
+    const float2 n23 = fma2(v.h23, -ai, fma2s(v.c23.x, v.c23.y, inv, -cn));
+    const float2 f01 = fma2(v.h01, ai, fma2s(v.c01.x, v.c01.y, inv, -cf));
+    const float2 f23 = fma2(v.h23, ai, fma2s(v.c23.x, v.c23.y, inv, -cf));
+    return {{n01.x, n01.y, n23.x, n23.y}, {f01.x, f01.y, f23.x, f23.y}};
+}
+
 // Reception judgment on segment o + s d, s in [0, tseg], of a ray that has travelled L
 // metres before it: every Rx whose foot lies on the segment and whose error angle
 // (Eq. 3) is within the cone emits a record.  Candidates come from the receivers' 4-wide
@@ -269,7 +278,8 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
     if (!(tcap >= 0.0f)) return;
     float rad = (st.L + tcap) * a.tan_cone * 1.001f + 1e-5f;
     const float oix = r.o.x * r.inv.x, oiy = r.o.y * r.inv.y, oiz = r.o.z * r.inv.z;
-    const float gx = rad * fabsf(r.inv.x), gy = rad * fabsf(r.inv.y), gz = rad * fabsf(r.inv.z);
+    const float aix = fabsf(r.inv.x), aiy = fabsf(r.inv.y), aiz = fabsf(r.inv.z);
+    const float gx = rad * aix, gy = rad * aiy, gz = rad * aiz;
     const float cnx = oix + gx, cny = oiy + gy, cnz = oiz + gz;
     const float cfx = oix - gx, cfy = oiy - gy, cfz = oiz - gz;
     const float tfar = tcap * 1.0000005f + 1e-6f;
@@ -277,9 +287,10 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
         // the receivers' bounding box, grown like the node boxes: one slab test before the
         // walk (most segments, e.g. those rising above every receiver, end here; 2-3 %
         // of the trace measured on the canyon and the large city)
-        const float nx = r.nx ? R.hi[0] : R.lo[0], fx = r.nx ? R.lo[0] : R.hi[0];
-        const float ny = r.ny ? R.hi[1] : R.lo[1], fy = r.ny ? R.lo[1] : R.hi[1];
-        const float nz = r.nz ? R.hi[2] : R.lo[2], fz = r.nz ? R.lo[2] : R.hi[2];
+        const bool bx = r.inv.x < 0.0f, by = r.inv.y < 0.0f, bz = r.inv.z < 0.0f;
+        const float nx = bx ? R.hi[0] : R.lo[0], fx = bx ? R.lo[0] : R.hi[0];
+        const float ny = by ? R.hi[1] : R.lo[1], fy = by ? R.lo[1] : R.hi[1];
+        const float nz = bz ? R.hi[2] : R.lo[2], fz = bz ? R.lo[2] : R.hi[2];
         const float tn = max3f(fmaf(nx, r.inv.x, -cnx), fmaf(ny, r.inv.y, -cny), fmaxf(fmaf(nz, r.inv.z, -cnz), 0.0f));
         const float tf = min3f(fmaf(fx, r.inv.x, -cfx), fmaf(fy, r.inv.y, -cfy), fminf(fmaf(fz, r.inv.z, -cfz), tfar));
         if (!(tn <= tf * 1.0000005f)) return;
@@ -290,19 +301,10 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
     for (;;) {
         if (!is_leaf(node)) {
             const float4 *nd = R.nodes4 + 8 * (size_t)node;
-            float4 nxv = __ldg(nd + r.nx), fxv = __ldg(nd + 1 - r.nx);
-            float4 nyv = __ldg(nd + 2 + r.ny), fyv = __ldg(nd + 3 - r.ny);
-            float4 nzv = __ldg(nd + 4 + r.nz), fzv = __ldg(nd + 5 - r.nz);
-            int4 refs = __ldg(reinterpret_cast<const int4 *>(nd + 6));
-            const float2 nx01 = fma2s(nxv.x, nxv.y, r.inv.x, -cnx), nx23 = fma2s(nxv.z, nxv.w, r.inv.x, -cnx);
-            const float2 fx01 = fma2s(fxv.x, fxv.y, r.inv.x, -cfx), fx23 = fma2s(fxv.z, fxv.w, r.inv.x, -cfx);
-            const float2 ny01 = fma2s(nyv.x, nyv.y, r.inv.y, -cny), ny23 = fma2s(nyv.z, nyv.w, r.inv.y, -cny);
-            const float2 fy01 = fma2s(fyv.x, fyv.y, r.inv.y, -cfy), fy23 = fma2s(fyv.z, fyv.w, r.inv.y, -cfy);
-            const float2 nz01 = fma2s(nzv.x, nzv.y, r.inv.z, -cnz), nz23 = fma2s(nzv.z, nzv.w, r.inv.z, -cnz);
-            const float2 fz01 = fma2s(fzv.x, fzv.y, r.inv.z, -cfz), fz23 = fma2s(fzv.z, fzv.w, r.inv.z, -cfz);
-            const float tnx[4] = {nx01.x, nx01.y, nx23.x, nx23.y}, tfx[4] = {fx01.x, fx01.y, fx23.x, fx23.y};
-            const float tny[4] = {ny01.x, ny01.y, ny23.x, ny23.y}, tfy[4] = {fy01.x, fy01.y, fy23.x, fy23.y};
-            const float tnz[4] = {nz01.x, nz01.y, nz23.x, nz23.y}, tfz[4] = {fz01.x, fz01.y, fz23.x, fz23.y};
+            const Node4 v4 = load_node4(nd);
+            const int4 refs = v4.refs;
+            const Slab4 sx = slab4_grown(v4.x, r.inv.x, cnx, cfx, aix), sy = slab4_grown(v4.y, r.inv.y, cny, cfy, aiy),
+                        sz = slab4_grown(v4.z, r.inv.z, cnz, cfz, aiz);
             const int rf[4] = {refs.x, refs.y, refs.z, refs.w};
             int next = 0x7fffffff;
             if (SBR_CHECKED_ON && sp + 3 > a.scene.stack_limit) {   // up to three pushes follow
@@ -311,8 +313,8 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                float tn = max3f(tnx[c], tny[c], fmaxf(tnz[c], 0.0f));
-                float tf = min3f(tfx[c], tfy[c], fminf(tfz[c], tfar)) * 1.0000005f;
+                float tn = max3f(sx.n[c], sy.n[c], fmaxf(sz.n[c], 0.0f));
+                float tf = min3f(sx.f[c], sy.f[c], fminf(sz.f[c], tfar)) * 1.0000005f;
                 if (tn <= tf) {
                     if (next == 0x7fffffff) next = rf[c];
                     else stack[sp++] = rf[c];

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <cuda_fp16.h>
 #include <math.h>
 
 #include "sbr_internal.h"
@@ -40,21 +41,22 @@ __device__ __forceinline__ double dnorm(dvec3 a) { return sqrt(ddot(a, a)); }
 struct RayPre {
     float3 o, d, inv;
     float3 mx, my, mz;
-    int nx, ny, nz;   // 1 where 1/d < 0: the near slab plane is the box's hi side
 };
+
+// 1 / x to one ulp, for the slab tests (their margins cover it); |x| < 1e-30 counts as 1e-30: the
+// tests stay correct for axis-parallel rays (huge but finite t), and box * inv - o * inv never
+// forms inf - inf.
+__device__ __forceinline__ float slab_rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fabsf(x) > 1e-30f ? x : copysignf(1e-30f, x)));
+    return r;
+}
 
 __device__ __forceinline__ RayPre make_ray(float3 o, float3 d) {
     RayPre r;
     r.o = o;
     r.d = d;
-    // A zero component is replaced by 1e-30 before inverting: the slab tests stay correct
-    // for axis-parallel rays (huge but finite t), and box * inv - o * inv never forms
-    // inf - inf.
-    r.inv = make_float3(1.0f / (d.x != 0.0f ? d.x : 1e-30f), 1.0f / (d.y != 0.0f ? d.y : 1e-30f),
-                        1.0f / (d.z != 0.0f ? d.z : 1e-30f));
-    r.nx = r.inv.x < 0.0f;
-    r.ny = r.inv.y < 0.0f;
-    r.nz = r.inv.z < 0.0f;
+    r.inv = make_float3(slab_rcp(d.x), slab_rcp(d.y), slab_rcp(d.z));
     float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
     int kz = (ax > ay) ? (ax > az ? 0 : 2) : (ay > az ? 1 : 2);
     int kx = kz == 2 ? 0 : kz + 1;
@@ -135,6 +137,73 @@ __device__ __forceinline__ float2 fma2s(float ax, float ay, float b, float c) {
     return r;
 }
 
+__device__ __forceinline__ float2 fma2(float2 a, float b, float2 c) {
+    float2 r;
+    asm("{\n\t.reg .b64 pa, pb, pc, pd;\n\t"
+        "mov.b64 pa, {%2, %3};\n\t"
+        "mov.b64 pb, {%4, %4};\n\t"
+        "mov.b64 pc, {%5, %6};\n\t"
+        "fma.rn.f32x2 pd, pa, pb, pc;\n\t"
+        "mov.b64 {%0, %1}, pd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b), "f"(c.x), "f"(c.y));
+    return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float b) {
+    float2 r;
+    asm("{\n\t.reg .b64 pa, pb, pd;\n\t"
+        "mov.b64 pa, {%2, %3};\n\t"
+        "mov.b64 pb, {%4, %4};\n\t"
+        "mul.rn.f32x2 pd, pa, pb;\n\t"
+        "mov.b64 {%0, %1}, pd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b));
+    return r;
+}
+
+// A 4-wide node (layout: sbr_internal.h).
+struct NodeAxis {
+    float2 c01, c23, h01, h23;
+};
+struct Node4 {
+    NodeAxis x, y, z;
+    int4 refs;
+};
+__device__ __forceinline__ float2 half_pair(unsigned v) { return __half22float2(*reinterpret_cast<__half2 *>(&v)); }
+__device__ __forceinline__ void set_axis(NodeAxis &v, float4 c, unsigned h01, unsigned h23) {
+    v.c01 = make_float2(c.x, c.y);
+    v.c23 = make_float2(c.z, c.w);
+    v.h01 = half_pair(h01);
+    v.h23 = half_pair(h23);
+}
+__device__ __forceinline__ Node4 load_node4(const float4 *nd) {
+    Node4 v;
+    const float4 cx = __ldg(nd), cy = __ldg(nd + 1), cz = __ldg(nd + 2);
+    const uint4 hxy = __ldg(reinterpret_cast<const uint4 *>(nd + 3));
+    const uint2 hz = __ldg(reinterpret_cast<const uint2 *>(nd + 4));
+    v.refs = __ldg(reinterpret_cast<const int4 *>(nd + 5));
+    set_axis(v.x, cx, hxy.x, hxy.y);
+    set_axis(v.y, cy, hxy.z, hxy.w);
+    set_axis(v.z, cz, hz.x, hz.y);
+    return v;
+}
+// Where a ray enters and leaves the children's slabs of one axis, t = (c / d - o / d) -+ h / |d|,
+// two children per packed FMA.  The walk keeps the SM's issue slots, its ALU pipe and its L1 data
+// pipe (a visit's rows come back at 128 bytes a cycle) busy together, so a visit pays for its
+// bytes as for its instructions.  Centres and half extents need no near / far row picked by the
+// ray's direction signs, so one address serves all rows where lo / hi planes took seven (a visit
+// 110 -> 95 instructions, L1 73 -> 81 % busy); FP16 half extents then cut a visit from 112 to 88
+// bytes for 12 conversions.  Large city trace 36.19 -> 34.45 ms, canyon 822 -> 802 us.
+struct Slab4 {
+    float n[4], f[4];
+};
+__device__ __forceinline__ Slab4 slab4(const NodeAxis &v, float inv, float oi, float ai) {
+    const float2 t01 = fma2s(v.c01.x, v.c01.y, inv, -oi), t23 = fma2s(v.c23.x, v.c23.y, inv, -oi);
+    const float2 n01 = fma2(v.h01, -ai, t01), n23 = fma2(v.h23, -ai, t23);
+    const float2 f01 = fma2(v.h01, ai, t01), f23 = fma2(v.h23, ai, t23);
+    return {{n01.x, n01.y, n23.x, n23.y}, {f01.x, f01.y, f23.x, f23.y}};
+}
+
 // Pop the next stack entry whose entry distance (sdist, beside the refs in stack) is within
 // tcull (the closest-hit range grown by the slab test's tolerance); false once the stack
 // holds none.
@@ -153,8 +222,8 @@ __device__ __forceinline__ bool pop_near(const int *stack, const float *sdist, i
 // tests a leaf once it reaches one ("while-while"): a warp then runs the leaf branch only
 // when its lanes stand at leaves, not on every step where one lane does.  Per node, slab
 // tests of the four child boxes as
-// t = plane * (1/d) - o * (1/d), the near / far planes picked by the ray's direction
-// signs (so no per-axis min/max), two children per packed FMA and three-input min/max;
+// t = (centre - o) / d -+ half extent / |d| (slab4: no per-axis min/max or sign), two children
+// per packed FMA and three-input min/max;
 // the nearest hit child is visited next and the others are pushed with their entry
 // distances; a popped entry whose entry distance already lies beyond the closest hit
 // found since its push is dropped unvisited (the box test it would face against the
@@ -173,35 +242,28 @@ __device__ __forceinline__ int closest_hit4(const SceneDev &S, const RayPre &r, 
     float tcull = tmax * 1.0000005f;   // entries entering beyond this are dropped at pop
     int best = -1, bface = 0x7fffffff;
     const float oix = r.o.x * r.inv.x, oiy = r.o.y * r.inv.y, oiz = r.o.z * r.inv.z;
+    const float aix = fabsf(r.inv.x), aiy = fabsf(r.inv.y), aiz = fabsf(r.inv.z);
     for (;;) {
         bool done = false;
         while (!is_leaf(node)) {
             ++nodes_visited;
             const float4 *nd = S.nodes4 + 8 * (size_t)node;
-            float4 nxv = __ldg(nd + r.nx), fxv = __ldg(nd + 1 - r.nx);
-            float4 nyv = __ldg(nd + 2 + r.ny), fyv = __ldg(nd + 3 - r.ny);
-            float4 nzv = __ldg(nd + 4 + r.nz), fzv = __ldg(nd + 5 - r.nz);
-            int4 refs = __ldg(reinterpret_cast<const int4 *>(nd + 6));
-            const float2 nx01 = fma2s(nxv.x, nxv.y, r.inv.x, -oix), nx23 = fma2s(nxv.z, nxv.w, r.inv.x, -oix);
-            const float2 fx01 = fma2s(fxv.x, fxv.y, r.inv.x, -oix), fx23 = fma2s(fxv.z, fxv.w, r.inv.x, -oix);
-            const float2 ny01 = fma2s(nyv.x, nyv.y, r.inv.y, -oiy), ny23 = fma2s(nyv.z, nyv.w, r.inv.y, -oiy);
-            const float2 fy01 = fma2s(fyv.x, fyv.y, r.inv.y, -oiy), fy23 = fma2s(fyv.z, fyv.w, r.inv.y, -oiy);
-            const float2 nz01 = fma2s(nzv.x, nzv.y, r.inv.z, -oiz), nz23 = fma2s(nzv.z, nzv.w, r.inv.z, -oiz);
-            const float2 fz01 = fma2s(fzv.x, fzv.y, r.inv.z, -oiz), fz23 = fma2s(fzv.z, fzv.w, r.inv.z, -oiz);
-            const float tnx[4] = {nx01.x, nx01.y, nx23.x, nx23.y}, tfx[4] = {fx01.x, fx01.y, fx23.x, fx23.y};
-            const float tny[4] = {ny01.x, ny01.y, ny23.x, ny23.y}, tfy[4] = {fy01.x, fy01.y, fy23.x, fy23.y};
-            const float tnz[4] = {nz01.x, nz01.y, nz23.x, nz23.y}, tfz[4] = {fz01.x, fz01.y, fz23.x, fz23.y};
-            float dist[4];
+            const Node4 v4 = load_node4(nd);
+            const int4 refs = v4.refs;
+            const Slab4 sx = slab4(v4.x, r.inv.x, oix, aix), sy = slab4(v4.y, r.inv.y, oiy, aiy),
+                        sz = slab4(v4.z, r.inv.z, oiz, aiz);
+            // hit iff tn <= tf (1 + 5e-7): tn, or +inf on a miss, as an FMA, a product with +inf
+            // (-inf or NaN on a hit) and a max, keeping the compare and select off the busier
+            // ALU pipe
+            float tn[4], tf[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                // hit iff tn <= tf (1 + 5e-7): tn, or +inf on a miss, as an FMA, a product
-                // with +inf (-inf or NaN on a hit) and a max, keeping the compare and select
-                // off the busier ALU pipe
-                float tn = max3f(tnx[c], tny[c], fmaxf(tnz[c], tmin));
-                float tf = min3f(tfx[c], tfy[c], fminf(tfz[c], tbest));
-                dist[c] = fmaxf(tn, fmaf(-tf, 1.0000005f, tn) * INFINITY);
+                tn[c] = max3f(sx.n[c], sy.n[c], fmaxf(sz.n[c], tmin));
+                tf[c] = min3f(sx.f[c], sy.f[c], fminf(sz.f[c], tbest));
             }
-            float d0 = dist[0], d1 = dist[1], d2 = dist[2], d3 = dist[3];
+            const float2 m01 = mul2(fma2(make_float2(tf[0], tf[1]), -1.0000005f, make_float2(tn[0], tn[1])), INFINITY);
+            const float2 m23 = mul2(fma2(make_float2(tf[2], tf[3]), -1.0000005f, make_float2(tn[2], tn[3])), INFINITY);
+            const float d0 = fmaxf(tn[0], m01.x), d1 = fmaxf(tn[1], m01.y), d2 = fmaxf(tn[2], m23.x), d3 = fmaxf(tn[3], m23.y);
             float dmin = fminf(min3f(d0, d1, d2), d3);
             if (dmin < INFINITY) {
                 if (SBR_CHECKED_ON && sp + 3 > S.stack_limit) {   // up to three pushes follow
@@ -256,23 +318,15 @@ __device__ __forceinline__ bool any_hit4(const SceneDev &S, const RayPre &r, flo
     int sp = 0;
     int node = 0;
     const float oix = r.o.x * r.inv.x, oiy = r.o.y * r.inv.y, oiz = r.o.z * r.inv.z;
+    const float aix = fabsf(r.inv.x), aiy = fabsf(r.inv.y), aiz = fabsf(r.inv.z);
     for (;;) {
         bool done = false;
         while (!is_leaf(node)) {
             const float4 *nd = S.nodes4 + 8 * (size_t)node;
-            float4 nxv = __ldg(nd + r.nx), fxv = __ldg(nd + 1 - r.nx);
-            float4 nyv = __ldg(nd + 2 + r.ny), fyv = __ldg(nd + 3 - r.ny);
-            float4 nzv = __ldg(nd + 4 + r.nz), fzv = __ldg(nd + 5 - r.nz);
-            int4 refs = __ldg(reinterpret_cast<const int4 *>(nd + 6));
-            const float2 nx01 = fma2s(nxv.x, nxv.y, r.inv.x, -oix), nx23 = fma2s(nxv.z, nxv.w, r.inv.x, -oix);
-            const float2 fx01 = fma2s(fxv.x, fxv.y, r.inv.x, -oix), fx23 = fma2s(fxv.z, fxv.w, r.inv.x, -oix);
-            const float2 ny01 = fma2s(nyv.x, nyv.y, r.inv.y, -oiy), ny23 = fma2s(nyv.z, nyv.w, r.inv.y, -oiy);
-            const float2 fy01 = fma2s(fyv.x, fyv.y, r.inv.y, -oiy), fy23 = fma2s(fyv.z, fyv.w, r.inv.y, -oiy);
-            const float2 nz01 = fma2s(nzv.x, nzv.y, r.inv.z, -oiz), nz23 = fma2s(nzv.z, nzv.w, r.inv.z, -oiz);
-            const float2 fz01 = fma2s(fzv.x, fzv.y, r.inv.z, -oiz), fz23 = fma2s(fzv.z, fzv.w, r.inv.z, -oiz);
-            const float tnx[4] = {nx01.x, nx01.y, nx23.x, nx23.y}, tfx[4] = {fx01.x, fx01.y, fx23.x, fx23.y};
-            const float tny[4] = {ny01.x, ny01.y, ny23.x, ny23.y}, tfy[4] = {fy01.x, fy01.y, fy23.x, fy23.y};
-            const float tnz[4] = {nz01.x, nz01.y, nz23.x, nz23.y}, tfz[4] = {fz01.x, fz01.y, fz23.x, fz23.y};
+            const Node4 v4 = load_node4(nd);
+            const int4 refs = v4.refs;
+            const Slab4 sx = slab4(v4.x, r.inv.x, oix, aix), sy = slab4(v4.y, r.inv.y, oiy, aiy),
+                        sz = slab4(v4.z, r.inv.z, oiz, aiz);
             const int rf[4] = {refs.x, refs.y, refs.z, refs.w};
             int next = 0x7fffffff;
             if (SBR_CHECKED_ON && sp + 3 > S.stack_limit) {   // up to three pushes follow
@@ -281,8 +335,8 @@ __device__ __forceinline__ bool any_hit4(const SceneDev &S, const RayPre &r, flo
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                float tn = max3f(tnx[c], tny[c], fmaxf(tnz[c], tmin));
-                float tf = min3f(tfx[c], tfy[c], fminf(tfz[c], tmax)) * 1.0000005f;
+                float tn = max3f(sx.n[c], sy.n[c], fmaxf(sz.n[c], tmin));
+                float tf = min3f(sx.f[c], sy.f[c], fminf(sz.f[c], tmax)) * 1.0000005f;
                 if (tn <= tf) {
                     if (next == 0x7fffffff) next = rf[c];
                     else stack[sp++] = rf[c];

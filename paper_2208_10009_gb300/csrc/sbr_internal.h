@@ -54,10 +54,11 @@ struct __align__(32) Plane64 {
     double x, y, z, w;
 };
 
-// BVH4 node (128 bytes = 8 x float4) used by the trace kernel: the four children's boxes
-// in structure-of-arrays form, f[0] = lo.x of children 0..3, f[1] = hi.x, f[2] = lo.y,
-// f[3] = hi.y, f[4] = lo.z, f[5] = hi.z; f[6] = the four child refs (same encoding as
-// BVH2; an empty slot is a leaf with 0 primitives and a far-away point box); f[7] unused.
+// BVH4 node (128 bytes = 8 x float4): the four children's boxes as centres (FP32) and half
+// extents (FP16, rounded up), structure of arrays: f[0], f[1], f[2] = centre x, y, z of children
+// 0..3; f[3] = half extents x then y, the first half of f[4] = half extents z, 4 x FP16 each;
+// f[5] = the four child refs (same encoding as BVH2; an empty slot is a leaf with 0 primitives
+// and a far-away point box); the rest unused.  A visit reads 88 bytes of it.
 
 struct SceneDev {
     const float4 *nodes4;     // 8 per BVH4 node
