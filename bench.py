@@ -678,7 +678,7 @@ def run_grad(args):
                       "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
                       "data": "synthetic", "config": {"workload": "1M fixed face-sequence paths of orders 1-6 from the "
                                                                   "urban canyon, Tx/Rx jittered +-1 m", "paths": P},
-                      "roofline": {"bound": "hbm", "kernel": "unfold_bwd_staged_kernel", "achieved": bwd_bytes / (bwd_ms / 1e3) / 1e9,
+                      "roofline": {"bound": "hbm", "kernel": "unfold_staged_kernel<true>", "achieved": bwd_bytes / (bwd_ms / 1e3) / 1e9,
                                    "peak": peaks.get("hbm_gbs"), "unit": "GB/s",
                                    "frac": bwd_bytes / (bwd_ms / 1e3) / 1e9 / peaks.get("hbm_gbs", 6800.0),
                                    "traffic": traffic,

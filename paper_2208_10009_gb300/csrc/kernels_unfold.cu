@@ -36,27 +36,30 @@ __device__ __forceinline__ void angles(float3 w, float &az, float &el) {
 // image txk = M_k(...M_1(Tx)).  With C_j = M_1 o ... o M_j and M_j(x) = H_j x + 2 h_j n_j:
 // C_j(x) = A_{j-1} H_j x + (a_{j-1} + 2 h_j A_{j-1} n_j), so each face costs one plane load
 // and A n once.  The loop runs the path's own order (a warp: its longest path), not the
-// maximum order.  face(j) gives face j's id; false if one lies outside [0, nf).
-template <class FaceAt>
-__device__ __forceinline__ bool unfold_pass(const SceneDev &S, int nf, int k, FaceAt face, float3 tx, float m[9],
+// maximum order; it is unrolled so that the 8 face ids stay in registers.  False if one of the
+// first k lies outside [0, nf).
+struct FaceIds {
+    int4 lo, hi;
+};
+__device__ __forceinline__ bool unfold_pass(const SceneDev &S, int nf, int k, const FaceIds &ids, float3 tx, float m[9],
                                             float3 &a0, float3 &txk) {
+    const int f[kMaxOrder] = {ids.lo.x, ids.lo.y, ids.lo.z, ids.lo.w, ids.hi.x, ids.hi.y, ids.hi.z, ids.hi.w};
     m[0] = 1.0f; m[1] = 0.0f; m[2] = 0.0f;
     m[3] = 0.0f; m[4] = 1.0f; m[5] = 0.0f;
     m[6] = 0.0f; m[7] = 0.0f; m[8] = 1.0f;
     float o[3] = {0.0f, 0.0f, 0.0f};
     float3 x = tx;
-    // the ids first (independent loads), so that the walk below can load each next plane
-    // under the current face's arithmetic
+    unsigned top = 0;
+#pragma unroll
+    for (int j = 0; j < kMaxOrder; ++j) top = max(top, j < k ? (unsigned)f[j] : 0u);
+    if (k > 0 && top >= (unsigned)nf) return false;
+    // each next plane is loaded under the current face's arithmetic
+    float4 pl = k > 0 ? __ldg(S.planes + f[0]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
     for (int j = 0; j < kMaxOrder; ++j) {
         if (j >= k) break;
-        const int f = face(j);
-        if (f < 0 || f >= nf) return false;
-    }
-    float4 pl = k > 0 ? __ldg(S.planes + face(0)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll 1
-    for (int j = 0; j < k; ++j) {
-        const float4 pn = __ldg(S.planes + face(j + 1 < k ? j + 1 : j));
+        float4 pn = pl;
+        if (j + 1 < kMaxOrder && j + 1 < k) pn = __ldg(S.planes + f[j + 1 < kMaxOrder ? j + 1 : j]);
         const float3 n = f3(pl);
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
@@ -85,24 +88,18 @@ __device__ __forceinline__ void angles_grad_fast(float3 w, float3 &gaz, float3 &
     gel = make_float3(-w.x * w.z * c, -w.y * w.z * c, rho2 * c);
 }
 
-__global__ void unfold_fwd_kernel(UnfoldArgs a) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.n; i += (long long)gridDim.x * blockDim.x) {
-        const float3 tx = make_float3(a.tx[3 * i], a.tx[3 * i + 1], a.tx[3 * i + 2]);
-        const float3 rx = make_float3(a.rx[3 * i], a.rx[3 * i + 1], a.rx[3 * i + 2]);
-        const int ord = a.order[i];
-        const int k = ord < 0 ? 0 : (ord > kMaxOrder ? kMaxOrder : ord);
-        const int *fp = a.faces + 8 * i;
-        float m[9];
-        float3 a0, txk;
-        float *o = a.out + 8 * i;
-        if (!unfold_pass(a.scene, a.nf, k, [&](int j) { return __ldg(fp + j); }, tx, m, a0, txk)) {
-            for (int j = 0; j < 8; ++j) o[j] = __int_as_float(0x7fc00000);
-            continue;
-        }
+// The forward map of one path from its loaded inputs.  A path with an id outside [0, nf) gets NaN
+// outputs.
+__device__ __forceinline__ void fwd_path(const UnfoldArgs &a, float3 tx, float3 rx, float az, float el, int k,
+                                         const FaceIds &face, long long i) {
+    float m[9];
+    float3 a0, txk;
+    float o[8];
+    if (unfold_pass(a.scene, a.nf, k, face, tx, m, a0, txk)) {
         const float3 w = mul_A(m, rx) + a0 - tx;
         float se, ce, sa, ca;
-        sincosf(a.az_el[2 * i + 1], &se, &ce);
-        sincosf(a.az_el[2 * i], &sa, &ca);
+        sincosf(el, &se, &ce);
+        sincosf(az, &sa, &ca);
         const float3 d = make_float3(ce * ca, ce * sa, se);
         const float3 miss = mul_AT(m, w - d * dot(w, d));
         const float3 v = txk - rx;
@@ -112,7 +109,37 @@ __global__ void unfold_fwd_kernel(UnfoldArgs a) {
         o[3] = sqrtf(dot(w, w)) * (float)(1.0 / kC0);
         angles(w, o[4], o[5]);
         angles(v, o[6], o[7]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) o[j] = __int_as_float(0x7fc00000);
     }
+    if ((reinterpret_cast<uintptr_t>(a.out) & 15) == 0) {   // every row then is 16-byte aligned
+        float4 *dst = reinterpret_cast<float4 *>(a.out) + 2 * i;
+        dst[0] = make_float4(o[0], o[1], o[2], o[3]);
+        dst[1] = make_float4(o[4], o[5], o[6], o[7]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a.out[8 * i + j] = o[j];
+    }
+}
+
+// the 8 ids of a path in global memory (the array is 16-byte aligned, so every row is)
+__device__ __forceinline__ FaceIds load_faces(const int32_t *p) {
+    return {__ldg(reinterpret_cast<const int4 *>(p)), __ldg(reinterpret_cast<const int4 *>(p) + 1)};
+}
+
+// The inputs of path i straight from global memory.
+__device__ __forceinline__ void fwd_direct_path(const UnfoldArgs &a, long long i) {
+    const float3 tx = make_float3(a.tx[3 * i], a.tx[3 * i + 1], a.tx[3 * i + 2]);
+    const float3 rx = make_float3(a.rx[3 * i], a.rx[3 * i + 1], a.rx[3 * i + 2]);
+    const int ord = a.order[i];
+    const int k = ord < 0 ? 0 : (ord > kMaxOrder ? kMaxOrder : ord);
+    fwd_path(a, tx, rx, a.az_el[2 * i], a.az_el[2 * i + 1], k, load_faces(a.faces + 8 * i), i);
+}
+
+__global__ void __launch_bounds__(256) unfold_fwd_kernel(UnfoldArgs a) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.n; i += (long long)gridDim.x * blockDim.x)
+        fwd_direct_path(a, i);
 }
 
 __device__ __forceinline__ void load_grad_row(const UnfoldArgs &a, long long i, float g[8]) {
@@ -129,11 +156,10 @@ __device__ __forceinline__ void load_grad_row(const UnfoldArgs &a, long long i, 
     }
 }
 
-// The adjoint of one path from its loaded inputs (g: the row of 8 output gradients);
-// face(j) gives its face ids.  A path with an id outside [0, nf) gets NaN gradients.
-template <class FaceAt>
+// The adjoint of one path from its loaded inputs (g: the row of 8 output gradients).  A path with
+// an id outside [0, nf) gets NaN gradients.
 __device__ __forceinline__ void bwd_path(const UnfoldArgs &a, float3 tx, float3 rx, float az, float el, int k,
-                                         FaceAt face, const float g[8], long long i) {
+                                         const FaceIds &face, const float g[8], long long i) {
     float m[9];
     float3 a0, txk;
     if (!unfold_pass(a.scene, a.nf, k, face, tx, m, a0, txk)) {
@@ -185,8 +211,7 @@ __device__ __forceinline__ void bwd_direct_path(const UnfoldArgs &a, long long i
     const int k = ord < 0 ? 0 : (ord > kMaxOrder ? kMaxOrder : ord);
     float g[8];
     load_grad_row(a, i, g);
-    const int *fp = a.faces + 8 * i;
-    bwd_path(a, tx, rx, a.az_el[2 * i], a.az_el[2 * i + 1], k, [&](int j) { return __ldg(fp + j); }, g, i);
+    bwd_path(a, tx, rx, a.az_el[2 * i], a.az_el[2 * i + 1], k, load_faces(a.faces + 8 * i), g, i);
 }
 
 
@@ -198,28 +223,31 @@ __global__ void __launch_bounds__(256, 4) unfold_bwd_kernel(UnfoldArgs a) {
         bwd_direct_path(a, i);
 }
 
-// ---------------------------------------------------------------- staged adjoint
-// The adjoint reads 100 bytes per path (Tx, Rx, az/el, order, 8 face ids, 8 output
-// gradients) and writes 32; per path it then walks the order's face planes (an L1-resident
-// table) once.  Loading a path's inputs in the thread that computes it leaves the thread
-// idle for a DRAM round trip per path.  Here each warp owns whole 32-path chunks
-// (persistent, chunk += all warps): one lane issues six bulk copies (cp.async.bulk, one per
-// input array: a chunk's part of every array is one contiguous, 16-byte aligned range) into
-// the warp's shared-memory buffer, completing on that buffer's mbarrier, and the next
-// chunk's copies are issued before the current chunk is computed (two buffers a warp), so
-// the copies run under the arithmetic.  Warps never wait for one another.  The ragged last
-// chunk is read from global memory.
+// ---------------------------------------------------------------- staged forms
+// The forward map reads 68 bytes a path (Tx, Rx, az/el, order, 8 face ids) and writes 32; the
+// adjoint reads 100 (+ 8 output gradients) and writes 32; per path both then walk the order's
+// face planes (an L1-resident table) once.  Loading a path's inputs in the thread that computes
+// it leaves the thread idle for a DRAM round trip per path.  Here each warp owns whole 32-path
+// chunks (persistent, chunk += all warps): one lane issues a bulk copy (cp.async.bulk) per input
+// array (a chunk's part of every array is one contiguous, 16-byte aligned range) into the
+// warp's shared-memory buffer, completing on that buffer's mbarrier, and the next chunk's copies
+// are issued before the current chunk is computed (two buffers a warp), so the copies run under
+// the arithmetic.  Warps never wait for one another.  The ragged last chunk is read from global
+// memory.  At 3.73M paths of orders 1-6: forward 134 us (direct loads) -> 107
+// us, adjoint 105 -> 98 us with the ids in registers (from shared memory every id cost an 8-way
+// bank conflict); now bound by issue (75 / 70 %), 22-24 of 32 lanes for the paths' unlike orders.
 constexpr int kChunk = 32;
 constexpr int kStageWarps = 8;   // warps a block
 constexpr unsigned kCTx = 12 * kChunk, kCAzEl = 8 * kChunk, kCOrder = 4 * kChunk, kCFaces = 32 * kChunk,
                    kCGrad = 32 * kChunk;
 constexpr unsigned kOffTx = 0, kOffRx = kOffTx + kCTx, kOffAzEl = kOffRx + kCTx, kOffOrder = kOffAzEl + kCAzEl,
-                   kOffFaces = kOffOrder + kCOrder, kOffGrad = kOffFaces + kCFaces,
-                   kChunkBytes = kOffGrad + kCGrad;   // 3,200 bytes a chunk
-constexpr unsigned kBarOff = kStageWarps * 2 * kChunkBytes;
-constexpr unsigned kBwdSmem = kBarOff + kStageWarps * 16;   // two buffers + two mbarriers a warp
+                   kOffFaces = kOffOrder + kCOrder, kOffGrad = kOffFaces + kCFaces;
+// bytes of a chunk: 2,176 forward, 3,200 adjoint
+__host__ __device__ constexpr unsigned chunk_bytes(bool bwd) { return kOffGrad + (bwd ? kCGrad : 0); }
+// two buffers + two mbarriers a warp
+__host__ __device__ constexpr unsigned stage_smem(bool bwd) { return kStageWarps * (2 * chunk_bytes(bwd) + 16); }
 static_assert(kOffRx % 16 == 0 && kOffAzEl % 16 == 0 && kOffOrder % 16 == 0 && kOffFaces % 16 == 0 &&
-              kOffGrad % 16 == 0 && kChunkBytes % 16 == 0, "bulk-copy alignment");
+              kOffGrad % 16 == 0 && chunk_bytes(true) % 16 == 0, "bulk-copy alignment");
 // an mbarrier wait that has not completed after this long gives up (nanoseconds)
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;
 
@@ -238,21 +266,22 @@ __device__ __forceinline__ void bulk_g2s(unsigned dst, const void *src, unsigned
                  :: "r"(dst), "l"(src), "r"(bytes), "r"(mbar) : "memory");
 }
 
-// Issue the six copies of chunk c into the buffer at buf (one lane).
+// Issue the copies of chunk c into the buffer at buf (one lane).
+template <bool kBwd>
 __device__ __forceinline__ void issue_chunk(const UnfoldArgs &a, long long c, unsigned buf, unsigned mbar) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mbar), "r"(kChunkBytes) : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mbar), "r"(chunk_bytes(kBwd)) : "memory");
     const long long p = c * kChunk;
     bulk_g2s(buf + kOffTx, a.tx + 3 * p, kCTx, mbar);
     bulk_g2s(buf + kOffRx, a.rx + 3 * p, kCTx, mbar);
     bulk_g2s(buf + kOffAzEl, a.az_el + 2 * p, kCAzEl, mbar);
     bulk_g2s(buf + kOffOrder, a.order + p, kCOrder, mbar);
     bulk_g2s(buf + kOffFaces, a.faces + 8 * p, kCFaces, mbar);
-    bulk_g2s(buf + kOffGrad, a.grad_out + 8 * p, kCGrad, mbar);
+    if (kBwd) bulk_g2s(buf + kOffGrad, a.grad_out + 8 * p, kCGrad, mbar);
 }
 
 // Wait for phase `parity` of the mbarrier, at most kWaitLimitNs; false on giving up.
 __device__ __forceinline__ bool wait_parity(unsigned mbar, unsigned parity) {
-    const unsigned long long t0 = global_ns();
+    unsigned long long t0 = 0;   // read once the first try has failed
     for (;;) {
         unsigned done;
         asm volatile("{\n\t.reg .pred p;\n\t"
@@ -260,22 +289,26 @@ __device__ __forceinline__ bool wait_parity(unsigned mbar, unsigned parity) {
                      "selp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
         if (done) return true;
-        if (global_ns() - t0 > kWaitLimitNs) return false;
+        const unsigned long long t = global_ns();
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > kWaitLimitNs) return false;
     }
 }
 
-#ifndef SBR_STAGE_BLOCKS
-#define SBR_STAGE_BLOCKS 3
-#endif
-__global__ void __launch_bounds__(kStageWarps * 32, SBR_STAGE_BLOCKS) unfold_bwd_staged_kernel(UnfoldArgs a) {
+// Resident blocks of 256 threads per SM (registers: 64 forward, 80 adjoint; forward with 3 / 4 / 5
+// blocks 107 / 108 / 119 us, adjoint with 2 / 3 / 4 102 / 99 / 130 us at 3.7M paths).
+constexpr int kFwdBlocks = 4, kBwdBlocks = 3;
+template <bool kBwd>
+__global__ void __launch_bounds__(kStageWarps * 32, kBwd ? kBwdBlocks : kFwdBlocks) unfold_staged_kernel(UnfoldArgs a) {
+    constexpr unsigned kBytes = chunk_bytes(kBwd);
     extern __shared__ __align__(16) unsigned char smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long full = a.n / kChunk;   // chunks read by bulk copies
     const long long chunks = (a.n + kChunk - 1) / kChunk;
     const long long nwarps = (long long)gridDim.x * kStageWarps;
-    unsigned char *wbuf = smem + w * 2 * kChunkBytes;
+    unsigned char *wbuf = smem + w * 2 * kBytes;
     const unsigned base = smem_addr(wbuf);
-    const unsigned mb0 = smem_addr(smem + kBarOff) + 16 * w, mb1 = mb0 + 8;
+    const unsigned mb0 = smem_addr(smem + kStageWarps * 2 * kBytes) + 16 * w, mb1 = mb0 + 8;
     if (lane == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mb0) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mb1) : "memory");
@@ -283,28 +316,32 @@ __global__ void __launch_bounds__(kStageWarps * 32, SBR_STAGE_BLOCKS) unfold_bwd
     }
     __syncwarp();
     long long c = (long long)blockIdx.x * kStageWarps + w;
-    if (lane == 0 && c < full) issue_chunk(a, c, base, mb0);
+    if (lane == 0 && c < full) issue_chunk<kBwd>(a, c, base, mb0);
     for (unsigned it = 0; c < chunks; ++it, c += nwarps) {
         if (c >= full) {   // the ragged last chunk
             const long long i = c * kChunk + lane;
-            if (i < a.n) bwd_direct_path(a, i);
+            if (i < a.n) kBwd ? bwd_direct_path(a, i) : fwd_direct_path(a, i);
             continue;
         }
         const unsigned cur = it & 1, mbar = cur ? mb1 : mb0;
         const long long nxt = c + nwarps;
         // the other buffer was last read in the previous iteration, which ended with a
         // warp barrier: refill it with the next chunk before computing this one
-        if (lane == 0 && nxt < full) issue_chunk(a, nxt, base + (cur ^ 1) * kChunkBytes, cur ? mb0 : mb1);
+        if (lane == 0 && nxt < full) issue_chunk<kBwd>(a, nxt, base + (cur ^ 1) * kBytes, cur ? mb0 : mb1);
         const bool ok = wait_parity(mbar, (it >> 1) & 1);
         if (__any_sync(0xffffffffu, !ok)) {
-            // the copies did not arrive in time: NaN gradients for this warp's remaining
+            // the copies did not arrive in time: NaN results for this warp's remaining
             // paths, then wait (bounded) for the copies still in flight before leaving
             const float nan = __int_as_float(0x7fc00000);
             for (long long r = c; r < chunks; r += nwarps) {
                 const long long i = r * kChunk + lane;
                 if (i >= a.n) continue;
-                for (int j = 0; j < 3; ++j) a.grad_tx[3 * i + j] = a.grad_rx[3 * i + j] = nan;
-                a.grad_az_el[2 * i] = a.grad_az_el[2 * i + 1] = nan;
+                if (kBwd) {
+                    for (int j = 0; j < 3; ++j) a.grad_tx[3 * i + j] = a.grad_rx[3 * i + j] = nan;
+                    a.grad_az_el[2 * i] = a.grad_az_el[2 * i + 1] = nan;
+                } else {
+                    for (int j = 0; j < 8; ++j) a.out[8 * i + j] = nan;
+                }
             }
             if (lane == 0) {
                 wait_parity(mbar, (it >> 1) & 1);
@@ -312,18 +349,23 @@ __global__ void __launch_bounds__(kStageWarps * 32, SBR_STAGE_BLOCKS) unfold_bwd
             }
             return;
         }
-        const unsigned char *sb = wbuf + cur * kChunkBytes;
+        const unsigned char *sb = wbuf + cur * kBytes;
         const float *stx = reinterpret_cast<const float *>(sb + kOffTx) + 3 * lane;
         const float *srx = reinterpret_cast<const float *>(sb + kOffRx) + 3 * lane;
         const float2 ae = reinterpret_cast<const float2 *>(sb + kOffAzEl)[lane];
-        const int *sf = reinterpret_cast<const int *>(sb + kOffFaces) + 8 * lane;
-        const float4 *sg = reinterpret_cast<const float4 *>(sb + kOffGrad) + 2 * lane;
+        const int4 *sf = reinterpret_cast<const int4 *>(sb + kOffFaces) + 2 * lane;
         const int ord = reinterpret_cast<const int *>(sb + kOffOrder)[lane];
         const int k = ord < 0 ? 0 : (ord > kMaxOrder ? kMaxOrder : ord);
-        const float4 g0 = sg[0], g1 = sg[1];
-        const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-        bwd_path(a, make_float3(stx[0], stx[1], stx[2]), make_float3(srx[0], srx[1], srx[2]), ae.x, ae.y, k,
-                 [&](int j) { return sf[j]; }, g, c * kChunk + lane);
+        const float3 tx = make_float3(stx[0], stx[1], stx[2]), rx = make_float3(srx[0], srx[1], srx[2]);
+        const FaceIds face = {sf[0], sf[1]};
+        if (kBwd) {
+            const float4 *sg = reinterpret_cast<const float4 *>(sb + kOffGrad) + 2 * lane;
+            const float4 g0 = sg[0], g1 = sg[1];
+            const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+            bwd_path(a, tx, rx, ae.x, ae.y, k, face, g, c * kChunk + lane);
+        } else {
+            fwd_path(a, tx, rx, ae.x, ae.y, k, face, c * kChunk + lane);
+        }
         __syncwarp();   // this buffer is refilled in the next iteration
     }
 }
@@ -337,34 +379,36 @@ static int unfold_grid(long long n) {
     return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
-cudaError_t launch_unfold_fwd(const UnfoldArgs &a, cudaStream_t s) {
-    unfold_fwd_kernel<<<unfold_grid(a.n), 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
 // The staged form needs every input array 16-byte aligned (each chunk's range then is) and
-// pays off once there are a few chunks per warp; it runs persistent, four blocks per SM.
-cudaError_t launch_unfold_bwd(const UnfoldArgs &a, cudaStream_t s) {
+// pays off once there are a few chunks per warp; it runs persistent.
+template <bool kBwd>
+static cudaError_t launch_unfold(const UnfoldArgs &a, cudaStream_t s) {
     auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long chunks = (a.n + kChunk - 1) / kChunk;
     const bool staged = al16(a.tx) && al16(a.rx) && al16(a.az_el) && al16(a.order) && al16(a.faces) &&
-                        al16(a.grad_out) && chunks >= 16LL * sms;
+                        (!kBwd || al16(a.grad_out)) && chunks >= 16LL * sms;
     if (!staged) {
-        unfold_bwd_kernel<<<unfold_grid(a.n), 256, 0, s>>>(a);
+        if (kBwd) unfold_bwd_kernel<<<unfold_grid(a.n), 256, 0, s>>>(a);
+        else unfold_fwd_kernel<<<unfold_grid(a.n), 256, 0, s>>>(a);
         return cudaGetLastError();
     }
     static bool attr_set[64] = {};
     if (dev < 64 && !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(unfold_bwd_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmem);
+        cudaError_t e = cudaFuncSetAttribute(unfold_staged_kernel<kBwd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             stage_smem(kBwd));
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    const long long grid = std::min<long long>((chunks + kStageWarps - 1) / kStageWarps, (long long)SBR_STAGE_BLOCKS * sms);
-    unfold_bwd_staged_kernel<<<(int)grid, kStageWarps * 32, kBwdSmem, s>>>(a);
+    const long long grid = std::min<long long>((chunks + kStageWarps - 1) / kStageWarps,
+                                               (long long)(kBwd ? kBwdBlocks : kFwdBlocks) * sms);
+    unfold_staged_kernel<kBwd><<<(int)grid, kStageWarps * 32, stage_smem(kBwd), s>>>(a);
     return cudaGetLastError();
 }
+
+cudaError_t launch_unfold_fwd(const UnfoldArgs &a, cudaStream_t s) { return launch_unfold<false>(a, s); }
+cudaError_t launch_unfold_bwd(const UnfoldArgs &a, cudaStream_t s) { return launch_unfold<true>(a, s); }
 
 }  // namespace sbr
