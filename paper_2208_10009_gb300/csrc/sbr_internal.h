@@ -32,7 +32,9 @@ enum Counter {
     kRayHead, kBatchHead, kBatchDone, kErrorFlags, kWedgeTests, kDiffRecords, kDiffCand, kNonFinite,
     kDiffPending,   // diffraction receptions parked at the top of the record array for diffract_occlusion
     kDiffBase,      // the record count before them (the trace's records)
-    kNumCounters = 18
+    kDiffHead,      // groups of places the diffraction search has taken
+    kDiffPairs,     // (wedge, 32 places) pairs its beams left for the exact test
+    kNumCounters = 20
 };
 
 // BVH node: both children's boxes in one 64-byte node (4 x float4).
