@@ -1080,7 +1080,9 @@ sbr_status sbr_refine_pair(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *path
     A.index = paths->pair_off + npairs + 1;
     {
         Range r("sbr_refine_pair: iterations + validity + outputs");
-        SBR_CUDA(launch_refine(A, (count + 127) / 128, 128, ctx->stream));
+        // a warp a path up to twelve paths an SM, then a thread a path
+        const int per_block = count <= 12 * ctx->num_sms ? 4 : 128;
+        SBR_CUDA(launch_refine(A, (count + per_block - 1) / per_block, 128, ctx->stream));
     }
     return SBR_OK;
 }

@@ -234,15 +234,6 @@ __device__ __noinline__ float4 unfold_rx32(const SceneDev &S, const PathGeo &g) 
                        df_round(df_sub(x.z, df_of(g.tx.z))), 0.0f);
 }
 
-__device__ __forceinline__ void build_unf(const SceneDev &S, const PathGeo &g, UnfD &ud, UnfF &uf) {
-    for (int j = 0; j < g.k; ++j) {
-        ud.p[j] = unfold_plane(S, g, j);
-        uf.p[j] = unfold_plane32(S, g, j);
-    }
-    ud.w = unfold_rx(S, g);
-    uf.w = unfold_rx32(S, g);
-}
-
 // |d x W|^2 of sub-ray d (+inf if invalid); dw = d . W
 __device__ __forceinline__ float key32(const UnfF &u, int k, float3 d, float &dw) {
     float pn = 0.0f, pd = 1.0f;   // T_{j-1} = pn / pd, T_0 = 0
@@ -889,131 +880,6 @@ __device__ __forceinline__ long long path_count(const RefineArgs &A) {
     return n < A.path_cap ? n : A.path_cap;
 }
 
-// a6-a8, one thread per path (static grid-stride schedule).
-__global__ void __launch_bounds__(256) refine_kernel(RefineArgs A) {
-    const long long total = A.range ? (long long)(A.range[1] - A.range[0]) : path_count(A);
-    const int off = c_sub.off[A.K];
-    const double shrink = c_sub.shrink[A.K];
-    const float shrinkf = c_sub.shrink_f[A.K];
-    const double stall = 1.0 / (1.0 - shrink) + 2.0 * shrink;
-    const float stallf = (float)stall;
-    __shared__ SubTab64 tab;
-    load_sub64(tab);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        long long pi = A.range ? (long long)A.index[A.range[0] + i] : i;
-        sbr_path_record p = A.paths[pi];
-        if (!path_ids_ok(A, p)) {
-            A.paths[pi].valid = 0;
-            A.paths[pi].flags = SBR_PATH_TRACE_FAIL;
-            continue;
-        }
-        PathGeo g;
-        load_path(A, p, g);
-        UnfD ud;
-        UnfF uf;
-        build_unf(A.scene, g, ud, uf);
-        // FP32 phase while the cone radius is >= fp64_below (the radius R0 = max(theta_launch,
-        // rough error) is a float, so the first test is exact)
-        float Rf = fmaxf(A.theta_launch, p.rough_err);
-        bool fp64 = Rf < A.fp64_below_f, fail = false;
-        float3 cf = make_float3((float)p.dir[0], (float)p.dir[1], (float)p.dir[2]);
-        float keyf = INFINITY, dwf = 0.0f;
-        int it = 0, flags = 0, stop = kStopNone;
-        if (!fp64) {
-            keyf = key32(uf, g.k, cf, dwf);
-            while (it < A.max_iters) {
-                if (reached32(A, g, uf, cf, keyf, dwf)) {
-                    stop = kStopReached;
-                    break;
-                }
-                if (stalled32(keyf, dwf, Rf, stallf)) {
-                    stop = kStopStalled;
-                    break;
-                }
-                if (Rf < A.fp64_below_f) break;   // on to the FP64 iterations
-                const int ax = A.choice_log ? frame_axis32(cf) : 0;
-                const int bk = iterate32(uf, g.k, A.K, off, Rf, cf, keyf, dwf);
-                if (bk < 0) {
-                    fail = true;
-                    break;
-                }
-                if (A.choice_log) A.choice_log[pi * A.max_iters + it] = choice_entry(bk, ax);
-                Rf *= shrinkf;
-                ++it;
-            }
-        }
-        dvec3 c = dv(cf.x, cf.y, cf.z);
-        double key = INFINITY, dw = 0.0;
-        if (!fail && Rf < A.fp64_below_f) {
-            double R = cone_radius64(A, p.rough_err, it, shrink);
-            if (fp64) {
-                c = dv(p.dir[0], p.dir[1], p.dir[2]);
-                key = key64(ud, g.k, c, dw);
-            } else {
-                key = keyf;
-                dw = dwf;
-            }
-            stop = kStopNone;   // the FP64 phase judges the state again
-            while (it < A.max_iters) {
-                if (reached(A, g, ud, c, key, dw)) {
-                    stop = kStopReached;
-                    break;
-                }
-                if (stalled(key, dw, R, stall)) {
-                    stop = kStopStalled;
-                    break;
-                }
-                const int ax = A.choice_log ? frame_axis64(c) : 0;
-                const int bk = iterate64(ud, g.k, A.K, off, tab, R, c, key, dw);
-                if (bk < 0) {
-                    fail = true;
-                    break;
-                }
-                flags |= SBR_PATH_FP64;
-                fp64 = true;
-                if (A.choice_log) A.choice_log[pi * A.max_iters + it] = choice_entry(bk, ax);
-                R *= shrink;
-                ++it;
-            }
-        }
-        if (fail) flags |= SBR_PATH_TRACE_FAIL;
-        else if (stop == kStopStalled) flags |= SBR_PATH_STALLED;
-        p.iters = it;
-        p.flags = flags | (it > 0 ? SBR_PATH_REFINED : 0);
-        p.dir[0] = c.x;
-        p.dir[1] = c.y;
-        p.dir[2] = c.z;
-        p.err = error_angle(key, dw, keyf, dwf, fp64);
-        finalize_path(A, g, c, p, converged_bound(it, cone_radius64(A, p.rough_err, it, shrink)));
-        store_result(A.paths + pi, p);
-    }
-}
-
-// Lists path pi in its order group for batch_finalize_kernel (group offsets from
-// batch_unfold_kernel's counts), so that a warp there holds paths of one order.  Inside the
-// group, paths whose error meets the convergence bound 2 R + 1e-7 (the validity test's
-// condition; R is the cone radius after the iterations, here only an ordering hint) fill it
-// from the front and the others, which the validity test rejects at once, from the back:
-// a warp's lanes then run their BVH queries, or skip them, together.
-__device__ __forceinline__ void list_for_finalize(const RefineArgs &A, const PathGeo &g, long long pi, double err,
-                                                  double R) {
-    const int grp = order_group(g);
-    unsigned long long at = 0;
-    for (int b = 0; b < grp; ++b) at += A.order_cnt[b];
-    if (err <= 2.0 * R + 1e-7) at += atomicAdd(A.order_cnt + 16 + grp, 1ULL);
-    else at += A.order_cnt[grp] - 1ULL - atomicAdd(A.order_cnt + 48 + grp, 1ULL);
-    A.order_idx[at] = (int)pi;
-}
-
-// a9: persistent work-queue form.  A group of G lanes (G = 1, 8, 16 or 32) owns one path at
-// a time: lane l evaluates the sub-rays k = l, l + G, ... of each iteration and the group
-// takes the argmin with shuffles (lowest k on ties, as in the plain form; one lane runs
-// the plain form's iterate32).  When a path is finished (iteration cap, target reached,
-// stalled, or all sub-rays invalid) the group takes the next path index from the device
-// queue head with one atomic, so paths that stop early free their group at once.  With
-// many paths, a path whose cone falls below the FP64 threshold moves on to
-// batch_refine64_kernel; the validity test and outputs follow in batch_finalize_kernel.
 template <int G>
 __device__ __forceinline__ void group_argmin(float &e, int &k, unsigned gmask) {
 #pragma unroll
@@ -1108,6 +974,212 @@ __device__ void group_finalize(const RefineArgs &A, const PathGeo &g, dvec3 c, s
     if (gl == 0) path_outputs(A, g, c, last, tsum, gain_db, p);
 }
 
+// ----------------------------------------------------------------------------- phases
+// The state of a path's iterations: cone centre, |d x W|^2 and d . W in the precision of the
+// phase that set them (fp64: in FP64), iterations done, flags and why they ended.
+struct Iterated {
+    float3 cf;
+    float keyf, dwf, Rf;
+    dvec3 c;
+    double key, dw, R;
+    int it, flags, stop;
+    bool fp64, fail;
+};
+
+// FP32 phase while the cone radius is >= fp64_below (the radius R0 = max(theta_launch, rough
+// error) is a float, so the first test is exact), from the rough direction x.cf.  G lanes share a
+// path (state identical in them), G = 1: a thread its own.
+template <int G>
+__device__ __forceinline__ void fp32_phase(const RefineArgs &A, const PathGeo &g, const UnfF &uf, int off, float rough_err,
+                                           float shrinkf, float stallf, long long pi, int gl, unsigned gmask, Iterated &x) {
+    x.Rf = fmaxf(A.theta_launch, rough_err);
+    x.fp64 = x.Rf < A.fp64_below_f;
+    x.fail = false;
+    x.keyf = INFINITY;
+    x.dwf = 0.0f;
+    x.it = x.flags = 0;
+    x.stop = kStopNone;
+    if (x.fp64) return;
+    x.keyf = key32(uf, g.k, x.cf, x.dwf);
+    while (x.it < A.max_iters) {
+        if (reached32(A, g, uf, x.cf, x.keyf, x.dwf)) {
+            x.stop = kStopReached;
+            break;
+        }
+        if (stalled32(x.keyf, x.dwf, x.Rf, stallf)) {
+            x.stop = kStopStalled;
+            break;
+        }
+        if (x.Rf < A.fp64_below_f) break;   // on to the FP64 iterations
+        const int ax = A.choice_log ? frame_axis32(x.cf) : 0;
+        const int bk = G == 1 ? iterate32(uf, g.k, A.K, off, x.Rf, x.cf, x.keyf, x.dwf)
+                              : group_iterate32<G>(uf, g.k, A.K, off, x.Rf, x.cf, x.keyf, x.dwf, gl, gmask);
+        if (bk < 0) {
+            x.fail = true;
+            break;
+        }
+        if (A.choice_log && gl == 0) A.choice_log[pi * A.max_iters + x.it] = choice_entry(bk, ax);
+        x.Rf *= shrinkf;
+        ++x.it;
+    }
+}
+
+// FP64 phase, from the FP32 phase's centre with its |d x W|^2 and d . W, or, with no iteration
+// done, from the FP64 rough direction.  A thread a path; several may run it in step (log: one of
+// them writes the choice log).
+__device__ __forceinline__ void fp64_phase(const RefineArgs &A, const PathGeo &g, const UnfD &ud, int off,
+                                           const SubTab64 &tab, const sbr_path_record &p, double shrink, double stall,
+                                           long long pi, bool log, Iterated &x) {
+    x.R = cone_radius64(A, p.rough_err, x.it, shrink);
+    if (x.fp64) {
+        x.c = dv(p.dir[0], p.dir[1], p.dir[2]);
+        x.key = key64(ud, g.k, x.c, x.dw);
+    } else {
+        x.c = dv(x.cf.x, x.cf.y, x.cf.z);
+        x.key = x.keyf;
+        x.dw = x.dwf;
+    }
+    x.stop = kStopNone;   // this phase judges the state again
+    while (x.it < A.max_iters) {
+        if (reached(A, g, ud, x.c, x.key, x.dw)) {
+            x.stop = kStopReached;
+            break;
+        }
+        if (stalled(x.key, x.dw, x.R, stall)) {
+            x.stop = kStopStalled;
+            break;
+        }
+        const int ax = A.choice_log ? frame_axis64(x.c) : 0;
+        const int bk = iterate64(ud, g.k, A.K, off, tab, x.R, x.c, x.key, x.dw);
+        if (bk < 0) {
+            x.fail = true;
+            break;
+        }
+        x.flags |= SBR_PATH_FP64;
+        x.fp64 = true;
+        if (log) A.choice_log[pi * A.max_iters + x.it] = choice_entry(bk, ax);
+        x.R *= shrink;
+        ++x.it;
+    }
+}
+
+// The result of the iterations in the record: direction, error angle, iterations and flags.
+__device__ __forceinline__ void put_iterated(const Iterated &x, dvec3 c, sbr_path_record &p) {
+    int flags = x.flags;
+    if (x.fail) flags |= SBR_PATH_TRACE_FAIL;
+    else if (x.stop == kStopStalled) flags |= SBR_PATH_STALLED;
+    p.iters = x.it;
+    p.flags = flags | (x.it > 0 ? SBR_PATH_REFINED : 0);
+    p.dir[0] = c.x;
+    p.dir[1] = c.y;
+    p.dir[2] = c.z;
+    p.err = error_angle(x.key, x.dw, x.keyf, x.dwf, x.fp64);
+}
+
+// a6-a8 in one launch with nothing shared between paths (static schedule): the plain and per-pair
+// forms.  A thread a path, or, while there are at most kPlainWide paths a warp of the grid, a warp
+// a path: few paths leave the chip idle and a thread's own chain of mirrors, K sub-rays, bounce
+// points and occlusion queries is what the launch waits for, so its lanes take them side by
+// side, as in the batched form's groups (110 paths of a cluttered room: 193 -> 45 us).
+constexpr int kPlainWide = 3;
+__global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
+    __shared__ SubTab64 tab;
+    __shared__ UnfF s_uf[4];
+    __shared__ UnfD s_ud[4];
+    const long long total = A.range ? (long long)(A.range[1] - A.range[0]) : path_count(A);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+    const bool wide = total <= kPlainWide * warps;
+    const int off = c_sub.off[A.K];
+    const double shrink = c_sub.shrink[A.K];
+    const float shrinkf = c_sub.shrink_f[A.K];
+    const double stall = 1.0 / (1.0 - shrink) + 2.0 * shrink;
+    const float stallf = (float)stall;
+    load_sub64(tab);
+    const long long first = wide ? (long long)blockIdx.x * (blockDim.x >> 5) + wid
+                                 : blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long stride = wide ? warps : (long long)gridDim.x * blockDim.x;
+    for (long long i = first; i < total; i += stride) {
+        const long long pi = A.range ? (long long)A.index[A.range[0] + i] : i;
+        sbr_path_record p = A.paths[pi];
+        if (!path_ids_ok(A, p)) {
+            if (!wide || lane == 0) {
+                A.paths[pi].valid = 0;
+                A.paths[pi].flags = SBR_PATH_TRACE_FAIL;
+            }
+            continue;
+        }
+        PathGeo g;
+        load_path(A, p, g);
+        Iterated x;
+        x.cf = make_float3((float)p.dir[0], (float)p.dir[1], (float)p.dir[2]);
+        x.key = INFINITY;
+        x.dw = 0.0;
+        UnfD ud;
+        if (wide) {
+            UnfF &uf = s_uf[wid];
+            __syncwarp();
+            if (lane < g.k) uf.p[lane] = unfold_plane32(A.scene, g, lane);
+            if (lane == 31) uf.w = unfold_rx32(A.scene, g);
+            __syncwarp();
+            fp32_phase<32>(A, g, uf, off, p.rough_err, shrinkf, stallf, pi, lane, 0xffffffffu, x);
+        } else {
+            UnfF uf;
+            for (int j = 0; j < g.k; ++j) uf.p[j] = unfold_plane32(A.scene, g, j);
+            uf.w = unfold_rx32(A.scene, g);
+            fp32_phase<1>(A, g, uf, off, p.rough_err, shrinkf, stallf, pi, 0, 0, x);
+        }
+        dvec3 c = dv(x.cf.x, x.cf.y, x.cf.z);
+        if (!x.fail && x.Rf < A.fp64_below_f) {
+            if (wide) {
+                if (lane < g.k) s_ud[wid].p[lane] = unfold_plane(A.scene, g, lane);
+                if (lane == 31) s_ud[wid].w = unfold_rx(A.scene, g);
+                __syncwarp();
+                for (int j = 0; j < g.k; ++j) ud.p[j] = s_ud[wid].p[j];
+                ud.w = s_ud[wid].w;
+            } else {
+                for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
+                ud.w = unfold_rx(A.scene, g);
+            }
+            fp64_phase(A, g, ud, off, tab, p, shrink, stall, pi, A.choice_log && (!wide || lane == 0), x);
+            c = x.c;
+        }
+        put_iterated(x, c, p);
+        const double bound = converged_bound(x.it, cone_radius64(A, p.rough_err, x.it, shrink));
+        if (wide) {
+            group_finalize<32>(A, g, c, p, lane, 0xffffffffu, bound);
+            if (lane == 0) store_result(A.paths + pi, p);
+        } else {
+            finalize_path(A, g, c, p, bound);
+            store_result(A.paths + pi, p);
+        }
+    }
+}
+
+// Lists path pi in its order group for batch_finalize_kernel (group offsets from
+// batch_unfold_kernel's counts), so that a warp there holds paths of one order.  Inside the
+// group, paths whose error meets the convergence bound 2 R + 1e-7 (the validity test's
+// condition; R is the cone radius after the iterations, here only an ordering hint) fill it
+// from the front and the others, which the validity test rejects at once, from the back:
+// a warp's lanes then run their BVH queries, or skip them, together.
+__device__ __forceinline__ void list_for_finalize(const RefineArgs &A, const PathGeo &g, long long pi, double err,
+                                                  double R) {
+    const int grp = order_group(g);
+    unsigned long long at = 0;
+    for (int b = 0; b < grp; ++b) at += A.order_cnt[b];
+    if (err <= 2.0 * R + 1e-7) at += atomicAdd(A.order_cnt + 16 + grp, 1ULL);
+    else at += A.order_cnt[grp] - 1ULL - atomicAdd(A.order_cnt + 48 + grp, 1ULL);
+    A.order_idx[at] = (int)pi;
+}
+
+// a9: persistent work-queue form.  A group of G lanes (G = 1, 8, 16 or 32) owns one path at
+// a time: lane l evaluates the sub-rays k = l, l + G, ... of each iteration and the group
+// takes the argmin with shuffles (lowest k on ties, as in the plain form; one lane runs
+// the plain form's iterate32).  When a path is finished (iteration cap, target reached,
+// stalled, or all sub-rays invalid) the group takes the next path index from the device
+// queue head with one atomic, so paths that stop early free their group at once.  With
+// many paths, a path whose cone falls below the FP64 threshold moves on to
+// batch_refine64_kernel; the validity test and outputs follow in batch_finalize_kernel.
 // At most 85 registers a thread, so that three 256-thread blocks fit on an SM (measured
 // faster than the uncapped 124-128 registers of the 8- and 32-lane forms).
 // G = 1 is the one-lane form: each thread evaluates all K sub-rays of its own path (no
@@ -1170,68 +1242,39 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
             cf = make_float3((float)p.dir[0], (float)p.dir[1], (float)p.dir[2]);
         }
         __syncwarp(gmask);
-        // FP32 phase, every operand in FP32 (see cone_radius64); state identical in the G lanes
-        float Rf = fmaxf(A.theta_launch, p.rough_err);
-        bool fp64 = Rf < A.fp64_below_f, fail = false;
-        float keyf = INFINITY, dwf = 0.0f;
-        int it = 0, flags = 0, stop = kStopNone;
-        if (!fp64) {
-            keyf = key32(uf, g.k, cf, dwf);
-            while (it < A.max_iters) {
-                if (reached32(A, g, uf, cf, keyf, dwf)) {
-                    stop = kStopReached;
-                    break;
-                }
-                if (stalled32(keyf, dwf, Rf, stallf)) {
-                    stop = kStopStalled;
-                    break;
-                }
-                if (Rf < A.fp64_below_f) break;   // on to the FP64 iterations
-                const int ax = A.choice_log ? frame_axis32(cf) : 0;
-                const int bk = G == 1 ? iterate32(uf, g.k, A.K, off, Rf, cf, keyf, dwf)
-                                      : group_iterate32<G>(uf, g.k, A.K, off, Rf, cf, keyf, dwf, gl, gmask);
-                if (bk < 0) {
-                    fail = true;
-                    break;
-                }
-                if (A.choice_log && gl == 0) A.choice_log[pi * A.max_iters + it] = choice_entry(bk, ax);
-                Rf *= shrinkf;
-                ++it;
-            }
-        }
-        if (!fail && Rf < A.fp64_below_f) {
+        // FP32 phase, every operand in FP32 (see cone_radius64)
+        Iterated x;
+        x.cf = cf;
+        fp32_phase<G>(A, g, uf, off, p.rough_err, shrinkf, stallf, pi, gl, gmask, x);
+        if (gl != 0) continue;
+        sbr_path_record *dst = A.paths + pi;
+        if (!x.fail && x.Rf < A.fp64_below_f) {
             // the FP64 iterations run in batch_refine64_kernel, one thread per path.  The
             // record keeps the iterations done; the path's unf slot keeps the cone centre and
             // |d x W|^2 of the FP32 phase, the record's err field d . W.  With many paths listed
             // by order group (group offsets from batch_unfold_kernel's counts), so that the
             // tail kernel's warps run paths of one order; with few in one group.
-            if (gl == 0) {
-                sbr_path_record *dst = A.paths + pi;
-                dst->iters = it;
-                dst->err = dwf;
-                A.unf[kUnfStride * pi + kMaxOrder + 1] = make_float4(cf.x, cf.y, cf.z, keyf);
-                const int grp = prebuilt ? order_group(g) : 0;
-                unsigned long long at = 0;
-                for (int b = 0; b < grp; ++b) at += A.order_cnt[b];
-                at += atomicAdd(A.order_cnt + 32 + grp, 1ULL);
-                A.fp64_idx[at] = (int)pi;
-            }
+            dst->iters = x.it;
+            dst->err = x.dwf;
+            A.unf[kUnfStride * pi + kMaxOrder + 1] = make_float4(x.cf.x, x.cf.y, x.cf.z, x.keyf);
+            const int grp = prebuilt ? order_group(g) : 0;
+            unsigned long long at = 0;
+            for (int b = 0; b < grp; ++b) at += A.order_cnt[b];
+            at += atomicAdd(A.order_cnt + 32 + grp, 1ULL);
+            A.fp64_idx[at] = (int)pi;
             continue;
         }
-        if (fail) flags |= SBR_PATH_TRACE_FAIL;
-        else if (stop == kStopStalled) flags |= SBR_PATH_STALLED;
-        if (gl == 0) {
-            p.err = error_angle(INFINITY, 0.0, keyf, dwf, false);
-            if (prebuilt) list_for_finalize(A, g, pi, p.err, (double)Rf);
-            // iteration results; the validity test and outputs follow in batch_finalize_kernel
-            sbr_path_record *dst = A.paths + pi;
-            dst->iters = it;
-            dst->dir[0] = cf.x;
-            dst->dir[1] = cf.y;
-            dst->dir[2] = cf.z;
-            dst->err = p.err;
-            dst->flags = flags | (it > 0 ? SBR_PATH_REFINED : 0);
-        }
+        x.key = INFINITY;
+        x.dw = 0.0;
+        put_iterated(x, dv(x.cf.x, x.cf.y, x.cf.z), p);
+        if (prebuilt) list_for_finalize(A, g, pi, p.err, (double)x.Rf);
+        // iteration results; the validity test and outputs follow in batch_finalize_kernel
+        dst->iters = p.iters;
+        dst->dir[0] = p.dir[0];
+        dst->dir[1] = p.dir[1];
+        dst->dir[2] = p.dir[2];
+        dst->err = p.err;
+        dst->flags = p.flags;
     }
 }
 
@@ -1289,62 +1332,31 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
             ud.w = unfold_rx(A.scene, g);
         }
         const float4 cu = u[kMaxOrder + 1];
-        const float3 cf = f3(cu);
-        const float keyf = cu.w, dwf = (float)p.err;
-        int it = p.iters, flags = 0;
-        bool fp64 = it == 0, fail = false;
-        double R = cone_radius64(A, p.rough_err, it, shrink);
-        dvec3 c;
-        double key, dw = 0.0;
-        if (fp64) {
-            c = dv(p.dir[0], p.dir[1], p.dir[2]);
-            key = key64(ud, g.k, c, dw);
-        } else {
-            c = dv(cf.x, cf.y, cf.z);
-            key = keyf;
-            dw = dwf;
-        }
-        int stop = kStopNone;
-        while (it < A.max_iters) {
-            if (reached(A, g, ud, c, key, dw)) {
-                stop = kStopReached;
-                break;
-            }
-            if (stalled(key, dw, R, stall)) {
-                stop = kStopStalled;
-                break;
-            }
-            const int ax = A.choice_log ? frame_axis64(c) : 0;
-            const int bk = iterate64(ud, g.k, A.K, off, tab, R, c, key, dw);
-            if (bk < 0) {
-                fail = true;
-                break;
-            }
-            flags |= SBR_PATH_FP64;
-            fp64 = true;
-            if (A.choice_log && (!wide || lane == 0)) A.choice_log[pi * A.max_iters + it] = choice_entry(bk, ax);
-            R *= shrink;
-            ++it;
-        }
-        if (fail) flags |= SBR_PATH_TRACE_FAIL;
-        else if (stop == kStopStalled) flags |= SBR_PATH_STALLED;
-        if (!fp64) c = dv(cf.x, cf.y, cf.z);
+        Iterated x;
+        x.cf = f3(cu);
+        x.keyf = cu.w;
+        x.dwf = (float)p.err;
+        x.it = p.iters;
+        x.flags = 0;
+        x.fp64 = x.it == 0;
+        x.fail = false;
+        fp64_phase(A, g, ud, off, tab, p, shrink, stall, pi, A.choice_log && (!wide || lane == 0), x);
         if (wide && lane != 0) continue;   // the lanes agree
-        const double err = error_angle(key, dw, keyf, dwf, fp64);
-        if (many) list_for_finalize(A, g, pi, err, R);
+        put_iterated(x, x.fp64 ? x.c : dv(x.cf.x, x.cf.y, x.cf.z), p);
+        if (many) list_for_finalize(A, g, pi, p.err, x.R);
         sbr_path_record *dst = A.paths + pi;
-        dst->iters = it;
-        dst->dir[0] = c.x;
-        dst->dir[1] = c.y;
-        dst->dir[2] = c.z;
-        dst->err = err;
-        dst->flags = flags | (it > 0 ? SBR_PATH_REFINED : 0);
+        dst->iters = p.iters;
+        dst->dir[0] = p.dir[0];
+        dst->dir[1] = p.dir[1];
+        dst->dir[2] = p.dir[2];
+        dst->err = p.err;
+        dst->flags = p.flags;
     }
 }
 
 // Batched form, first pass (from split_min paths on), one thread per path: the FP64
 // unfolding of the path's face planes into Tx's space and of the receiver (the same
-// arithmetic as the plain form's build_unf), stored rounded to FP32 for the iteration
+// arithmetic as the plain form's), stored rounded to FP32 for the iteration
 // kernel, with the rough launch direction rounded to FP32.  GB300 runs FP64 at 1/64 of
 // the FP32 rate; with one path per lane every FP64 instruction serves 32 paths, where the
 // iteration kernel's lane groups would serve one.
