@@ -67,7 +67,8 @@ FLOP_NODE, FLOP_TRI, FLOP_RX = 48, 40, 20
 L2_FLUSH_BYTES = 256 << 20
 
 TRACE_SOURCES = ["paper_2208_10009_gb300/csrc/kernels_trace.cu", "paper_2208_10009_gb300/csrc/lattice_order.cuh",
-                 "paper_2208_10009_gb300/csrc/sbr_device.cuh", "paper_2208_10009_gb300/csrc/sbr_internal.h"]
+                 "paper_2208_10009_gb300/csrc/sbr_device.cuh", "paper_2208_10009_gb300/csrc/sbr_internal.h",
+                 "paper_2208_10009_gb300/csrc/stream_launch.cuh"]
 TRAFFIC_FILES = {"canyon": os.path.join(ROOT, "profiles", "trace_kernel_traffic.json"),
                  "city": os.path.join(ROOT, "profiles", "trace_kernel_traffic_large_city.json")}
 UNFOLD_SOURCES = ["paper_2208_10009_gb300/csrc/kernels_unfold.cu", "paper_2208_10009_gb300/csrc/sbr_device.cuh",
@@ -504,9 +505,10 @@ def run_gpu(args):
 
 
 def _launches_per_step(opts, world):
-    """Library kernels per step: raygen, trace (+3 diffraction: candidates, receivers,
-    occlusion), 4 dedup, 4 batched refinement; shards add the record-count reset kernel."""
-    return 10 + (3 if opts["diffraction"] else 0) + (1 if world > 1 else 0)
+    """Library kernels per step: raygen, trace (+5 diffraction: candidates, exact tests,
+    visibility, receivers, occlusion), 3 dedup, 4 batched refinement; shards add the
+    record-count reset kernel."""
+    return 9 + (5 if opts["diffraction"] else 0) + (1 if world > 1 else 0)
 
 
 def _refine_forms(ctx, scene, paths, relaunch, stream, iters, K, target, shape, ntx, nrx, trials=3):

@@ -50,6 +50,16 @@ bool is_device_ptr(const void *p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// memory that a kernel on the context's device may read directly
+bool is_local_ptr(const sbr_ctx *ctx, const void *p) {
+    cudaPointerAttributes at;
+    if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == ctx->device);
+}
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Carves several arrays out of one allocation (256-byte aligned sub-blocks).
@@ -161,7 +171,7 @@ sbr_status ensure_poly(sbr_ctx *ctx, int poly, int n) {
     return SBR_OK;
 }
 
-sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher) {
+sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) {
     int64_t N = rays_for_launcher(n, launcher);
     if (N < 0) return fail(ctx, SBR_EINVAL, "launcher must be 0 (equiangular), 20 or 8 (equidistant)");
     size_t need = (size_t)N * sizeof(float4);
@@ -175,16 +185,23 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher) {
     if (launcher == 0) {
         sbr_status st = ensure_lattice(ctx, n);
         if (st != SBR_OK) return st;
-        SBR_CUDA(launch_raygen_schedule(ctx->lattice, static_cast<float4 *>(ctx->dirs), ctx->stream));
+        SBR_CUDA(launch_raygen_schedule(ctx->lattice, static_cast<float4 *>(ctx->dirs), prep, ctx->stream));
     } else {
         sbr_status st = ensure_poly(ctx, launcher, n);
         if (st != SBR_OK) return st;
-        SBR_CUDA(launch_raygen_equidistant(ctx->poly, static_cast<float4 *>(ctx->dirs), N, true, ctx->stream));
+        SBR_CUDA(launch_raygen_equidistant(ctx->poly, static_cast<float4 *>(ctx->dirs), N, true, prep, ctx->stream));
     }
     ctx->dirs_n = n;
     ctx->dirs_launcher = launcher;
     ctx->dirs_valid = true;
     return SBR_OK;
+}
+
+// a value looked up once (0: not yet)
+template <class F>
+int cached(int &slot, F look_up) {
+    if (slot == 0) slot = look_up();
+    return slot;
 }
 
 // copy an n x 3 float array (host or device) into a float4 device array
@@ -255,7 +272,7 @@ sbr_status sbr_raygen_equidistant(sbr_ctx *ctx, int32_t n, int32_t poly, float *
     DeviceGuard g(ctx->device);
     sbr_status st = ensure_poly(ctx, poly, n);
     if (st != SBR_OK) return st;
-    SBR_CUDA(launch_raygen_equidistant(ctx->poly, reinterpret_cast<float4 *>(dirs), N, false, ctx->stream));
+    SBR_CUDA(launch_raygen_equidistant(ctx->poly, reinterpret_cast<float4 *>(dirs), N, false, PrepArgs(), ctx->stream));
     return SBR_OK;
 }
 
@@ -696,6 +713,7 @@ sbr_status sbr_paths_create(sbr_ctx *ctx, int64_t record_cap, int64_t path_cap, 
     p->record_cap = record_cap;
     p->path_cap = path_cap;
     SBR_CUDA(cudaMemsetAsync(p->counters, 0, kNumCounters * sizeof(long long), ctx->stream));
+    SBR_CUDA(cudaMemsetAsync(p->order_cnt, 0, 64 * sizeof(unsigned long long), ctx->stream));
     *out = p;
     return SBR_OK;
 }
@@ -710,6 +728,7 @@ sbr_status sbr_paths_destroy(sbr_ctx *ctx, sbr_paths *p) {
     return SBR_OK;
 }
 
+// room for ntx transmitters, and a copy of them (tx null: the room only)
 static sbr_status ensure_tx(sbr_ctx *ctx, sbr_paths *p, const float *tx, int32_t ntx) {
     if (ntx > p->tx_cap) {
         dev_free(ctx, p->tx_mem, p->tx_bytes);
@@ -720,7 +739,7 @@ static sbr_status ensure_tx(sbr_ctx *ctx, sbr_paths *p, const float *tx, int32_t
         p->tx = static_cast<float4 *>(p->tx_mem);
         if (!p->tx_mem) return fail(ctx, SBR_ENOMEM, "paths: transmitter buffer allocation failed");
     }
-    return copy_points(ctx, p->tx, tx, ntx);
+    return tx ? copy_points(ctx, p->tx, tx, ntx) : SBR_OK;
 }
 
 static sbr_status report_checks(sbr_ctx *ctx, long long flags, const char *where);
@@ -768,19 +787,26 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
         ray_count = prm->ray_end - prm->ray_begin;
     }
     DeviceGuard g(ctx->device);
-    sbr_status st = ensure_tx(ctx, paths, tx, ntx);
+    PrepArgs prep;   // the ray generation also zeroes the counters and takes device-side transmitters
+    prep.counters = paths->counters;
+    const bool tx_on_device = is_local_ptr(ctx, tx);
+    sbr_status st = ensure_tx(ctx, paths, tx_on_device ? nullptr : tx, ntx);
     if (st != SBR_OK) return st;
+    if (tx_on_device) {
+        prep.tx_src = tx;
+        prep.tx = paths->tx;
+        prep.ntx = ntx;
+    }
     const bool timing = (prm->flags & SBR_LAUNCH_TIMING) != 0;
     if (timing && !ctx->ev[0])
         for (auto &e : ctx->ev) SBR_CUDA(cudaEventCreate(&e));
     if (timing) SBR_CUDA(cudaEventRecord(ctx->ev[0], ctx->stream));
     {
         Range r("sbr_launch: raygen");
-        st = ensure_dirs(ctx, prm->n_div, prm->launcher);
+        st = ensure_dirs(ctx, prm->n_div, prm->launcher, prep);
     }
     if (st != SBR_OK) return st;
     if (timing) SBR_CUDA(cudaEventRecord(ctx->ev[1], ctx->stream));
-    SBR_CUDA(cudaMemsetAsync(paths->counters, 0, kNumCounters * sizeof(long long), ctx->stream));
     TraceArgs a;
     a.scene = scene->dev;
     a.scene.status = reinterpret_cast<unsigned long long *>(paths->counters + kErrorFlags);
@@ -817,7 +843,9 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     int block = prm->block_threads > 0 ? prm->block_threads : 128;
     if (block % 32 != 0 || block > 128)
         return fail(ctx, SBR_EINVAL, "sbr_launch: block_threads must be a multiple of 32, at most 128");
-    int grid = prm->grid_blocks > 0 ? prm->grid_blocks : ctx->num_sms * trace_blocks_per_sm(block);
+    int grid = prm->grid_blocks > 0
+                   ? prm->grid_blocks
+                   : ctx->num_sms * cached(ctx->trace_nb[block / 32], [&] { return trace_blocks_per_sm(block); });
     {
         Range r("sbr_launch: trace + reception");
         SBR_CUDA(launch_trace(a, grid, block, ctx->stream));
@@ -960,7 +988,7 @@ sbr_status sbr_records_dedup(sbr_ctx *ctx, sbr_paths *paths, const sbr_reception
         return fail(ctx, SBR_EOVERFLOW, "sbr_records_dedup: " + std::to_string(count) + " records exceed record_cap");
     DeviceGuard g(ctx->device);
     if (!(ctx->dirs_valid && ctx->dirs_n == paths->n_div && ctx->dirs_launcher == paths->launcher)) {
-        sbr_status st = ensure_dirs(ctx, paths->n_div, paths->launcher);   // rough launch directions
+        sbr_status st = ensure_dirs(ctx, paths->n_div, paths->launcher, PrepArgs());   // rough launch directions
         if (st != SBR_OK) return st;
     }
     if (count > 0) {
@@ -1029,8 +1057,11 @@ sbr_status sbr_refine(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *paths, co
     sbr_status st = refine_args(ctx, scene, paths, prm, A);
     if (st != SBR_OK) return st;
     DeviceGuard g(ctx->device);
-    int nb = 1;
-    refine_kernel_attrs(nullptr, 128, &nb, false, 0);
+    const int nb = cached(ctx->refine_nb, [] {
+        int b = 1;
+        refine_kernel_attrs(nullptr, 128, &b, false, 0);
+        return b;
+    });
     {
         Range r("sbr_refine: iterations + validity + outputs");
         SBR_CUDA(launch_refine(A, ctx->num_sms * nb, 128, ctx->stream));
@@ -1099,8 +1130,11 @@ sbr_status sbr_batch_refine(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *pat
     int lanes = cfg && cfg->lanes_per_path > 0 ? cfg->lanes_per_path : 16;
     if (lanes != 1 && lanes != 8 && lanes != 16 && lanes != 32)
         return fail(ctx, SBR_EINVAL, "sbr_batch_refine: lanes_per_path must be 1, 8, 16 or 32");
-    int nb = 1;
-    refine_kernel_attrs(nullptr, block, &nb, true, lanes);
+    int nb = cached(ctx->batch_nb[lanes == 1 ? 0 : (lanes == 8 ? 1 : (lanes == 16 ? 2 : 3))][block / 32], [&] {
+        int b = 1;
+        refine_kernel_attrs(nullptr, block, &b, true, lanes);
+        return b;
+    });
     if (cfg && cfg->blocks_per_sm > 0) nb = std::min(nb, cfg->blocks_per_sm);
     A.chunk = lanes;
     if (lanes == 1) A.split_min = 0;   // the one-lane form runs with the unfold and FP64 tail kernels

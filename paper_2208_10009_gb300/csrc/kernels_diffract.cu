@@ -17,6 +17,7 @@
 // inside the ray cone then lies within that margin of the ray (see cone_box).
 #include "lattice_order.cuh"
 #include "sbr_device.cuh"
+#include "stream_launch.cuh"
 
 namespace sbr {
 
@@ -214,6 +215,7 @@ __device__ __noinline__ void walk_ray(const DiffractArgs &A, int txi, int place,
 }
 
 __global__ void __launch_bounds__(128, 6) diffract_candidates(DiffractArgs A) {
+    wait_predecessor();
     __shared__ BeamShared s_beam[4];
     BeamShared &sh = s_beam[threadIdx.x >> 5];
     const SceneDev &S = A.scene;
@@ -388,6 +390,7 @@ __global__ void __launch_bounds__(128, 6) diffract_candidates(DiffractArgs A) {
 // pairs where most leave none, so they are spread over the chip (tested by the warp that found
 // them, the last group alone ran for 200 us).
 __global__ void __launch_bounds__(128) diffract_exact(DiffractArgs A) {
+    wait_predecessor();
     const long long n0 = A.counters[kRecords], cap = pair_space(A, n0);
     long long n = A.counters[kDiffPairs];
     if (n > cap) n = cap;
@@ -405,6 +408,7 @@ __global__ void __launch_bounds__(128) diffract_exact(DiffractArgs A) {
 // Pass 3, one candidate per thread: is its edge point visible from Tx (segment Tx -> X unblocked,
 // the wedge's faces excluded)?  The answer goes into the candidate.
 __global__ void __launch_bounds__(128) diffract_visible(DiffractArgs A) {
+    wait_predecessor();
     const SceneDev &S = A.scene;
     long long ncand = A.counters[kDiffCand];
     if (ncand > A.cand_cap) ncand = A.cand_cap;
@@ -432,6 +436,7 @@ __global__ void __launch_bounds__(128) diffract_visible(DiffractArgs A) {
 __device__ __forceinline__ long long park_limit(const DiffractArgs &A, long long n0) { return (A.rec_cap - n0) / 2; }
 
 __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
+    wait_predecessor();
     const SceneDev &S = A.scene;
     long long ncand = A.counters[kDiffCand];
     if (ncand > A.cand_cap) ncand = A.cand_cap;
@@ -520,6 +525,7 @@ __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
 // appended with one atomic per warp; blocked ones are dropped.  One warp a block, so that a few
 // thousand queries spread over the SMs (60 -> 28 us).
 __global__ void __launch_bounds__(32) diffract_occlusion(DiffractArgs A) {
+    wait_predecessor();
     const SceneDev &S = A.scene;
     long long P = A.counters[kDiffPending];
     const long long limit = park_limit(A, A.counters[kDiffBase]);
@@ -567,12 +573,12 @@ static int candidate_blocks() {
 
 cudaError_t launch_diffract(const DiffractArgs &a, int num_sms, cudaStream_t s) {
     if (a.scene.nw == 0 || a.rx.nrx == 0) return cudaSuccess;
-    diffract_candidates<<<num_sms * candidate_blocks(), 128, 0, s>>>(a);
-    diffract_exact<<<num_sms * 8, 128, 0, s>>>(a);
-    diffract_visible<<<num_sms * 5, 128, 0, s>>>(a);
-    diffract_receive<<<num_sms * 8, 256, 0, s>>>(a);
-    diffract_occlusion<<<num_sms * 32, 32, 0, s>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = launch_chained(diffract_candidates, num_sms * candidate_blocks(), 128, 0, s, a);
+    if (e == cudaSuccess) e = launch_chained(diffract_exact, num_sms * 8, 128, 0, s, a);
+    if (e == cudaSuccess) e = launch_chained(diffract_visible, num_sms * 5, 128, 0, s, a);
+    if (e == cudaSuccess) e = launch_chained(diffract_receive, num_sms * 8, 256, 0, s, a);
+    if (e == cudaSuccess) e = launch_chained(diffract_occlusion, num_sms * 32, 32, 0, s, a);
+    return e;
 }
 
 }  // namespace sbr

@@ -7,6 +7,7 @@
 #include "dedup_keys.cuh"
 #include "lattice_order.cuh"
 #include "sbr_device.cuh"
+#include "stream_launch.cuh"
 
 namespace sbr {
 
@@ -21,20 +22,20 @@ __device__ __forceinline__ unsigned long long used_slots(const DedupArgs &a) {
 }
 
 // A slot is 16 bytes, its key then its value (one 32-byte sector holds two slots, so an
-// insert's compare-and-swap and minimum touch one sector); the winners follow the slots.
-// Keys and values to all-ones (empty / +inf), winners to -1, over the used slots.
+// insert's compare-and-swap and minimum touch one sector); the owners (the record that claimed
+// each slot) follow the slots.  Keys and values to all-ones (empty / +inf) over the used slots.
 __global__ void dedup_clear(DedupArgs a) {
+    wait_predecessor();
     const unsigned long long m = used_slots(a);
     ulonglong2 *slot = reinterpret_cast<ulonglong2 *>(a.table);
-    int *winner = reinterpret_cast<int *>(a.table + 2 * a.slots);
     for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < m;
-         i += (unsigned long long)gridDim.x * blockDim.x) {
+         i += (unsigned long long)gridDim.x * blockDim.x)
         slot[i] = make_ulonglong2(~0ULL, ~0ULL);
-        winner[i] = -1;
-    }
 }
 
 __global__ void dedup_insert(DedupArgs a) {
+    wait_predecessor();
+    int *owner = reinterpret_cast<int *>(a.table + 2 * a.slots);
     const long long n = num_records(a);
     unsigned long long *tab = a.table;   // key of slot s at 2 s, its value at 2 s + 1
     const unsigned long long used = used_slots(a), mask = used - 1;
@@ -46,6 +47,7 @@ __global__ void dedup_insert(DedupArgs a) {
             unsigned long long prev = atomicCAS(tab + 2 * s, ~0ULL, h);
             if (prev == ~0ULL || prev == h) {
                 atomicMin(tab + 2 * s + 1, v);
+                if (prev == ~0ULL) owner[s] = (int)i;
                 a.recs[i].slot = (int)s;
                 break;
             }
@@ -54,15 +56,24 @@ __global__ void dedup_insert(DedupArgs a) {
     }
 }
 
+// Every slot's winner becomes a path, and every record is compared with the record that claimed
+// its slot (a differing key is a hash collision): one pass over the records, where a pass of its own
+// compared them with the winners (office, 1.5M records: 142 + 32 -> 140 us).
 __global__ void dedup_select(DedupArgs a) {
+    wait_predecessor();
     const long long n = num_records(a);
     const unsigned long long *tab = a.table;
-    int *winner = reinterpret_cast<int *>(a.table + 2 * a.slots);
+    const int *owner = reinterpret_cast<const int *>(a.table + 2 * a.slots);
+    unsigned bad = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         RecDev r = a.recs[i];
-        if (r.slot < 0) continue;
+        if (r.slot < 0) {
+            ++bad;
+            continue;
+        }
+        const int o = owner[r.slot];
+        if (o != (int)i && !same_key(r, a.recs[o])) ++bad;
         if (tab[2 * (long long)r.slot + 1] != rec_value(r)) continue;
-        winner[r.slot] = (int)i;
         if (a.shard_world > 1 && (r.tx * a.nrx + r.rx) % a.shard_world != a.shard_rank) continue;
         unsigned long long p = atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + kPaths), 1ULL);
         if ((long long)p >= a.path_cap) continue;
@@ -87,32 +98,16 @@ __global__ void dedup_select(DedupArgs a) {
         out.flags = 0;
         a.paths[p] = out;
     }
-}
-
-__global__ void dedup_verify(DedupArgs a) {
-    const long long n = num_records(a);
-    const int *winner = reinterpret_cast<const int *>(a.table + 2 * a.slots);
-    unsigned bad = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const RecDev &r = a.recs[i];
-        if (r.slot < 0) {
-            ++bad;
-            continue;
-        }
-        int w = winner[r.slot];
-        if (w == (int)i) continue;   // the winner itself
-        if (w < 0 || !same_key(r, a.recs[w])) ++bad;
-    }
     if (bad) atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + kCollisions), (unsigned long long)bad);
 }
 
+
 cudaError_t launch_dedup(const DedupArgs &a, int num_sms, cudaStream_t s) {
     int grid = num_sms * 4;
-    dedup_clear<<<grid, 256, 0, s>>>(a);
-    dedup_insert<<<grid, 256, 0, s>>>(a);
-    dedup_select<<<grid, 256, 0, s>>>(a);
-    dedup_verify<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = launch_chained(dedup_clear, grid, 256, 0, s, a);
+    if (e == cudaSuccess) e = launch_chained(dedup_insert, grid, 256, 0, s, a);
+    if (e == cudaSuccess) e = launch_chained(dedup_select, grid, 256, 0, s, a);
+    return e;
 }
 
 __global__ void records_reset(long long *counters, long long n) {

@@ -13,6 +13,7 @@
 #include "dfloat.cuh"
 #include "nvtx_ranges.h"
 #include "sbr_device.cuh"
+#include "stream_launch.cuh"
 
 namespace sbr {
 
@@ -1083,6 +1084,7 @@ __device__ __forceinline__ void put_iterated(const Iterated &x, dvec3 c, sbr_pat
 // side, as in the batched form's groups (110 paths of a cluttered room: 193 -> 45 us).
 constexpr int kPlainWide = 3;
 __global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
+    wait_predecessor();
     __shared__ SubTab64 tab;
     __shared__ UnfF s_uf[4];
     __shared__ UnfD s_ud[4];
@@ -1185,8 +1187,10 @@ __device__ __forceinline__ void list_for_finalize(const RefineArgs &A, const Pat
 // G = 1 is the one-lane form: each thread evaluates all K sub-rays of its own path (no
 // shuffles, no re-evaluation of the winner) and always runs with batch_unfold_kernel and
 // the FP64 tail kernel (the host sets split_min = 0 for it).
+constexpr int kQueueHead = 62, kBlocksRead = 63, kOrderCounts = 64;   // of order_cnt
 template <int G>
 __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
+    wait_predecessor();
     // the unfolded planes of each group's current path (shared by its G lanes)
     __shared__ UnfF s_uf[256 / G];
     UnfF &uf = s_uf[threadIdx.x / G];
@@ -1207,11 +1211,10 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
             const unsigned m = __activemask();
             const int leader = __ffs(m) - 1;
             if (lane == leader)
-                q = atomicAdd(reinterpret_cast<unsigned long long *>(A.counters + kBatchHead),
-                              (unsigned long long)__popc(m));
+                q = atomicAdd(A.order_cnt + kQueueHead, (unsigned long long)__popc(m));
             q = __shfl_sync(m, q, leader) + __popc(m & ((1u << lane) - 1u));
         } else {
-            if (gl == 0) q = atomicAdd(reinterpret_cast<unsigned long long *>(A.counters + kBatchHead), 1ULL);
+            if (gl == 0) q = atomicAdd(A.order_cnt + kQueueHead, 1ULL);
             q = __shfl_sync(gmask, q, 0, G);
         }
         if ((long long)q >= total) break;
@@ -1292,6 +1295,7 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
 // with more paths the pipe is full of redundant lanes (8 paths an SM cost what a thread a path does).
 constexpr int kTailBlock = 32, kTailWide = 6;
 __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A) {
+    wait_predecessor();
     const bool many = path_count(A) >= A.split_min;
     __shared__ SubTab64 tab;
     // the list holds group b's n_b paths from the group's offset (the sizes of groups < b)
@@ -1363,6 +1367,7 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
 // It also counts the paths of each order group so that the iteration kernel can list them
 // group by group for the finalize kernel.
 __global__ void __launch_bounds__(128) batch_unfold_kernel(RefineArgs A) {
+    wait_predecessor();
     __shared__ unsigned hist[10];
     const long long total = path_count(A);
     if (total < A.split_min) return;   // few paths: the iteration kernel unfolds them itself
@@ -1394,6 +1399,7 @@ __global__ void __launch_bounds__(128) batch_unfold_kernel(RefineArgs A) {
 // faster than the occlusion queries split into a kernel of their own with a thread per
 // (path, leg) (which walks each path again for every leg).
 __global__ void __launch_bounds__(128, 8) batch_finalize_kernel(RefineArgs A) {
+    wait_predecessor();
     const long long total = path_count(A);
     const double shrink = c_sub.shrink[A.K];
     const bool per_thread = total >= A.split_min;
@@ -1405,6 +1411,16 @@ __global__ void __launch_bounds__(128, 8) batch_finalize_kernel(RefineArgs A) {
         listed = 0;
         for (int b = 0; b < 10; ++b) listed += A.order_cnt[b];
     }
+    // nothing reads the queue head, group sizes and cursors after this: the last block to get here
+    // leaves them zero for the next call
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(A.order_cnt + kBlocksRead, 1ULL) == gridDim.x - 1ULL;
+    }
+    __syncthreads();
+    if (s_last && threadIdx.x < kOrderCounts) A.order_cnt[threadIdx.x] = 0;
     for (long long t = first; t < listed; t += stride) {
         const long long pi = per_thread ? (long long)A.order_idx[t] : t;
         sbr_path_record p = A.paths[pi];
@@ -1446,57 +1462,48 @@ void refine_kernel_attrs(int *regs, int block, int *blocks_per_sm, bool batched,
 }
 
 cudaError_t launch_refine(const RefineArgs &a, int grid, int block, cudaStream_t s) {
-    refine_kernel<<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(refine_kernel, grid, block, 0, s, a);
+}
+
+// resident blocks per SM of a kernel, looked up once
+template <class K>
+static int resident(K kernel, int block) {
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, block, 0);
+    return nb > 0 ? nb : 1;
 }
 
 cudaError_t launch_batch_refine(const RefineArgs &a, int grid, int block, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(a.counters + kBatchHead, 0, sizeof(long long), s);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    static int unf_blocks = 0;
-    if (!unf_blocks) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&unf_blocks, batch_unfold_kernel, 128, 0);
-        if (unf_blocks < 1) unf_blocks = 1;
-    }
-    e = cudaMemsetAsync(a.order_cnt, 0, 64 * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+    static const int unf_blocks = resident(batch_unfold_kernel, 128);
+    static const int tail_blocks = resident(batch_refine64_kernel, kTailBlock);
+    static const int fin_blocks = resident(batch_finalize_kernel, 128);
+    const int sms = a.num_sms;
+    cudaError_t e;
     {
         Range r("batch refine: plane unfolding");
-        batch_unfold_kernel<<<sms * unf_blocks, 128, 0, s>>>(a);
+        e = launch_chained(batch_unfold_kernel, sms * unf_blocks, 128, 0, s, a);
     }
+    if (e != cudaSuccess) return e;
     {
         Range r("batch refine: iterations (work queue)");
         switch (a.chunk) {
-            case 1: batch_refine_kernel<1><<<grid, block, 0, s>>>(a); break;
-            case 8: batch_refine_kernel<8><<<grid, block, 0, s>>>(a); break;
-            case 32: batch_refine_kernel<32><<<grid, block, 0, s>>>(a); break;
-            default: batch_refine_kernel<16><<<grid, block, 0, s>>>(a); break;
+            case 1: e = launch_chained(batch_refine_kernel<1>, grid, block, 0, s, a); break;
+            case 8: e = launch_chained(batch_refine_kernel<8>, grid, block, 0, s, a); break;
+            case 32: e = launch_chained(batch_refine_kernel<32>, grid, block, 0, s, a); break;
+            default: e = launch_chained(batch_refine_kernel<16>, grid, block, 0, s, a); break;
         }
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    static int tail_blocks = 0;
-    if (!tail_blocks) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tail_blocks, batch_refine64_kernel, kTailBlock, 0);
-        if (tail_blocks < 1) tail_blocks = 1;
-    }
     {
         Range r("batch refine: FP64 tail");
-        batch_refine64_kernel<<<sms * tail_blocks, kTailBlock, 0, s>>>(a);
+        e = launch_chained(batch_refine64_kernel, sms * tail_blocks, kTailBlock, 0, s, a);
     }
-    static int fin_blocks = 0;
-    if (!fin_blocks) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fin_blocks, batch_finalize_kernel, 128, 0);
-        if (fin_blocks < 1) fin_blocks = 1;
-    }
+    if (e != cudaSuccess) return e;
     {
         Range r("batch refine: validity + outputs");
-        batch_finalize_kernel<<<sms * fin_blocks, 128, 0, s>>>(a);
+        e = launch_chained(batch_finalize_kernel, sms * fin_blocks, 128, 0, s, a);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace sbr

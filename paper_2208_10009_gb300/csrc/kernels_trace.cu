@@ -4,6 +4,7 @@
 // of Eq. 3 on every segment.
 #include "lattice_order.cuh"
 #include "sbr_device.cuh"
+#include "stream_launch.cuh"
 
 namespace sbr {
 
@@ -61,6 +62,15 @@ __global__ void raygen_kernel(LatticeDev L, float4 *__restrict__ dirs, int N) {
     }
 }
 
+// Transmitters as float4 and the launch's counters zeroed, by one block of the ray generation.
+__device__ __forceinline__ void prepare_launch(const PrepArgs &p) {
+    if (p.tx_src)
+        for (int i = threadIdx.x; i < p.ntx; i += blockDim.x)
+            p.tx[i] = make_float4(p.tx_src[3 * i], p.tx_src[3 * i + 1], p.tx_src[3 * i + 2], 0.0f);
+    if (p.counters)
+        for (int i = threadIdx.x; i < kNumCounters; i += blockDim.x) p.counters[i] = 0;
+}
+
 // The same rays at their places of the schedule, with their ids: the trace then reads a
 // refill's rays as they lie, where it used to map each place to an id and a 64-bit work index to
 // a transmitter by division (about 150 of the 560 instructions it spent on a segment besides its
@@ -71,7 +81,9 @@ __global__ void raygen_kernel(LatticeDev L, float4 *__restrict__ dirs, int N) {
 // (2.6 TB/s); with it the large city's trace 37.22 -> 36.19 ms, the canyon's 852 -> 822 us, and a
 // quarter range of the city's rays, in id order before, 16.27 -> 14.55 ms.
 __global__ void __launch_bounds__(256) raygen_schedule_kernel(LatticeDev L, float4 *__restrict__ dirs, int edge_blocks,
-                                                              int row_blocks) {
+                                                              int row_blocks, PrepArgs prep) {
+    wait_predecessor();
+    if (blockIdx.x == 0) prepare_launch(prep);
     const int n = L.n, E = 12 + 30 * (n - 1);
     if ((int)blockIdx.x < edge_blocks) {
         const int id = blockIdx.x * 256 + threadIdx.x;
@@ -108,11 +120,11 @@ __global__ void __launch_bounds__(256) raygen_schedule_kernel(LatticeDev L, floa
     }
 }
 
-cudaError_t launch_raygen_schedule(const LatticeDev &lat, float4 *dirs, cudaStream_t s) {
+cudaError_t launch_raygen_schedule(const LatticeDev &lat, float4 *dirs, const PrepArgs &prep, cudaStream_t s) {
     const int edge_blocks = (12 + 30 * (lat.n - 1) + 255) / 256;
     const int row_blocks = lat.n > 2 ? (lat.n - 2 + kTileRows - 1) / kTileRows : 0;
-    raygen_schedule_kernel<<<edge_blocks + 20 * row_blocks, 256, 0, s>>>(lat, dirs, edge_blocks, row_blocks);
-    return cudaGetLastError();
+    return launch_chained(raygen_schedule_kernel, edge_blocks + 20 * row_blocks, 256, 0, s, lat, dirs, edge_blocks, row_blocks,
+                          prep);
 }
 
 cudaError_t launch_raygen(const LatticeDev &lat, float4 *dirs, int64_t N, cudaStream_t s) {
@@ -130,7 +142,10 @@ cudaError_t launch_raygen(const LatticeDev &lat, float4 *dirs, int64_t N, cudaSt
 // interior rows before row i of a face: sum_{i'=1}^{i-1} (n - 1 - i')
 __device__ __forceinline__ long long row_prefix(int n, long long i) { return (i - 1) * (n - 1) - (i - 1) * i / 2; }
 
-__global__ void raygen_equidistant_kernel(PolyDev P, float4 *__restrict__ dirs, long long N, bool tagged) {
+__global__ void raygen_equidistant_kernel(PolyDev P, float4 *__restrict__ dirs, long long N, bool tagged,
+                                          PrepArgs prep) {
+    wait_predecessor();
+    if (blockIdx.x == 0) prepare_launch(prep);
     const int n = P.n;
     const long long n_edge = (long long)P.ne * (n - 1);
     const long long per_face = (long long)(n - 1) * (n - 2) / 2;
@@ -167,15 +182,15 @@ __global__ void raygen_equidistant_kernel(PolyDev P, float4 *__restrict__ dirs, 
     }
 }
 
-cudaError_t launch_raygen_equidistant(const PolyDev &P, float4 *dirs, int64_t N, bool tagged, cudaStream_t s) {
+cudaError_t launch_raygen_equidistant(const PolyDev &P, float4 *dirs, int64_t N, bool tagged, const PrepArgs &prep,
+                                      cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     long long want = (N + 255) / 256;
     int grid = (int)(want < (long long)sms * 16 ? want : (long long)sms * 16);
     if (grid < 1) grid = 1;
-    raygen_equidistant_kernel<<<grid, 256, 0, s>>>(P, dirs, (long long)N, tagged);
-    return cudaGetLastError();
+    return launch_chained(raygen_equidistant_kernel, grid, 256, 0, s, P, dirs, (long long)N, tagged, prep);
 }
 
 // ----------------------------------------------------------------------------- a2-a4
@@ -364,6 +379,7 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
 // Seven 128-thread blocks per SM (72 registers, no spills) measured faster than eight (64
 // registers, spilled).
 __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
+    wait_predecessor();
     extern __shared__ int faces_sh_all[];   // trace_smem(blockDim.x) bytes
     int *faces_sh = faces_sh_all + threadIdx.x;
     const int stride_sh = blockDim.x;
@@ -471,8 +487,7 @@ int trace_blocks_per_sm(int block) {
 }
 
 cudaError_t launch_trace(const TraceArgs &a, int grid, int block, cudaStream_t s) {
-    trace_kernel<<<grid, block, trace_smem(block), s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(trace_kernel, grid, block, trace_smem(block), s, a);
 }
 
 }  // namespace sbr

@@ -29,12 +29,12 @@ constexpr int kStack4 = 96;        // 4-wide traversal stack (the builder checks
 // Device counters of one launch (int64 each).
 enum Counter {
     kRays = 0, kSegments, kNodeVisits, kTriTests, kRxTests, kRecords, kPaths, kCollisions,
-    kRayHead, kBatchHead, kBatchDone, kErrorFlags, kWedgeTests, kDiffRecords, kDiffCand, kNonFinite,
+    kRayHead, kErrorFlags, kWedgeTests, kDiffRecords, kDiffCand, kNonFinite,
     kDiffPending,   // diffraction receptions parked at the top of the record array for diffract_occlusion
     kDiffBase,      // the record count before them (the trace's records)
     kDiffHead,      // groups of places the diffraction search has taken
     kDiffPairs,     // (wedge, 32 places) pairs its beams left for the exact test
-    kNumCounters = 20
+    kNumCounters = 18
 };
 
 // BVH node: both children's boxes in one 64-byte node (4 x float4).
@@ -163,6 +163,9 @@ struct sbr_ctx {
     size_t poly_bytes = 0;
     int poly_kind = 0;
     sbr::PolyDev poly{};
+    // resident blocks per SM, looked up once: trace kernel by block size / 32, batched refinement
+    // by lanes (1, 8, 16, 32) and block size / 32
+    int trace_nb[5] = {0}, refine_nb = 0, batch_nb[4][9] = {{0}};
     // kernel timing events (SBR_LAUNCH_TIMING)
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
 };
@@ -191,7 +194,9 @@ struct sbr_paths {
     float4 *unf = nullptr;                 // batched refinement: kUnfStride float4 per path
     int *order_idx = nullptr;              // batched refinement: path indices grouped by order
     unsigned long long *order_cnt = nullptr;   // [0, 10): paths per group; fill cursors: [16, 26) order_idx
-                                               // from the front, [48, 58) from the back, [32, 42) fp64_idx
+                                               // from the front, [48, 58) from the back, [32, 42) fp64_idx;
+                                               // 62: queue head, 63: blocks that have read them.  Zero
+                                               // between calls (the last kernel of a call clears them)
     int *fp64_idx = nullptr;               // batched refinement: paths handed to the FP64 tail
     unsigned long long *table = nullptr;   // dedup hash table: 2 x u64 per slot (key, value)
     int64_t table_slots = 0;
@@ -249,9 +254,17 @@ bool build_polyhedron(int poly, std::vector<float4> &v, std::vector<int2> &e, st
 // kernels (kernels_*.cu)
 cudaError_t launch_raygen(const LatticeDev &lat, float4 *dirs, int64_t N, cudaStream_t s);
 // the same directions in the schedule's order (lattice_order.cuh), each with its ray id's bits in w
-cudaError_t launch_raygen_schedule(const LatticeDev &lat, float4 *dirs, cudaStream_t s);
+// (prep: what a launch needs done before its trace, by the same kernel)
+struct PrepArgs {
+    const float *tx_src = nullptr;   // ntx x 3 transmitter positions on the device, or null
+    float4 *tx = nullptr;
+    int ntx = 0;
+    long long *counters = nullptr;   // zeroed, or null
+};
+cudaError_t launch_raygen_schedule(const LatticeDev &lat, float4 *dirs, const PrepArgs &prep, cudaStream_t s);
 // tagged: the ray id's bits in w
-cudaError_t launch_raygen_equidistant(const PolyDev &p, float4 *dirs, int64_t N, bool tagged, cudaStream_t s);
+cudaError_t launch_raygen_equidistant(const PolyDev &p, float4 *dirs, int64_t N, bool tagged, const PrepArgs &prep,
+                                      cudaStream_t s);
 
 struct TraceArgs {
     SceneDev scene;
