@@ -197,6 +197,14 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) 
     return SBR_OK;
 }
 
+// The first segments' frontier (frontier_kernel) pays from about two million rays: it takes 45 us
+// of latency whatever their number, and saves 20 us of a trace of 0.9M rays (street receivers,
+// 10k triangles), 105 of 4.9M, 5.1 ms of 194M (1.07M triangles); and on trees worth skipping (a
+// room of a dozen boxes has four levels).  Past 4 GB of lists (64 places a transmitter take 64
+// bytes: 4.3e9 first segments) the walks start at the root.
+constexpr int64_t kFrontMinRays = 3000000, kFrontMinNodes = 1024;
+constexpr size_t kFrontMaxBytes = (size_t)4 << 30;
+
 // a value looked up once (0: not yet)
 template <class F>
 int cached(int &slot, F look_up) {
@@ -319,6 +327,7 @@ sbr_status sbr_ctx_destroy(sbr_ctx *ctx) {
     dev_free(ctx, ctx->dirs, ctx->dirs_bytes);
     dev_free(ctx, ctx->lattice_mem, ctx->lattice_bytes);
     dev_free(ctx, ctx->poly_mem, ctx->poly_bytes);
+    dev_free(ctx, ctx->front, ctx->front_bytes);
     cudaStreamSynchronize(ctx->stream);
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
@@ -530,6 +539,7 @@ sbr_status sbr_scene_upload(sbr_ctx *ctx, const float *verts, int64_t nv, const 
     if (const char *lim = std::getenv("SBR_CHECKED_STACK_LIMIT"))
         sc->dev.stack_limit = std::max(1, std::min(kStack4, std::atoi(lim)));
 #endif
+    sc->max_stack4 = bvh.max_stack4;
     sc->wedges = std::move(wl);
     sc->info.num_wedges = nw;
     sc->info.num_triangles = nt;
@@ -819,13 +829,18 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     a.id_order_n = prm->launcher == 0 && (prm->flags & SBR_LAUNCH_ID_ORDER) ? prm->n_div : 0;
     a.first = ray_begin;
     a.count = ray_count;
-    if (prm->launcher == 0 && !a.id_order_n && ray_count > 0 && ray_count < N) {
+    int64_t place0 = ray_begin, places = ray_count;   // the places of dirs that hold the range's rays
+    if (prm->launcher == 0 && ray_count > 0 && ray_count < N) {
         // a range of ids on the schedule: whole faces, of which the ids outside the range are
         // passed over (the range cuts at most its first and last face)
         const int64_t E = 12 + 30LL * (prm->n_div - 1), per = (int64_t)(prm->n_div - 1) * (prm->n_div - 2) / 2;
-        if (ray_begin >= E) a.first = E + (ray_begin - E) / per * per;
+        if (ray_begin >= E) place0 = E + (ray_begin - E) / per * per;
         const int64_t last = a.ray_end - 1;
-        a.count = (last < E ? a.ray_end : E + ((last - E) / per + 1) * per) - a.first;
+        places = (last < E ? a.ray_end : E + ((last - E) / per + 1) * per) - place0;
+    }
+    if (!a.id_order_n) {
+        a.first = place0;
+        a.count = places;
     }
     a.inv_count = a.count > 0 ? 1.0f / (float)a.count : 0.0f;
     a.max_order = prm->max_order;
@@ -840,6 +855,35 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     a.dump_faces = prm->dump_faces;
     a.dump_per_tx = prm->dump_stride > 0 ? (N + prm->dump_stride - 1) / prm->dump_stride : 0;
     a.refill_min = prm->refill_min > 0 ? std::min(prm->refill_min, 32) : 24;
+    a.front = nullptr;
+    a.group0 = a.groups = 0;
+    if (scene->dev.nnodes >= kFrontMinNodes && ntx * places >= kFrontMinRays && places > 0 &&
+        scene->max_stack4 + kFrontEntries <= kStack4) {
+        const int64_t group0 = place0 / kFrontRays, groups = (place0 + places + kFrontRays - 1) / kFrontRays - group0;
+        const size_t need = (size_t)ntx * groups * kFrontEntries * sizeof(int2);
+        if (need <= kFrontMaxBytes && ctx->front_bytes < need) {
+            dev_free(ctx, ctx->front, ctx->front_bytes);
+            ctx->front = dev_alloc(ctx, need);
+            ctx->front_bytes = ctx->front ? need : 0;
+        }
+        if (ctx->front && need <= ctx->front_bytes) {
+            FrontArgs f;
+            f.scene = a.scene;
+            f.dirs = a.dirs;
+            f.tx = a.tx;
+            f.ntx = ntx;
+            f.first = place0;
+            f.count = places;
+            f.ray_begin = a.ray_begin;
+            f.ray_end = a.ray_end;
+            f.group0 = a.group0 = group0;
+            f.groups = a.groups = groups;
+            f.front = static_cast<int2 *>(ctx->front);
+            a.front = f.front;
+            Range r("sbr_launch: first segments' frontier");
+            SBR_CUDA(launch_frontier(f, ctx->stream));
+        }
+    }
     int block = prm->block_threads > 0 ? prm->block_threads : 128;
     if (block % 32 != 0 || block > 128)
         return fail(ctx, SBR_EINVAL, "sbr_launch: block_threads must be a multiple of 32, at most 128");

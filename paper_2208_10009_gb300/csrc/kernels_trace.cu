@@ -198,6 +198,7 @@ struct LaneRay {
     float3 o, d;
     float L;
     int k, prev, txi, ray;
+    int place;   // of the schedule
 };
 
 // Receptions a lane buffers during one segment before its warp flushes them.  Emitting
@@ -369,6 +370,156 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
     }
 }
 
+// ----------------------------------------------------------------------------- frontier
+// Interval of 1 / |d| over a beam's directions on one axis, the sign of d, and whether d changes
+// sign (then s = 0: only |centre - o| - half extent bounds the entry, and nothing the exit).
+struct BeamAxis {
+    float o, s, lo, hi;
+};
+
+__device__ __forceinline__ BeamAxis beam_axis(float o, float dl, float dh) {
+    BeamAxis b;
+    const float al = fminf(fabsf(dl), fabsf(dh)), ah = fmaxf(fabsf(dl), fabsf(dh));
+    const bool cross = !(dl * dh > 0.0f);
+    b.o = o;
+    b.s = cross ? 0.0f : (dl > 0.0f ? 1.0f : -1.0f);
+    b.lo = __fdividef(1.0f, ah) * 0.999999f;
+    b.hi = cross || al < 1e-30f ? INFINITY : __fdividef(1.0f, al) * 1.000001f;
+    return b;
+}
+
+// Bounds over the beam of where its rays enter (not before) and leave (not after) a slab.
+__device__ __forceinline__ void beam_slab(const BeamAxis &b, float c, float h, float &tn, float &tf) {
+    const float x = c - b.o, p = b.s == 0.0f ? fabsf(x) : x * b.s;
+    const float np = p - h, fp = p + h;
+    tn = fmaxf(tn, fminf(np * b.lo, np * b.hi));
+    tf = fminf(tf, fmaxf(fp * b.lo, fp * b.hi));
+}
+
+// The frontier of the first segments: a group's rays leave Tx within a degree or less of each
+// other and would each walk the same upper tree; one thread walks it for all of them with the
+// interval of their directions, always opening the nearest inner node, until the list is full or
+// kFrontOpen nodes were opened.
+// A ray then starts among a few nodes and leaves next to what it hits, and a group that looks
+// into the sky has an empty list.  (First segments are 43 % of the large city's segments and a
+// third of its node visits.)  Groups of 32 / 64 / 128 places cost the trace the same (29.4-29.5 ms on
+// the city) and themselves 1,050 / 617 / 548 us there, 67 / 51 / 100 us on the canyon, where one
+// thread's chain of openings is what it waits for; 6 / 8 / 12 entries: 29.9 / 29.4 / 29.4 ms.
+// Large city trace 34.6 -> 29.5 ms + 0.62, canyon 820 -> 714 us + 51.
+__global__ void __launch_bounds__(128) frontier_kernel(FrontArgs A) {
+    wait_predecessor();
+    const int lane = threadIdx.x & 31;
+    const long long g0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    if (g0 >= A.groups) return;
+    // directions' intervals: the warp reads group by group, lane g keeps group g's.  d + 2 is positive,
+    // so its bits order like it; its rounding (2^-22) is given back below.
+    float lo[3] = {1.0f, 1.0f, 1.0f}, hi[3] = {-1.0f, -1.0f, -1.0f};
+    bool some = false;
+#pragma unroll 4
+    for (int g = 0; g < 32; ++g) {
+        unsigned mn[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, mx[3] = {0, 0, 0}, any = 0;
+#pragma unroll
+        for (int q = 0; q < kFrontRays; q += 32) {
+            const long long place = (A.group0 + g0 + g) * kFrontRays + q + lane;
+            if (g0 + g >= A.groups || place < A.first || place >= A.first + A.count) continue;
+            const float4 dd = __ldg(A.dirs + place);
+            const int ray = __float_as_int(dd.w);
+            if (ray < A.ray_begin || ray >= A.ray_end) continue;
+            const float v[3] = {dd.x, dd.y, dd.z};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const unsigned u = __float_as_uint(v[k] + 2.0f);
+                mn[k] = min(mn[k], u);
+                mx[k] = max(mx[k], u);
+            }
+            any = 1;
+        }
+        any = __any_sync(0xffffffffu, any);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            mn[k] = __reduce_min_sync(0xffffffffu, mn[k]);
+            mx[k] = __reduce_max_sync(0xffffffffu, mx[k]);
+            if (lane == g) {
+                lo[k] = __uint_as_float(mn[k]) - 2.0f - 1e-6f;
+                hi[k] = __uint_as_float(mx[k]) - 2.0f + 1e-6f;
+            }
+        }
+        if (lane == g) some = any;
+    }
+    if (g0 + lane >= A.groups) return;
+    for (int t = 0; t < A.ntx; ++t) {
+        // the list stays in registers: every loop over it is unrolled.  Past its n entries dist = +inf.
+        int ref[kFrontEntries];
+        float dist[kFrontEntries];
+#pragma unroll
+        for (int j = 0; j < kFrontEntries; ++j) {
+            ref[j] = kNoRef;
+            dist[j] = INFINITY;
+        }
+        int n = 0;
+        if (some) {
+            const float3 o = f3(__ldg(A.tx + t));
+            const BeamAxis bx = beam_axis(o.x, lo[0], hi[0]), by = beam_axis(o.y, lo[1], hi[1]), bz = beam_axis(o.z, lo[2], hi[2]);
+            ref[0] = 0;
+            dist[0] = 0.0f;
+            n = 1;
+            // the nearest inner node is opened while its four children fit
+            for (int opened = 0; n <= kFrontEntries - 3 && opened < kFrontOpen; ++opened) {
+                int node = -1;
+                bool gone = false;
+#pragma unroll
+                for (int j = 0; j < kFrontEntries; ++j) {   // found: taken out, the entries after it move up
+                    if (!gone && ref[j] != kNoRef && !is_leaf(ref[j])) {
+                        node = ref[j];
+                        gone = true;
+                    }
+                    if (gone) {
+                        ref[j] = j + 1 < kFrontEntries ? ref[j + 1 < kFrontEntries ? j + 1 : j] : kNoRef;
+                        dist[j] = j + 1 < kFrontEntries ? dist[j + 1 < kFrontEntries ? j + 1 : j] : INFINITY;
+                    }
+                }
+                if (node < 0) break;
+                --n;
+                const Node4 v = load_node4(A.scene.nodes4 + 8 * (size_t)node);
+                const float cx[4] = {v.x.c01.x, v.x.c01.y, v.x.c23.x, v.x.c23.y}, hx[4] = {v.x.h01.x, v.x.h01.y, v.x.h23.x, v.x.h23.y};
+                const float cy[4] = {v.y.c01.x, v.y.c01.y, v.y.c23.x, v.y.c23.y}, hy[4] = {v.y.h01.x, v.y.h01.y, v.y.h23.x, v.y.h23.y};
+                const float cz[4] = {v.z.c01.x, v.z.c01.y, v.z.c23.x, v.z.c23.y}, hz[4] = {v.z.h01.x, v.z.h01.y, v.z.h23.x, v.z.h23.y};
+                const int rf[4] = {v.refs.x, v.refs.y, v.refs.z, v.refs.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float tn = 0.0f, tf = INFINITY;
+                    beam_slab(bx, cx[c], hx[c], tn, tf);
+                    beam_slab(by, cy[c], hy[c], tn, tf);
+                    beam_slab(bz, cz[c], hz[c], tn, tf);
+                    if (!(tn <= tf * 1.000001f) || rf[c] == leaf_ref(0, 0)) continue;
+                    ++n;
+                    // behind the entries at most as far
+#pragma unroll
+                    for (int j = kFrontEntries - 1; j >= 0; --j) {
+                        const bool before = j > 0 && dist[j > 0 ? j - 1 : 0] > tn;   // the one before moves here
+                        const bool here = !before && dist[j] > tn;
+                        if (before) {
+                            ref[j] = ref[j > 0 ? j - 1 : 0];
+                            dist[j] = dist[j > 0 ? j - 1 : 0];
+                        } else if (here) {
+                            ref[j] = rf[c];
+                            dist[j] = tn;
+                        }
+                    }
+                }
+            }
+        }
+        int4 *out = reinterpret_cast<int4 *>(A.front + ((size_t)t * A.groups + g0 + lane) * kFrontEntries);
+#pragma unroll
+        for (int j = 0; j < kFrontEntries; j += 2)
+            out[j / 2] = make_int4(ref[j], __float_as_int(dist[j]), ref[j + 1], __float_as_int(dist[j + 1]));
+    }
+}
+
+cudaError_t launch_frontier(const FrontArgs &a, cudaStream_t s) {
+    return launch_chained(frontier_kernel, (unsigned)((a.groups + 127) / 128), 128, 0, s, a);
+}
+
 // Persistent trace kernel.  Each warp keeps 32 rays in registers; after a segment, once at
 // least refill_min lanes hold a finished ray (miss or order cap), those lanes take fresh,
 // consecutive places of the schedule from a global counter with
@@ -398,7 +549,7 @@ __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
     LaneRay st;
     st.o = st.d = make_float3(0, 0, 0);
     st.L = 0.0f;
-    st.k = st.prev = st.txi = st.ray = 0;
+    st.k = st.prev = st.txi = st.ray = st.place = 0;
     for (;;) {
         unsigned need = __ballot_sync(0xffffffffu, !alive);
         if (need && !pool_empty && (__popc(need) >= a.refill_min || need == 0xffffffffu)) {
@@ -421,6 +572,7 @@ __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
                     st.o = f3(__ldg(a.tx + st.txi));
                     st.d = f3(dd);
                     st.ray = __float_as_int(dd.w);
+                    st.place = place;
                     st.L = 0.0f;
                     st.k = 0;
                     st.prev = -1;
@@ -439,9 +591,14 @@ __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
         }
         if (alive) {
             RayPre r = make_ray(st.o, st.d);
+            const int4 *first = nullptr;
+            if (a.front && st.k == 0)
+                first = reinterpret_cast<const int4 *>(
+                    a.front + ((size_t)st.txi * a.groups + (st.place / kFrontRays - a.group0)) * kFrontEntries);
             float th;
             int face;
-            const int hit = closest_hit4(a.scene, r, a.scene.tmin, INFINITY, st.prev, th, face, nodes, tris);
+            const int hit = closest_hit4(a.scene, r, a.scene.tmin, INFINITY, st.prev,
+                                         first, th, face, nodes, tris);
             ++seg;
             if (a.dump_stride > 0 && st.ray % a.dump_stride == 0)
                 a.dump_faces[((size_t)st.txi * a.dump_per_tx + st.ray / a.dump_stride) * (a.max_order + 1) + st.k] =

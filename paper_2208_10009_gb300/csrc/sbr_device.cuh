@@ -230,14 +230,28 @@ __device__ __forceinline__ bool pop_near(const int *stack, const float *sdist, i
 // shrunk range, so nothing it holds can win).  Closest hit along o + t d over t in (tmin, tmax],
 // skipping triangles of face `skip`; ties in t go to the lower face id, then the lower
 // triangle index.  Returns the triangle index (BVH order) or -1; t_out, face_out set on a
-// hit.  nodes_visited counts 4-wide nodes (four box tests each).
+// hit.  `front`: the entries to start from (FrontArgs) or null.  nodes_visited counts 4-wide nodes (four box tests each).
 __device__ __forceinline__ int closest_hit4(const SceneDev &S, const RayPre &r, float tmin, float tmax, int skip,
-                                            float &t_out, int &face_out, unsigned &nodes_visited,
+                                            const int4 *front, float &t_out, int &face_out, unsigned &nodes_visited,
                                             unsigned &tris_tested) {
     int stack[kStack4];    // node or leaf refs
     float sdist[kStack4];  // their entry distances
     int sp = 0;
     int node = 0;
+    if (front) {   // start from a frontier (nearest entry first) instead of the root
+        t_out = tmax;
+        face_out = 0x7fffffff;
+        int4 e[kFrontEntries / 2];
+#pragma unroll
+        for (int j = 0; j < kFrontEntries / 2; ++j) e[j] = __ldg(front + j);
+        if (e[0].x == kNoRef) return -1;
+#pragma unroll
+        for (int j = kFrontEntries / 2 - 1; j >= 0; --j) {
+            if (e[j].z != kNoRef) { stack[sp] = e[j].z; sdist[sp++] = __int_as_float(e[j].w); }
+            if (j > 0 && e[j].x != kNoRef) { stack[sp] = e[j].x; sdist[sp++] = __int_as_float(e[j].y); }
+        }
+        node = e[0].x;
+    }
     float tbest = tmax;
     float tcull = tmax * 1.0000005f;   // entries entering beyond this are dropped at pop
     int best = -1, bface = 0x7fffffff;

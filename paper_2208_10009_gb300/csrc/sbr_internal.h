@@ -152,6 +152,9 @@ struct sbr_ctx {
     size_t dirs_bytes = 0;
     int dirs_n = 0;
     bool dirs_valid = false;
+    // first segments' frontier
+    void *front = nullptr;
+    size_t front_bytes = 0;
     // lattice tables
     void *lattice_mem = nullptr;
     size_t lattice_bytes = 0;
@@ -175,6 +178,7 @@ struct sbr_scene {
     size_t bytes = 0;
     sbr::SceneDev dev{};
     sbr_scene_info info{};
+    int max_stack4 = 0;        // worst-case stack use of a 4-wide walk from the root
     std::vector<sbr::WedgeHost> wedges;   // host copy (sbr_scene_wedges)
 };
 
@@ -266,6 +270,22 @@ cudaError_t launch_raygen_schedule(const LatticeDev &lat, float4 *dirs, const Pr
 cudaError_t launch_raygen_equidistant(const PolyDev &p, float4 *dirs, int64_t N, bool tagged, const PrepArgs &prep,
                                       cudaStream_t s);
 
+// The first segments' frontier: per transmitter and group of kFrontRays consecutive places, up to
+// kFrontEntries (node or leaf ref, entry distance bits), nearest first, that together hold
+// everything the group's rays can meet; kNoRef past the last one.
+constexpr int kFrontRays = 64, kFrontEntries = 8, kFrontOpen = 16, kNoRef = 0x7fffffff;
+struct FrontArgs {
+    SceneDev scene;
+    const float4 *dirs;
+    const float4 *tx;
+    int ntx;
+    int64_t first, count;     // places, as in TraceArgs
+    int ray_begin, ray_end;
+    int64_t group0, groups;   // groups of places group0 .. group0 + groups hold them
+    int2 *front;              // [ntx][groups][kFrontEntries]
+};
+cudaError_t launch_frontier(const FrontArgs &a, cudaStream_t s);
+
 struct TraceArgs {
     SceneDev scene;
     RxDev rx;
@@ -276,6 +296,8 @@ struct TraceArgs {
     int ray_begin, ray_end;   // the ray ids in [ray_begin, ray_end) are traced
     float inv_count;          // 1 / count (transmitter of a work index, then fixed)
     int id_order_n;           // > 0: ray ids in turn (a place is an id) on the schedule of this n
+    const int2 *front;        // first segments' frontier (FrontArgs), or null: they start at the root
+    int64_t group0, groups;
     int max_order;
     float cone;               // reception cone half-angle (rad)
     float tan_cone;
