@@ -477,7 +477,10 @@ def run_gpu(args):
                                         "MEASURED_PEAKS.json)"),
                         "derived_peak": derived_tflops, "flops_per_launch": flops, "trace_ms": st_t["ms_trace"],
                         "issue_active": issue, "issue_source": None if issue is None else issue_rec.get("capture")},
-           "clocks": clocks, "gpu_launches": _launches_per_step(opts, world) * args.steps,
+           "clocks": clocks, "gpu_launches": _launches_per_step(
+               {"diffraction": opts["diffraction"],
+                "frontier": st_t["rays"] >= 3_000_000 and scene.info()["bvh_nodes"] >= 1024}, world,
+               shape["lanes_per_path"] == 1 or paths.path_cap >= 16 * 32 * sms) * args.steps,
            "wall_s": t_wall, "e2e": e2e}
     if rank == 0 and not args.no_cpu_baseline:
         acc = oracle_accuracy(sc, tx, rx, recs) if world == 1 else None
@@ -504,11 +507,14 @@ def run_gpu(args):
         dist.destroy_process_group()
 
 
-def _launches_per_step(opts, world):
-    """Library kernels per step: raygen, trace (+5 diffraction: candidates, exact tests,
-    visibility, receivers, occlusion), 3 dedup, 4 batched refinement; shards add the
-    record-count reset kernel."""
-    return 9 + (5 if opts["diffraction"] else 0) + (1 if world > 1 else 0)
+def _launches_per_step(opts, world, many):
+    """Library kernels per step: raygen, trace, 3 double-count removal and the batched
+    refinement's 3 (iterations, FP64 tail, validity + outputs), plus its 2 for many paths (plane
+    unfolding, bounce-point walk), the first segments' frontier (launches of 3M rays and more on
+    trees of 1,024 nodes), 5 diffraction (candidates, exact tests, visibility, receivers,
+    occlusion); shards add the record-count reset kernel."""
+    return 8 + (2 if many else 0) + (1 if opts["frontier"] else 0) + (5 if opts["diffraction"] else 0) + \
+        (1 if world > 1 else 0)
 
 
 def _refine_forms(ctx, scene, paths, relaunch, stream, iters, K, target, shape, ntx, nrx, trials=3):

@@ -707,7 +707,7 @@ sbr_status sbr_paths_create(sbr_ctx *ctx, int64_t record_cap, int64_t path_cap, 
     cv.add(&p->paths, (size_t)path_cap);
     cv.add(&p->unf, (size_t)path_cap * kUnfStride);
     cv.add(&p->order_idx, (size_t)path_cap);
-    cv.add(&p->order_cnt, (size_t)64);
+    cv.add(&p->order_cnt, (size_t)kOrderCounts);
     cv.add(&p->fp64_idx, (size_t)path_cap);
     cv.add(&table, (size_t)slots * 2 + (size_t)(slots + 1) / 2);   // (key, value) slots, winner ids
     cv.add(&p->counters, (size_t)kNumCounters);
@@ -723,7 +723,7 @@ sbr_status sbr_paths_create(sbr_ctx *ctx, int64_t record_cap, int64_t path_cap, 
     p->record_cap = record_cap;
     p->path_cap = path_cap;
     SBR_CUDA(cudaMemsetAsync(p->counters, 0, kNumCounters * sizeof(long long), ctx->stream));
-    SBR_CUDA(cudaMemsetAsync(p->order_cnt, 0, 64 * sizeof(unsigned long long), ctx->stream));
+    SBR_CUDA(cudaMemsetAsync(p->order_cnt, 0, kOrderCounts * sizeof(unsigned long long), ctx->stream));
     *out = p;
     return SBR_OK;
 }

@@ -775,13 +775,12 @@ __device__ __forceinline__ double converged_bound(int iters, double R_final) {
     return iters > 0 ? 2.0 * R_final + 1e-7 : INFINITY;
 }
 
-// a7/a8 for a diffraction path: the diffraction point Q is the point of the edge line
+// a7/a8 for a diffraction path but for its occlusion queries: the diffraction point Q is the point of the edge line
 // closest to the launched ray; valid iff Q lies on the edge segment and ahead of Tx, Tx and
 // Rx lie in the wedge's exterior, the refinement converged, and Tx -> Q and Q -> Rx are
 // unblocked (the wedge's faces excluded).  delay = (|Q - Tx| + |Rx - Q|) / c0, AOD = c,
 // AOA = Q - Rx, power = ptx + free-space loss (no diffraction coefficient).
-__device__ void wedge_finalize(const RefineArgs &A, const PathGeo &g, dvec3 c, sbr_path_record &p,
-                               double err_bound) {
+__device__ bool wedge_walk(const RefineArgs &A, const PathGeo &g, dvec3 c, sbr_path_record &p, double err_bound, dvec3 &Q) {
     const SceneDev &S = A.scene;
     const WedgeD w = wedge64(S, g.wedge);
     const dvec3 eb = w.b - w.a, w0 = g.txd - w.a;
@@ -789,24 +788,39 @@ __device__ void wedge_finalize(const RefineArgs &A, const PathGeo &g, dvec3 c, s
     const double den = Ac * C - B * B;
     const double u = den != 0.0 ? (Ac * E - B * D) / den : -1.0;
     const double sq = den != 0.0 ? (B * E - C * D) / den : -1.0;
-    const dvec3 Q = w.a + eb * u;
+    Q = w.a + eb * u;
     const dvec3 e = eb * (1.0 / sqrt(C));
-    bool valid = u >= 0.0 && u <= 1.0 && sq > 0.0 && exterior64(w, e, g.txd) && exterior64(w, e, g.rxd) &&
+    const bool valid = u >= 0.0 && u <= 1.0 && sq > 0.0 && exterior64(w, e, g.txd) && exterior64(w, e, g.rxd) &&
                  p.err <= err_bound;
-    for (int j = 0; j < 2 && valid; ++j) {
-        dvec3 from = j == 0 ? g.txd : Q, seg = (j == 0 ? Q : g.rxd) - from;
-        RayPre r = make_ray(make_float3((float)from.x, (float)from.y, (float)from.z),
-                            make_float3((float)seg.x, (float)seg.y, (float)seg.z));
-        if (any_hit4(S, r, 1e-6f, 1.0f - 1e-6f, w.f1, w.f2)) valid = false;
-    }
     const double len = dnorm(Q - g.txd) + dnorm(g.rxd - Q);
-    p.valid = valid ? 1 : 0;
     p.delay = len / kC0;
     az_el(c, p.aod);
     az_el(Q - g.rxd, p.aoa);
     const float lam = (float)(kC0 / A.freq);
     p.power_dbm = (float)A.ptx_dbm + 20.0f * log10f(lam / (4.0f * 3.14159265f * (float)len));
     p.flags |= SBR_PATH_DIFFRACTED;
+    return valid;
+}
+
+// leg j (0: Tx -> Q, 1: Q -> Rx) of a diffraction path: origin and extent in FP32
+__device__ __forceinline__ void wedge_leg(const PathGeo &g, dvec3 Q, int j, float3 &from, float3 &seg) {
+    const dvec3 f = j == 0 ? g.txd : Q, d = (j == 0 ? Q : g.rxd) - f;
+    from = make_float3((float)f.x, (float)f.y, (float)f.z);
+    seg = make_float3((float)d.x, (float)d.y, (float)d.z);
+}
+
+__device__ void wedge_finalize(const RefineArgs &A, const PathGeo &g, dvec3 c, sbr_path_record &p, double err_bound) {
+    dvec3 Q;
+    bool valid = wedge_walk(A, g, c, p, err_bound, Q);
+    if (valid) {
+        const WedgeD w = wedge64(A.scene, g.wedge);
+        for (int j = 0; j < 2 && valid; ++j) {
+            float3 from, seg;
+            wedge_leg(g, Q, j, from, seg);
+            if (any_hit4(A.scene, make_ray(from, seg), 1e-6f, 1.0f - 1e-6f, w.f1, w.f2)) valid = false;
+        }
+    }
+    p.valid = valid ? 1 : 0;
 }
 
 // Validity test and outputs for launch direction c; writes the result fields of p.
@@ -857,6 +871,50 @@ __device__ void finalize_path(const RefineArgs &A, const PathGeo &g, dvec3 c, sb
         if (any_hit4(S, r, 1e-6f, 1.0f - 1e-6f, fa, fb)) valid = false;
     }
     p.valid = valid ? 1 : 0;
+}
+
+// The same without the occlusion queries, in one walk: the legs of a path that passes so far go to
+// `legs` (6 floats each: origin, extent) for batch_occlusion_kernel; false: invalid.
+__device__ __forceinline__ bool finalize_walk(const RefineArgs &A, const PathGeo &g, dvec3 c, sbr_path_record &p,
+                                              double err_bound, float2 *legs) {
+    auto put = [&](int j, float3 from, float3 seg) {
+        legs[3 * j] = make_float2(from.x, from.y);
+        legs[3 * j + 1] = make_float2(from.z, seg.x);
+        legs[3 * j + 2] = make_float2(seg.y, seg.z);
+    };
+    if (g.wedge >= 0) {
+        dvec3 Q;
+        if (!wedge_walk(A, g, c, p, err_bound, Q)) return false;
+        for (int j = 0; j < 2; ++j) {
+            float3 from, seg;
+            wedge_leg(g, Q, j, from, seg);
+            put(j, from, seg);
+        }
+        return true;
+    }
+    const SceneDev &S = A.scene;
+    bool inside = p.err <= err_bound;
+    BounceWalk w;
+    w.start(g, c);
+    float gain_db = 0.0f;
+    for (int j = 0; j < g.k; ++j) {
+        const df3 from = w.o;
+        const int f = g.faces[j];
+        df den;
+        if (!w.step(S, f, den)) {
+            p.flags |= SBR_PATH_TRACE_FAIL;
+            p.delay = 0.0;
+            return false;
+        }
+        const float eps = __ldg(S.face_eps + f);
+        if (eps > 0.0f) gain_db += 20.0f * log10f(fresnel_perp_abs(fabsf(df_round(den)), eps));
+        inside = inside && point_in_face(S, f, w.o);
+        if (inside) put(j, df3_round(from), df3_round(df3_sub(w.o, from)));
+    }
+    inside = inside && rx_ahead(g, w.o, w.d);
+    if (inside) put(g.k, df3_round(w.o), df3_round(df3_sub(df3_of(g.rx), w.o)));
+    path_outputs(A, g, c, w.o, w.tsum, gain_db, p);
+    return inside;
 }
 
 __device__ __forceinline__ void store_result(sbr_path_record *dst, const sbr_path_record &p) {
@@ -1158,7 +1216,7 @@ __global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
     }
 }
 
-// Lists path pi in its order group for batch_finalize_kernel (group offsets from
+// Lists path pi in its order group for batch_walk_kernel (group offsets from
 // batch_unfold_kernel's counts), so that a warp there holds paths of one order.  Inside the
 // group, paths whose error meets the convergence bound 2 R + 1e-7 (the validity test's
 // condition; R is the cone radius after the iterations, here only an ordering hint) fill it
@@ -1181,13 +1239,14 @@ __device__ __forceinline__ void list_for_finalize(const RefineArgs &A, const Pat
 // stalled, or all sub-rays invalid) the group takes the next path index from the device
 // queue head with one atomic, so paths that stop early free their group at once.  With
 // many paths, a path whose cone falls below the FP64 threshold moves on to
-// batch_refine64_kernel; the validity test and outputs follow in batch_finalize_kernel.
+// batch_refine64_kernel; the validity test and outputs follow in batch_walk_kernel and
+// batch_occlusion_kernel.
 // At most 85 registers a thread, so that three 256-thread blocks fit on an SM (measured
 // faster than the uncapped 124-128 registers of the 8- and 32-lane forms).
 // G = 1 is the one-lane form: each thread evaluates all K sub-rays of its own path (no
 // shuffles, no re-evaluation of the winner) and always runs with batch_unfold_kernel and
 // the FP64 tail kernel (the host sets split_min = 0 for it).
-constexpr int kQueueHead = 62, kBlocksRead = 63, kOrderCounts = 64;   // of order_cnt
+constexpr int kQueueHead = 62, kBlocksRead = 63, kLegCounts = 64;   // of order_cnt
 template <int G>
 __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
     wait_predecessor();
@@ -1271,7 +1330,8 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
         x.dw = 0.0;
         put_iterated(x, dv(x.cf.x, x.cf.y, x.cf.z), p);
         if (prebuilt) list_for_finalize(A, g, pi, p.err, (double)x.Rf);
-        // iteration results; the validity test and outputs follow in batch_finalize_kernel
+        // iteration results; the validity test and outputs follow in batch_walk_kernel and
+// batch_occlusion_kernel
         dst->iters = p.iters;
         dst->dir[0] = p.dir[0];
         dst->dir[1] = p.dir[1];
@@ -1286,7 +1346,7 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
 // each instruction of GB300's narrow FP64 pipe serves 32 paths, where a lane group would serve
 // one.  The state carried over: a path that started in FP64 (no iteration done) takes its FP64
 // rough direction; otherwise the FP32 phase's centre with its |d x W|^2 and d . W.  With many
-// paths the path is then listed in its order group for batch_finalize_kernel.  One warp a
+// paths the path is then listed in its order group for batch_walk_kernel.  One warp a
 // block: the FP64 pipe belongs to the SM, so a short list (the large city's 17k paths are 535
 // warps) has to spread over as many SMs as it has warps.  A list of at most kTailWide paths an
 // SM takes a warp a path instead: its lanes unfold the planes side by side and then iterate
@@ -1389,54 +1449,114 @@ __global__ void __launch_bounds__(128) batch_unfold_kernel(RefineArgs A) {
     if (threadIdx.x < 10 && hist[threadIdx.x]) atomicAdd(A.order_cnt + threadIdx.x, (unsigned long long)hist[threadIdx.x]);
 }
 
-// a7/a8 of the batched form.  With many paths (>= split_min), one thread per path: every
-// lane of a warp runs the same validity test and bounce-point walk on its own path, the
-// paths taken in the lists the iteration kernels grouped by order.  With few paths, one
-// warp per path with the point-in-face and occlusion queries spread over its lanes
-// (latency).  The cone radius after `iters` iterations is recomputed with the same
-// multiplications.  The queries are latency-bound: eight blocks per SM (64 registers,
-// some spilled to L1) measured faster than four, five or six with fewer spills, and
-// faster than the occlusion queries split into a kernel of their own with a thread per
-// (path, leg) (which walks each path again for every leg).
-__global__ void __launch_bounds__(128, 8) batch_finalize_kernel(RefineArgs A) {
+// a7/a8 of the batched form, in two kernels.  With many paths (>= split_min), batch_walk_kernel walks
+// each path's bounce points, a thread per path in the order groups' lists, computes its outputs and
+// tests the points on their faces; the legs of the paths that pass go to their unf slots and the
+// paths to a list per order group.  batch_occlusion_kernel then runs the occlusion queries, a
+// thread per (path, leg), leg by leg over a group (neighbours in the list start near each other and
+// run alike), and marks the paths with a blocked leg.  One kernel with both, a thread per path, kept
+// 14.5 of 32 lanes (a path's later legs wait for its neighbours' and blocked paths idle), spilled
+// at 64 registers and walked twice, its L1 data pipe 80 % busy.  Office (942,656 paths, 448k valid):
+// 1,530 us -> 232 + 1,090, and 938 with 32-byte node loads (the L1 data pipe still bounds the
+// queries); the large city's 17.7k paths 290 -> 50 + 78 us.  Resident blocks: walk 4 / 6 / 8 an SM
+// 254 / 232 / 264 us, queries 6 / 8 / 10 1,112 / 1,097 / 1,237 us.
+// With few paths, one warp per path does both in the second kernel (latency), its lanes taking
+// the points and legs.  The cone radius after `iters` iterations is recomputed with the same
+// multiplications.
+__global__ void __launch_bounds__(128, 6) batch_walk_kernel(RefineArgs A) {
+    wait_predecessor();
+    if (path_count(A) < A.split_min) return;
+    const double shrink = c_sub.shrink[A.K];
+    long long listed = 0;   // paths with valid ids, listed by order group by the iteration kernels
+    for (int b = 0; b < 10; ++b) listed += A.order_cnt[b];
+    const int lane = threadIdx.x & 31;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < listed; t += (long long)gridDim.x * blockDim.x) {
+        const long long pi = (long long)A.order_idx[t];
+        sbr_path_record p = A.paths[pi];
+        PathGeo g;
+        load_path(A, p, g);
+        const double R = cone_radius64(A, p.rough_err, p.iters, shrink);
+        const dvec3 c = dv(p.dir[0], p.dir[1], p.dir[2]);
+        float2 *legs = reinterpret_cast<float2 *>(A.unf + kUnfStride * pi);
+        const bool valid = finalize_walk(A, g, c, p, converged_bound(p.iters, R), legs);
+        p.valid = valid ? 1 : 0;
+        store_result(A.paths + pi, p);
+        if (!valid) continue;
+        // onto its group's list: one atomic for the lanes of a group that arrive together
+        const int grp = order_group(g);
+        const unsigned m = __match_any_sync(__activemask(), grp);
+        const int leader = __ffs(m) - 1;
+        unsigned long long at = 0;
+        if (lane == leader) at = atomicAdd(A.order_cnt + kLegCounts + grp, (unsigned long long)__popc(m));
+        at = __shfl_sync(m, at, leader) + __popc(m & ((1u << lane) - 1u));
+        for (int b = 0; b < grp; ++b) at += A.order_cnt[b];
+        A.fp64_idx[at] = (int)pi;   // the FP64 tail is done with the list
+    }
+}
+
+__global__ void __launch_bounds__(128, 8) batch_occlusion_kernel(RefineArgs A) {
     wait_predecessor();
     const long long total = path_count(A);
-    const double shrink = c_sub.shrink[A.K];
-    const bool per_thread = total >= A.split_min;
-    const long long stride = per_thread ? (long long)gridDim.x * blockDim.x : (long long)gridDim.x * (blockDim.x >> 5);
-    const long long first = per_thread ? blockIdx.x * (long long)blockDim.x + threadIdx.x
-                                       : blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    long long listed = total;
-    if (per_thread) {   // paths with valid ids, listed by order group by the iteration kernel
-        listed = 0;
-        for (int b = 0; b < 10; ++b) listed += A.order_cnt[b];
+    const bool many = total >= A.split_min;
+    const int lane = threadIdx.x & 31;
+    __shared__ unsigned long long s_size[10], s_have[10];   // group sizes; paths with legs to test
+    __shared__ bool s_last;
+    if (threadIdx.x < 10) {
+        s_size[threadIdx.x] = A.order_cnt[threadIdx.x];
+        s_have[threadIdx.x] = A.order_cnt[kLegCounts + threadIdx.x];
     }
+    __syncthreads();
     // nothing reads the queue head, group sizes and cursors after this: the last block to get here
     // leaves them zero for the next call
-    __shared__ bool s_last;
-    __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         s_last = atomicAdd(A.order_cnt + kBlocksRead, 1ULL) == gridDim.x - 1ULL;
     }
     __syncthreads();
     if (s_last && threadIdx.x < kOrderCounts) A.order_cnt[threadIdx.x] = 0;
-    for (long long t = first; t < listed; t += stride) {
-        const long long pi = per_thread ? (long long)A.order_idx[t] : t;
+    if (many) {
+        const long long stride = (long long)gridDim.x * blockDim.x;
+        long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, base = 0;
+        unsigned long long off = 0;
+        for (int b = 0; b < 10; ++b) {
+            const unsigned have = (unsigned)s_have[b];
+            const long long queries = (long long)have * (b < 9 ? b + 1 : 2);
+            for (; t < base + queries; t += stride) {
+                const unsigned long long r = (unsigned long long)(t - base);
+                const int leg = (int)((r >> 32) == 0 ? (unsigned)r / have : r / have);
+                const long long pi = A.fp64_idx[off + (r - (unsigned long long)leg * have)];
+                sbr_path_record *p = A.paths + pi;
+                if (!p->valid) continue;   // another leg is blocked
+                const float2 *l = reinterpret_cast<const float2 *>(A.unf + kUnfStride * pi) + 3 * leg;
+                const float2 l0 = l[0], l1 = l[1], l2 = l[2];
+                int fa, fb;
+                if (b == 9) {
+                    const float4 *wp = A.scene.wedges + 4 * (size_t)(-1 - p->faces[0]);
+                    fa = __float_as_int(__ldg(wp).w);
+                    fb = __float_as_int(__ldg(wp + 1).w);
+                } else {
+                    fa = leg == 0 ? -1 : p->faces[leg - 1];
+                    fb = leg == b ? -1 : p->faces[leg];
+                }
+                if (any_hit4(A.scene, make_ray(make_float3(l0.x, l0.y, l1.x), make_float3(l1.y, l2.x, l2.y)), 1e-6f,
+                             1.0f - 1e-6f, fa, fb))
+                    p->valid = 0;
+            }
+            base += queries;
+            off += s_size[b];
+        }
+        return;
+    }
+    const double shrink = c_sub.shrink[A.K];
+    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+    for (long long pi = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); pi < total; pi += warps) {
         sbr_path_record p = A.paths[pi];
         if (!path_ids_ok(A, p)) continue;   // already flagged by the iteration kernel
         PathGeo g;
         load_path(A, p, g);
         const double R = cone_radius64(A, p.rough_err, p.iters, shrink);
-        dvec3 c = dv(p.dir[0], p.dir[1], p.dir[2]);
-        if (per_thread) {
-            finalize_path(A, g, c, p, converged_bound(p.iters, R));
-            store_result(A.paths + pi, p);
-        } else {
-            const int lane = threadIdx.x & 31;
-            group_finalize<32>(A, g, c, p, lane, 0xffffffffu, converged_bound(p.iters, R));
-            if (lane == 0) store_result(A.paths + pi, p);
-        }
+        group_finalize<32>(A, g, dv(p.dir[0], p.dir[1], p.dir[2]), p, lane, 0xffffffffu, converged_bound(p.iters, R));
+        if (lane == 0) store_result(A.paths + pi, p);
     }
 }
 
@@ -1476,10 +1596,14 @@ static int resident(K kernel, int block) {
 cudaError_t launch_batch_refine(const RefineArgs &a, int grid, int block, cudaStream_t s) {
     static const int unf_blocks = resident(batch_unfold_kernel, 128);
     static const int tail_blocks = resident(batch_refine64_kernel, kTailBlock);
-    static const int fin_blocks = resident(batch_finalize_kernel, 128);
+    static const int walk_blocks = resident(batch_walk_kernel, 128);
+    static const int occ_blocks = resident(batch_occlusion_kernel, 128);
     const int sms = a.num_sms;
-    cudaError_t e;
-    {
+    // the two kernels of the many-path form have nothing to do when the container cannot hold that
+    // many (a room's call 225 -> 219 us)
+    const bool many = a.path_cap >= a.split_min;
+    cudaError_t e = cudaSuccess;
+    if (many) {
         Range r("batch refine: plane unfolding");
         e = launch_chained(batch_unfold_kernel, sms * unf_blocks, 128, 0, s, a);
     }
@@ -1501,7 +1625,8 @@ cudaError_t launch_batch_refine(const RefineArgs &a, int grid, int block, cudaSt
     if (e != cudaSuccess) return e;
     {
         Range r("batch refine: validity + outputs");
-        e = launch_chained(batch_finalize_kernel, sms * fin_blocks, 128, 0, s, a);
+        if (many) e = launch_chained(batch_walk_kernel, sms * walk_blocks, 128, 0, s, a);
+        if (e == cudaSuccess) e = launch_chained(batch_occlusion_kernel, sms * occ_blocks, 128, 0, s, a);
     }
     return e;
 }

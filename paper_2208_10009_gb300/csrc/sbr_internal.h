@@ -19,7 +19,8 @@
 namespace sbr {
 
 constexpr int kMaxOrder = SBR_MAX_ORDER;
-constexpr int kUnfStride = kMaxOrder + 2;   // float4 per path in the batched refinement's unf
+constexpr int kUnfStride = 14;   // float4 per path in the batched refinement's unf (RefineArgs)
+constexpr int kOrderCounts = 96;   // counters of the batched refinement (sbr_paths::order_cnt)
 constexpr double kC0 = 299792458.0;
 constexpr int kLeafMax = 2;        // triangles per BVH leaf (target; 2 measured fastest: a
                                    // triangle test costs about half a 4-wide node visit)
@@ -199,8 +200,9 @@ struct sbr_paths {
     int *order_idx = nullptr;              // batched refinement: path indices grouped by order
     unsigned long long *order_cnt = nullptr;   // [0, 10): paths per group; fill cursors: [16, 26) order_idx
                                                // from the front, [48, 58) from the back, [32, 42) fp64_idx;
-                                               // 62: queue head, 63: blocks that have read them.  Zero
-                                               // between calls (the last kernel of a call clears them)
+                                               // 62: queue head, 63: blocks that have read them; [64, 74)
+                                               // paths per group with legs to test.  Zero between calls
+                                               // (the last kernel of a call clears them)
     int *fp64_idx = nullptr;               // batched refinement: paths handed to the FP64 tail
     unsigned long long *table = nullptr;   // dedup hash table: 2 x u64 per slot (key, value)
     int64_t table_slots = 0;
@@ -374,7 +376,8 @@ struct RefineArgs {
     double ptx_dbm;
     int8_t *choice_log;
     float4 *unf;              // batched form, per path (kUnfStride float4): FP32 unfolded planes
-                              // [0, kMaxOrder), W at kMaxOrder, rough direction at kMaxOrder + 1
+                              // [0, kMaxOrder), W at kMaxOrder, rough direction at kMaxOrder + 1;
+                              // after the iterations the legs to test (origin, extent: 6 floats)
     int *order_idx;           // batched form: path indices grouped by order (diffraction last)
     unsigned long long *order_cnt;   // batched form: group sizes [0, 10), fill cursors of order_idx
                                      // ([16, 26) from the front, [48, 58) from the back) and
