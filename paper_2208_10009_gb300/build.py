@@ -24,7 +24,7 @@ SO = os.path.join(OUT, "libsbr.so")
 SO_CHECKED = os.path.join(OUT, "libsbr_checked.so")
 SO_PROBE = os.path.join(OUT, "libsbr_probe.so")   # FP32 peak microbenchmark (measurement only)
 SOURCES = ["capi.cu", "host_geometry.cpp", "host_wedges.cpp", "host_faces.cpp", "kernels_trace.cu", "kernels_diffract.cu",
-           "kernels_paths.cu", "kernels_refine.cu", "kernels_unfold.cu", "noalloc.cu"]
+           "kernels_receivers.cu", "kernels_paths.cu", "kernels_refine.cu", "kernels_unfold.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 VARIANTS = {SO: [], SO_CHECKED: ["-DSBR_CHECKED"], SO_PROBE: []}
 VARIANT_SOURCES = {SO: SOURCES, SO_CHECKED: SOURCES, SO_PROBE: ["probe_fp32.cu"]}

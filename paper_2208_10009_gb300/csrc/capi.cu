@@ -616,6 +616,9 @@ sbr_status sbr_scene_get_info(const sbr_scene *sc, sbr_scene_info *out) {
 }
 
 // ------------------------------------------------------------------------------ receivers
+// Receiver sets whose tree the device builds (sbr_rx_upload: why these lines, both sides' times)
+static constexpr int kRxDeviceMin = 64, kRxDeviceMax = 131072;
+
 sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset **out) {
     if (!ctx || !out) return fail(ctx, SBR_EINVAL, "sbr_rx_upload: null argument");
     *out = nullptr;
@@ -632,11 +635,20 @@ sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset *
     }
     for (float v : host)
         if (!std::isfinite(v)) return fail(ctx, SBR_EINVAL, "sbr_rx_upload: non-finite receiver coordinate");
+    // The tree is built on the device (kernels_receivers.cu) between two lines: few receivers cost
+    // the host less than the launches, and beyond the upper one the device's ranks by counting (n^2
+    // comparisons) overtake the host's search.  Whole call, host -> device: 1 receiver 18 -> 23 us,
+    // 64 37 -> 35, 256 99 -> 51, 1,024 343 -> 69, 4,096 910 -> 125, 16,384 3,440 -> 481, 65,536
+    // 13,500 -> 4,420, 131,072 27,200 -> 15,900, 262,144 58,000 -> 60,000.
+    const bool on_device = nrx >= kRxDeviceMin && nrx <= kRxDeviceMax;
     BvhOut bvh;
     std::string err;
-    if (!build_bvh(host, host, 1, bvh, err)) return fail(ctx, SBR_EINVAL, err);
-    if (bvh.max_stack4 > kStack4) return fail(ctx, SBR_EINVAL, "sbr_rx_upload: receiver BVH too deep");
-    std::vector<float4> pts((size_t)std::max(nrx, 1)), by_id((size_t)std::max(nrx, 1));
+    if (!on_device) {
+        if (!build_bvh(host, host, 1, bvh, err)) return fail(ctx, SBR_EINVAL, err);
+        if (bvh.max_stack4 > kStack4) return fail(ctx, SBR_EINVAL, "sbr_rx_upload: receiver BVH too deep");
+    }
+    const size_t room = (size_t)std::max(nrx, 1);
+    std::vector<float4> by_id(room), pts(on_device ? 0 : room);
     sbr_rxset *rs = new (std::nothrow) sbr_rxset();
     if (!rs) return fail(ctx, SBR_ENOMEM, "rx: host allocation failed");
     for (int a = 0; a < 3; ++a) {
@@ -644,20 +656,20 @@ sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset *
         rs->dev.hi[a] = -INFINITY;
     }
     for (int i = 0; i < nrx; ++i) {
-        int o = bvh.prim_order[i];
-        pts[i] = make_float4(host[3 * o], host[3 * o + 1], host[3 * o + 2], bits_as_float(o));
         by_id[i] = make_float4(host[3 * i], host[3 * i + 1], host[3 * i + 2], 0.0f);
         for (int a = 0; a < 3; ++a) {
             rs->dev.lo[a] = std::min(rs->dev.lo[a], host[3 * i + a]);
             rs->dev.hi[a] = std::max(rs->dev.hi[a], host[3 * i + a]);
         }
+        if (on_device) continue;
+        const int o = bvh.prim_order[i];
+        pts[i] = make_float4(host[3 * o], host[3 * o + 1], host[3 * o + 2], bits_as_float(o));
     }
-    float4 *d_nodes, *d_nodes4, *d_pts, *d_by;
+    float4 *d_nodes4, *d_pts, *d_by;
     Carver cv;
-    cv.add(&d_nodes, bvh.nodes.size());
-    cv.add(&d_nodes4, bvh.nodes4.size());
-    cv.add(&d_pts, pts.size());
-    cv.add(&d_by, by_id.size());
+    cv.add(&d_nodes4, on_device ? (size_t)8 * rx_tree_nodes(nrx) : bvh.nodes4.size());
+    cv.add(&d_pts, room);
+    cv.add(&d_by, room);
     rs->mem = dev_alloc(ctx, cv.total);
     if (!rs->mem) {
         delete rs;
@@ -665,14 +677,25 @@ sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset *
     }
     rs->bytes = cv.total;
     cv.bind(rs->mem);
-    SBR_CUDA(cudaMemcpyAsync(d_nodes, bvh.nodes.data(), bvh.nodes.size() * sizeof(float4), cudaMemcpyHostToDevice,
-                             ctx->stream));
-    SBR_CUDA(cudaMemcpyAsync(d_nodes4, bvh.nodes4.data(), bvh.nodes4.size() * sizeof(float4), cudaMemcpyHostToDevice,
-                             ctx->stream));
-    SBR_CUDA(cudaMemcpyAsync(d_pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
     SBR_CUDA(cudaMemcpyAsync(d_by, by_id.data(), by_id.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
-    SBR_CUDA(cudaStreamSynchronize(ctx->stream));
-    rs->dev.nodes = d_nodes;
+    if (on_device) {
+        const size_t bytes = (size_t)rx_tree_scratch(nrx) * sizeof(float4);
+        float4 *scratch = bytes ? static_cast<float4 *>(dev_alloc(ctx, bytes)) : nullptr;
+        if (bytes && !scratch) {
+            dev_free(ctx, rs->mem, rs->bytes);
+            delete rs;
+            return fail(ctx, SBR_ENOMEM, "rx: device allocation failed");
+        }
+        cudaError_t e = launch_rx_tree(d_by, nrx, d_pts, scratch, d_nodes4, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+        dev_free(ctx, scratch, bytes);
+        SBR_CUDA(e);
+    } else {
+        SBR_CUDA(cudaMemcpyAsync(d_nodes4, bvh.nodes4.data(), bvh.nodes4.size() * sizeof(float4),
+                                 cudaMemcpyHostToDevice, ctx->stream));
+        SBR_CUDA(cudaMemcpyAsync(d_pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
+        SBR_CUDA(cudaStreamSynchronize(ctx->stream));
+    }
     rs->dev.nodes4 = d_nodes4;
     rs->dev.pts = d_pts;
     rs->dev.by_id = d_by;

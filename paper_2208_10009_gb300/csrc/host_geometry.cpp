@@ -288,21 +288,6 @@ void put_child(float4 *n, int slot, const Box &b) {
 
 }  // namespace
 
-// the smallest FP16 value >= x (x >= 0; +inf beyond 65504)
-static unsigned short half_up(double x) {
-    if (x > 65504.0) return 0x7C00;
-    if (x < 6.103515625e-05) {                            // subnormal: units of 2^-24
-        const double q = x * 16777216.0;
-        const int i = (int)q;
-        return (unsigned short)(i + ((double)i < q));
-    }
-    float f = (float)x;
-    if ((double)f < x) f = std::nextafter(f, INFINITY);
-    unsigned u;
-    std::memcpy(&u, &f, sizeof(u));
-    return (unsigned short)(((u + 0x1FFF) >> 13) - (112u << 10));
-}
-
 bool build_bvh(const std::vector<float> &lo, const std::vector<float> &hi, int leaf_max, BvhOut &out,
                std::string &err) {
     size_t n = lo.size() / 3;

@@ -3,7 +3,9 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <string>
 #include <vector>
@@ -63,6 +65,21 @@ struct __align__(32) Plane64 {
 // f[5] = the four child refs (same encoding as BVH2; an empty slot is a leaf with 0 primitives
 // and a far-away point box); the rest unused.  A visit reads 88 bytes of it.
 
+// the smallest FP16 value >= x (x >= 0; +inf beyond 65504)
+__host__ __device__ inline unsigned short half_up(double x) {
+    if (x > 65504.0) return 0x7C00;
+    if (x < 6.103515625e-05) {                            // subnormal: units of 2^-24
+        const double q = x * 16777216.0;
+        const int i = (int)q;
+        return (unsigned short)(i + ((double)i < q));
+    }
+    float f = (float)x;
+    if ((double)f < x) f = nextafterf(f, INFINITY);
+    unsigned u;
+    memcpy(&u, &f, sizeof(u));
+    return (unsigned short)(((u + 0x1FFF) >> 13) - (112u << 10));
+}
+
 struct SceneDev {
     const float4 *nodes4;     // 8 per BVH4 node
     const float4 *nodes;      // 4 per node
@@ -94,7 +111,6 @@ struct SceneDev {
 
 struct RxDev {
     const float4 *nodes4;     // 4-wide BVH over receivers (same node layout as the scene's)
-    const float4 *nodes;      // BVH over receivers (same node layout)
     const float4 *pts;        // BVH order: (x, y, z, original id bits)
     const float4 *by_id;      // original order: (x, y, z, 0)
     int nrx;
@@ -258,6 +274,11 @@ void build_face_outlines(const float *verts, const int32_t *tris, const int32_t 
 bool build_polyhedron(int poly, std::vector<float4> &v, std::vector<int2> &e, std::vector<int4> &f);
 
 // kernels (kernels_*.cu)
+// the receivers' tree (n >= 1; a walk stacks at most 36 entries): node count, build from by_id into
+// pts (tree order, ids in w) and nodes4, with scratch for that many points
+int rx_tree_nodes(int n);
+int64_t rx_tree_scratch(int n);
+cudaError_t launch_rx_tree(const float4 *by_id, int n, float4 *pts, float4 *scratch, float4 *nodes4, cudaStream_t s);
 cudaError_t launch_raygen(const LatticeDev &lat, float4 *dirs, int64_t N, cudaStream_t s);
 // the same directions in the schedule's order (lattice_order.cuh), each with its ray id's bits in w
 // (prep: what a launch needs done before its trace, by the same kernel)
