@@ -22,7 +22,9 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
 __device__ __forceinline__ unsigned long long rec_hash(const RecDev &r) {
     unsigned long long h = mix64(((unsigned long long)(unsigned)r.tx << 40) ^ ((unsigned long long)(unsigned)r.rx << 8) ^
                                  (unsigned long long)r.order);
-    for (int j = 0; j < r.order; ++j) h = mix64(h ^ (unsigned long long)(unsigned)(r.faces[j] + 1));
+#pragma unroll
+    for (int j = 0; j < kMaxOrder; ++j)   // unrolled: the record stays in registers
+        if (j < r.order) h = mix64(h ^ (unsigned long long)(unsigned)(r.faces[j] + 1));
     return h == ~0ULL ? 0x5bd1e995ULL : h;
 }
 
@@ -32,9 +34,10 @@ __device__ __forceinline__ unsigned long long rec_value(const RecDev &r) {
 
 __device__ __forceinline__ bool same_key(const RecDev &a, const RecDev &b) {
     if (a.tx != b.tx || a.rx != b.rx || a.order != b.order) return false;
-    for (int j = 0; j < a.order; ++j)
-        if (a.faces[j] != b.faces[j]) return false;
-    return true;
+    bool same = true;
+#pragma unroll
+    for (int j = 0; j < kMaxOrder; ++j) same &= j >= a.order || a.faces[j] == b.faces[j];
+    return same;
 }
 
 // Hash-table slots a dedup pass over n records uses: the smallest power of two >= 2 n

@@ -33,6 +33,41 @@ __global__ void dedup_clear(DedupArgs a) {
         slot[i] = make_ulonglong2(~0ULL, ~0ULL);
 }
 
+// A record or a path record moves as 32-byte pieces, a sector each: threads take whole records, so
+// 16-byte accesses would pass every sector twice.
+struct Piece {
+    int w[8];
+};
+__device__ __forceinline__ Piece load_piece(const void *p) {
+    Piece v;
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
+                   "=r"(v.w[7])
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_piece(void *p, const Piece &v) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v.w[0]), "r"(v.w[1]),
+                 "r"(v.w[2]), "r"(v.w[3]), "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]), "r"(v.w[7])
+                 : "memory");
+}
+__device__ __forceinline__ RecDev load_record(const RecDev *p) {
+    static_assert(sizeof(RecDev) == 64 && kMaxOrder == 8, "the record is two pieces");
+    const Piece a = load_piece(p), b = load_piece(reinterpret_cast<const char *>(p) + 32);
+    RecDev r;
+    r.tx = a.w[0], r.rx = a.w[1], r.ray = a.w[2], r.order = a.w[3];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) r.faces[j] = a.w[4 + j], r.faces[4 + j] = b.w[j];
+    r.err = __int_as_float(b.w[4]), r.dray = __int_as_float(b.w[5]), r.slot = b.w[6], r.pad = b.w[7];
+    return r;
+}
+
+// A record's key and value are read before they are written: most records find their path's slot
+// claimed (the office: 1.5M records, 236k paths), and many a smaller value in it, and then need no
+// atomic.  Keys are written once and values only fall, so an old read costs an atomic, no more.
+// Twice the blocks and this: 80 -> 75 us.  A table of 1.25 n instead of 2 n slots gave 4 us more
+// but long probe runs once every record is a path of its own.
 __global__ void dedup_insert(DedupArgs a) {
     wait_predecessor();
     int *owner = reinterpret_cast<int *>(a.table + 2 * a.slots);
@@ -40,14 +75,16 @@ __global__ void dedup_insert(DedupArgs a) {
     unsigned long long *tab = a.table;   // key of slot s at 2 s, its value at 2 s + 1
     const unsigned long long used = used_slots(a), mask = used - 1;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        RecDev r = a.recs[i];
+        const RecDev r = load_record(a.recs + i);
         unsigned long long h = rec_hash(r), v = rec_value(r);
         unsigned long long s = h & mask;
         for (unsigned long long probe = 0; probe < used; ++probe) {
-            unsigned long long prev = atomicCAS(tab + 2 * s, ~0ULL, h);
-            if (prev == ~0ULL || prev == h) {
-                atomicMin(tab + 2 * s + 1, v);
-                if (prev == ~0ULL) owner[s] = (int)i;
+            unsigned long long key, val;
+            asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(key), "=l"(val) : "l"(tab + 2 * s) : "memory");
+            if (key == ~0ULL) key = atomicCAS(tab + 2 * s, ~0ULL, h);
+            if (key == ~0ULL || key == h) {
+                if (v < val) atomicMin(tab + 2 * s + 1, v);
+                if (key == ~0ULL) owner[s] = (int)i;
                 a.recs[i].slot = (int)s;
                 break;
             }
@@ -58,52 +95,75 @@ __global__ void dedup_insert(DedupArgs a) {
 
 // Every slot's winner becomes a path, and every record is compared with the record that claimed
 // its slot (a differing key is a hash collision): one pass over the records, where a pass of its own
-// compared them with the winners (office, 1.5M records: 142 + 32 -> 140 us).
+// compared them with the winners (office, 1.5M records: 142 + 32 -> 140 us).  A warp takes places
+// for all its winners with one atomic, and the records stay in registers (indexed by the order they
+// had been in local memory): 123 -> 85 us for the office, 92 -> 55 for half of its records.  What
+// is left are scattered 32-byte reads of the table and the owners' records, 4 TB/s in all; loading
+// a record ahead, or more warps with fewer registers, changed nothing.
 __global__ void dedup_select(DedupArgs a) {
     wait_predecessor();
     const long long n = num_records(a);
     const unsigned long long *tab = a.table;
     const int *owner = reinterpret_cast<const int *>(a.table + 2 * a.slots);
+    const int lane = threadIdx.x & 31;
     unsigned bad = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        RecDev r = a.recs[i];
-        if (r.slot < 0) {
-            ++bad;
-            continue;
+    for (long long first = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); first < n;
+         first += (long long)gridDim.x * blockDim.x) {
+        const long long i = first + lane;
+        RecDev r;
+        bool win = false;
+        if (i < n) {
+            r = load_record(a.recs + i);
+            if (r.slot < 0) {
+                ++bad;
+            } else {
+                const int o = owner[r.slot];
+                win = tab[2 * (long long)r.slot + 1] == rec_value(r) &&
+                      (a.shard_world <= 1 || (r.tx * a.nrx + r.rx) % a.shard_world == a.shard_rank);
+                if (o != (int)i && !same_key(r, load_record(a.recs + o))) ++bad;
+            }
         }
-        const int o = owner[r.slot];
-        if (o != (int)i && !same_key(r, a.recs[o])) ++bad;
-        if (tab[2 * (long long)r.slot + 1] != rec_value(r)) continue;
-        if (a.shard_world > 1 && (r.tx * a.nrx + r.rx) % a.shard_world != a.shard_rank) continue;
-        unsigned long long p = atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + kPaths), 1ULL);
-        if ((long long)p >= a.path_cap) continue;
-        sbr_path_record out;
-        out.tx = r.tx;
-        out.rx = r.rx;
-        out.ray = r.ray;
-        out.order = r.order;
-        for (int j = 0; j < kMaxOrder; ++j) out.faces[j] = r.faces[j];
-        out.rough_err = r.err;
-        out.rough_dray = r.dray;
-        out.iters = 0;
-        out.valid = 0;
+        const unsigned winners = __ballot_sync(0xffffffffu, win);
+        if (winners == 0) continue;
+        unsigned long long p = 0;
+        if (lane == 0)
+            p = atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + kPaths), (unsigned long long)__popc(winners));
+        p = __shfl_sync(0xffffffffu, p, 0) + __popc(winners & ((1u << lane) - 1u));
+        if (!win || (long long)p >= a.path_cap) continue;
+        union {
+            sbr_path_record rec;
+            Piece piece[4];
+        } out;
+        static_assert(sizeof(out) == sizeof(sbr_path_record) && sizeof(out) == 128, "the path record is four pieces");
+        out.rec.tx = r.tx;
+        out.rec.rx = r.rx;
+        out.rec.ray = r.ray;
+        out.rec.order = r.order;
+#pragma unroll
+        for (int j = 0; j < kMaxOrder; ++j) out.rec.faces[j] = r.faces[j];
+        out.rec.rough_err = r.err;
+        out.rec.rough_dray = r.dray;
+        out.rec.iters = 0;
+        out.rec.valid = 0;
         float4 d = __ldg(a.dirs + (a.sched_n > 0 ? schedule_place(r.ray, a.sched_n) : r.ray));
-        out.dir[0] = d.x;
-        out.dir[1] = d.y;
-        out.dir[2] = d.z;
-        out.err = r.err;
-        out.delay = 0.0;
-        out.aod[0] = out.aod[1] = out.aoa[0] = out.aoa[1] = 0.0f;
-        out.power_dbm = 0.0f;
-        out.flags = 0;
-        a.paths[p] = out;
+        out.rec.dir[0] = d.x;
+        out.rec.dir[1] = d.y;
+        out.rec.dir[2] = d.z;
+        out.rec.err = r.err;
+        out.rec.delay = 0.0;
+        out.rec.aod[0] = out.rec.aod[1] = out.rec.aoa[0] = out.rec.aoa[1] = 0.0f;
+        out.rec.power_dbm = 0.0f;
+        out.rec.flags = 0;
+        char *dst = reinterpret_cast<char *>(a.paths + p);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) store_piece(dst + 32 * k, out.piece[k]);
     }
     if (bad) atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + kCollisions), (unsigned long long)bad);
 }
 
 
 cudaError_t launch_dedup(const DedupArgs &a, int num_sms, cudaStream_t s) {
-    int grid = num_sms * 4;
+    int grid = num_sms * 8;
     cudaError_t e = launch_chained(dedup_clear, grid, 256, 0, s, a);
     if (e == cudaSuccess) e = launch_chained(dedup_insert, grid, 256, 0, s, a);
     if (e == cudaSuccess) e = launch_chained(dedup_select, grid, 256, 0, s, a);
