@@ -2,8 +2,9 @@
 // records with the same (Tx, Rx, face sequence) keep the one with the smallest error
 // angle of Eq. 3, ties to the lowest ray id.  Implemented as an open-addressing hash table
 // keyed by a 64-bit hash of the face sequence with a 64-bit atomicMin on
-// (error-angle bits, ray id); a second pass checks every record against its slot's
-// winner so that a hash collision is detected, never silently merged.
+// (error-angle bits, ray id); the pass that selects the winners checks every record against
+// the record that claimed its slot, so that a hash collision is detected, never silently
+// merged.
 #include "dedup_keys.cuh"
 #include "lattice_order.cuh"
 #include "sbr_device.cuh"

@@ -558,10 +558,10 @@ __global__ void __launch_bounds__(128, 7) trace_kernel(TraceArgs a) {
         unsigned need = __ballot_sync(0xffffffffu, !alive);
         if (need && !pool_empty && (__popc(need) >= a.refill_min || need == 0xffffffffu)) {
             // near the pool's end no more than a warp's share of what was left: full takes leave
-            // the last rays to a few warps.  (Half the large city's rays 13.15 -> 13.05 ms, all of
-            // them 31.46 -> 31.34; floors of 4 and 8 measure the same.  Not for a warp's first
-            // take: a launch with fewer rays than lanes then runs in more, emptier warps, a room's
-            // trace 26 -> 30 us.)
+            // the last rays to a few warps.  (One of four shards of the large city 13.15 -> 13.05
+            // ms, the whole 31.46 -> 31.34; floors of 4 and 8 measure the same.  Not for a warp's
+            // first take: a launch with fewer rays than lanes then runs in more, emptier warps, a
+            // room's trace 26 -> 30 us.)
             const int take = min(__popc(need), quota);
             unsigned long long base = 0;
             if (lane == 0) base = atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + kRayHead),
