@@ -480,7 +480,7 @@ def run_gpu(args):
            "clocks": clocks, "gpu_launches": _launches_per_step(
                {"diffraction": opts["diffraction"],
                 "frontier": st_t["rays"] >= 3_000_000 and scene.info()["bvh_nodes"] >= 1024}, world,
-               shape["lanes_per_path"] == 1 or paths.path_cap >= 16 * 32 * sms) * args.steps,
+               shape["lanes_per_path"] == 1 or paths.path_cap >= 16 * sms) * args.steps,
            "wall_s": t_wall, "e2e": e2e}
     if rank == 0 and not args.no_cpu_baseline:
         acc = oracle_accuracy(sc, tx, rx, recs) if world == 1 else None

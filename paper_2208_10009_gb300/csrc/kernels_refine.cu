@@ -1289,7 +1289,7 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
         PathGeo g;
         load_path(A, p, g);
         // the path's unfolded planes and W into the group's shared slot: with many paths
-        // the FP32 copy computed by batch_unfold_kernel, with few computed here in FP64 by
+        // as computed by batch_unfold_kernel, with few computed here by the same functions in
         // lanes 0..k-1 (one plane each) and lane G-1 (the receiver; k <= 8 <= G).  The
         // previous path's data is no longer read once every lane has reached this point.
         __syncwarp(gmask);
@@ -1331,7 +1331,7 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
         put_iterated(x, dv(x.cf.x, x.cf.y, x.cf.z), p);
         if (prebuilt) list_for_finalize(A, g, pi, p.err, (double)x.Rf);
         // iteration results; the validity test and outputs follow in batch_walk_kernel and
-// batch_occlusion_kernel
+        // batch_occlusion_kernel
         dst->iters = p.iters;
         dst->dir[0] = p.dir[0];
         dst->dir[1] = p.dir[1];
@@ -1418,12 +1418,11 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
     }
 }
 
-// Batched form, first pass (from split_min paths on), one thread per path: the FP64
-// unfolding of the path's face planes into Tx's space and of the receiver (the same
-// arithmetic as the plain form's), stored rounded to FP32 for the iteration
-// kernel, with the rough launch direction rounded to FP32.  GB300 runs FP64 at 1/64 of
-// the FP32 rate; with one path per lane every FP64 instruction serves 32 paths, where the
-// iteration kernel's lane groups would serve one.
+// Batched form, first pass (from split_min paths on), one thread per path: the
+// unfolding of the path's face planes into Tx's space and of the receiver in compensated
+// FP32 pairs (the same arithmetic as the plain form's), stored rounded to FP32 for the
+// iteration kernel, with the rough launch direction rounded to FP32.  With one path per lane
+// every instruction serves 32 paths, where the iteration kernel's lane groups would serve one.
 // It also counts the paths of each order group so that the iteration kernel can list them
 // group by group for the finalize kernel.
 __global__ void __launch_bounds__(128) batch_unfold_kernel(RefineArgs A) {
@@ -1599,8 +1598,8 @@ cudaError_t launch_batch_refine(const RefineArgs &a, int grid, int block, cudaSt
     static const int walk_blocks = resident(batch_walk_kernel, 128);
     static const int occ_blocks = resident(batch_occlusion_kernel, 128);
     const int sms = a.num_sms;
-    // the two kernels of the many-path form have nothing to do when the container cannot hold that
-    // many (a room's call 225 -> 219 us)
+    // the two kernels of the many-path form (from split_min paths on) have nothing to do when the
+    // container cannot hold that many (a room's call 225 -> 219 us)
     const bool many = a.path_cap >= a.split_min;
     cudaError_t e = cudaSuccess;
     if (many) {

@@ -406,8 +406,8 @@ struct RefineArgs {
     int *fp64_idx;            // batched form: paths whose FP64 iterations run in the tail kernel,
                               // grouped by order like order_idx
     int chunk;                // lanes per path in the batched kernel (8, 16, 32)
-    long long split_min;      // batched form: from this many paths on, validity and outputs run
-                              // one thread per path in a second kernel
+    long long split_min;      // batched form: from this many paths on, planes are unfolded and
+                              // paths walked one thread per path, legs queried one thread each
     int num_sms;
     int ntx, nrx, nf, nw;     // bounds of the ids a path record may hold
 };
