@@ -638,8 +638,8 @@ sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset *
     // The tree is built on the device (kernels_receivers.cu) between two lines: few receivers cost
     // the host less than the launches, and beyond the upper one the device's ranks by counting (n^2
     // comparisons) overtake the host's search.  Whole call, host -> device: 1 receiver 18 -> 23 us,
-    // 64 37 -> 35, 256 99 -> 51, 1,024 343 -> 69, 4,096 910 -> 125, 16,384 3,440 -> 481, 65,536
-    // 13,500 -> 4,420, 131,072 27,200 -> 15,900, 262,144 58,000 -> 60,000.
+    // 64 37 -> 35, 256 99 -> 51, 1,024 343 -> 67, 4,096 910 -> 111, 16,384 3,440 -> 476, 65,536
+    // 13,500 -> 4,490, 131,072 27,200 -> 16,300, 262,144 both 57,000.
     const bool on_device = nrx >= kRxDeviceMin && nrx <= kRxDeviceMax;
     BvhOut bvh;
     std::string err;

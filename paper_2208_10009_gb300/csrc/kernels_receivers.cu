@@ -15,9 +15,9 @@
 //     the launches.  The three orders are written out; the next launch reads the chosen one.
 //   - rx_subtree_kernel: a block takes one segment of at most kRxSub points in shared memory down
 //     to the leaves.
-// 4,096 receivers: five splits of 26, 18, 13, 9 and 8 us and the subtrees' 29 (launches timed
+// 4,096 receivers: five splits of 17, 14, 11, 7 and 8 us and the subtrees' 29 (launches timed
 // alone), bound by the comparisons' issue at first and by the loads' and barriers' latency after;
-// the upload 910 -> 125 us, the street walk's step 1.97 -> 1.11 ms.
+// the upload 910 -> 111 us.
 #include "sbr_device.cuh"
 #include "sbr_internal.h"
 #include "stream_launch.cuh"
@@ -26,8 +26,9 @@ namespace sbr {
 namespace {
 
 // 32 points a block and their comparisons over its warps: 4,096 points are 128 blocks.  (256 points
-// a block, one per thread, were 16 blocks: the whole upload 268 us; now 125.)
-constexpr int kSplitWarps = 8;
+// a block, one per thread, were 16 blocks: the whole upload 268 us.)  8 / 16 / 32 warps: 4,096
+// receivers 124 / 111 / 106 us, 65,536 4.41 / 4.49 / 5.03 ms.
+constexpr int kSplitWarps = 16;
 constexpr int kRxSub = 128;   // 32, 64 and 256 measured the same within 1 us
 // Points per leaf at most: with 1 the same times, with 4 (a level of nodes less, four tests for a
 // visit) the traces of the office and the canyon ran 1 % longer.
