@@ -328,10 +328,11 @@ typedef struct {
  * sub-rays of an iteration in parallel (one lane: all K in turn, the form for many
  * paths); a group that finishes a path (iteration cap, target reached, stalled) takes the
  * next one from a device work queue (atomic head), so uneven iteration counts do not idle
- * the GPU.  With many paths (and always with one lane per path) a launch before it unfolds
- * every path's planes one path per thread and a launch after it runs the FP64 iterations
- * one path per thread.  A last launch runs the validity test and outputs (one thread per
- * path when there are many, one warp per path when there are few).  Results equal
+ * the GPU.  A launch after it runs the FP64 iterations, one path per thread (one per warp while
+ * few have them).  From 16 paths an SM on (and always with one lane per path) a launch before it
+ * unfolds every path's planes one path per thread, and two last launches walk the paths for the
+ * outputs and the points' faces, one path per thread, and test their legs for occlusion, one leg
+ * per thread; with fewer, one last launch does both with a warp per path.  Results equal
  * sbr_refine's.  Capturable in a CUDA graph (no host synchronisation, no allocation). */
 sbr_status sbr_batch_refine(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *paths,
                             const sbr_refine_params *params, const sbr_batch_config *cfg);

@@ -1424,7 +1424,7 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
 // iteration kernel, with the rough launch direction rounded to FP32.  With one path per lane
 // every instruction serves 32 paths, where the iteration kernel's lane groups would serve one.
 // It also counts the paths of each order group so that the iteration kernel can list them
-// group by group for the finalize kernel.
+// group by group for batch_walk_kernel.
 __global__ void __launch_bounds__(128) batch_unfold_kernel(RefineArgs A) {
     wait_predecessor();
     __shared__ unsigned hist[10];
