@@ -205,6 +205,26 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) 
 constexpr int64_t kFrontMinRays = 3000000, kFrontMinNodes = 1024;
 constexpr size_t kFrontMaxBytes = (size_t)4 << 30;
 
+// The container's room for a frontier of `need` bytes, or null (the walks start at the root).  What a
+// launch writes belongs to its container, so that launches into other containers may overlap it.  A
+// block outgrown stays until the container goes, since a captured launch may hold its address; sizes
+// at least double, so all of them together take at most twice the largest.  No room is made while the
+// stream captures: memory from inside a capture would live and die with the graph.
+void *front_room(sbr_ctx *ctx, sbr_paths *p, size_t need) {
+    if (need > kFrontMaxBytes) return nullptr;
+    const size_t have = p->front.empty() ? 0 : p->front.back().second;
+    if (have >= need) return p->front.back().first;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const size_t bytes = std::max(need, std::min(2 * have, kFrontMaxBytes));
+    void *block = dev_alloc(ctx, bytes);
+    if (block) p->front.push_back({block, bytes});
+    return block;
+}
+
 // a value looked up once (0: not yet)
 template <class F>
 int cached(int &slot, F look_up) {
@@ -327,7 +347,6 @@ sbr_status sbr_ctx_destroy(sbr_ctx *ctx) {
     dev_free(ctx, ctx->dirs, ctx->dirs_bytes);
     dev_free(ctx, ctx->lattice_mem, ctx->lattice_bytes);
     dev_free(ctx, ctx->poly_mem, ctx->poly_bytes);
-    dev_free(ctx, ctx->front, ctx->front_bytes);
     cudaStreamSynchronize(ctx->stream);
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
@@ -757,6 +776,7 @@ sbr_status sbr_paths_destroy(sbr_ctx *ctx, sbr_paths *p) {
     dev_free(ctx, p->mem, p->bytes);
     dev_free(ctx, p->tx_mem, p->tx_bytes);
     dev_free(ctx, p->pair_mem, p->pair_bytes);
+    for (auto &b : p->front) dev_free(ctx, b.first, b.second);
     delete p;
     return SBR_OK;
 }
@@ -884,12 +904,7 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
         scene->max_stack4 + kFrontEntries <= kStack4) {
         const int64_t group0 = place0 / kFrontRays, groups = (place0 + places + kFrontRays - 1) / kFrontRays - group0;
         const size_t need = (size_t)ntx * groups * kFrontEntries * sizeof(int2);
-        if (need <= kFrontMaxBytes && ctx->front_bytes < need) {
-            dev_free(ctx, ctx->front, ctx->front_bytes);
-            ctx->front = dev_alloc(ctx, need);
-            ctx->front_bytes = ctx->front ? need : 0;
-        }
-        if (ctx->front && need <= ctx->front_bytes) {
+        if (void *room = front_room(ctx, paths, need)) {
             FrontArgs f;
             f.scene = a.scene;
             f.dirs = a.dirs;
@@ -901,7 +916,7 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
             f.ray_end = a.ray_end;
             f.group0 = a.group0 = group0;
             f.groups = a.groups = groups;
-            f.front = static_cast<int2 *>(ctx->front);
+            f.front = static_cast<int2 *>(room);
             a.front = f.front;
             Range r("sbr_launch: first segments' frontier");
             SBR_CUDA(launch_frontier(f, ctx->stream));

@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/sbr.h"
@@ -169,9 +170,6 @@ struct sbr_ctx {
     size_t dirs_bytes = 0;
     int dirs_n = 0;
     bool dirs_valid = false;
-    // first segments' frontier
-    void *front = nullptr;
-    size_t front_bytes = 0;
     // lattice tables
     void *lattice_mem = nullptr;
     size_t lattice_bytes = 0;
@@ -235,6 +233,8 @@ struct sbr_paths {
     size_t tx_bytes = 0;
     int32_t ntx = 0, nrx = 0, n_div = 0, max_order = 0, launcher = 0;
     const sbr_rxset *rx = nullptr;
+    // first segments' frontier: blocks of growing size, the last in use (front_room in capi.cu)
+    std::vector<std::pair<void *, size_t>> front;
     float alpha = 1.0f;
     int64_t ray_begin = 0, ray_count = 0;  // ray ids traced per transmitter by the last launch
     bool timed = false;                    // last launch recorded kernel events
