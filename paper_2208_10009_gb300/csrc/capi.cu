@@ -1132,6 +1132,7 @@ static sbr_status refine_args(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *p
     // 70 -> 108 us, 2,677 118 -> 122, 11,589 209 -> 129; 4,026 paths with 60 iterations, the call,
     // 683 -> 608 us.
     A.split_min = 16LL * std::max(ctx->num_sms, 1);
+    A.deep = !A.target_on && A.theta_launch * std::pow(sh, prm->max_iters) < 1e-14;
     A.ntx = paths->ntx;
     A.nrx = paths->nrx;
     A.nf = scene->dev.nf;

@@ -488,85 +488,190 @@ __device__ __forceinline__ int iterate32(const UnfF &uf, int nk, int K, int off,
 // |e_k| exceeds the smallest by more than 2 delta has the larger key64, valid or not, so only
 // the others are evaluated, exactly as before: one as a rule, more within about 1e-14 of the
 // double floor.  Should the smallest be invalid (a face met out of order), all K are.
-// Office tail (942,656 paths, K = 16): 935 -> 302 us, FP64 pipe no longer the bound; large city
-// (17.7k paths, 12 FP64 iterations, K = 9): 590 -> 387 us; 4,026 room paths run to the double
-// floor (60 iterations, K = 6), whose FP64 iterations ran in lane groups: 1452 -> 530 us.
-__device__ __forceinline__ int iterate64(const UnfD &ud, int nk, int K, int off, const SubTab64 &tab, double R,
-                                         dvec3 &c, double &key_c, double &dw_c) {
-    dvec3 u, v;
-    frame64(c, u, v);
-    const dvec3 W = dv(ud.w.x, ud.w.y, ud.w.z), cw = dcross(c, W);
-    const float3 e0 = make_float3((float)cw.x, (float)cw.y, (float)cw.z);
-    const float3 Wf = make_float3((float)W.x, (float)W.y, (float)W.z);
-    float3 uW, vW;
-    {
+// Office tail (942,656 paths, K = 16): 935 -> 302 us, the FP64 pipe 71 % busy and still the bound; large
+// city (17.7k paths, 12 FP64 iterations, K = 9): 590 -> 387 us.
+struct Rank64 {   // |e_k|^2 of the sub-rays of one iteration
+    float3 e0, uW, vW;
+    float Rf, nW, rho, sa, ca;
+    __device__ __forceinline__ Rank64(const UnfD &ud, dvec3 c, double R) {
+        const dvec3 W = dv(ud.w.x, ud.w.y, ud.w.z), cw = dcross(c, W);
+        e0 = make_float3((float)cw.x, (float)cw.y, (float)cw.z);
+        const float3 Wf = make_float3((float)W.x, (float)W.y, (float)W.z);
         const float3 cf = make_float3((float)c.x, (float)c.y, (float)c.z);
         float3 uf, vf;
         frame32(cf, frame_axis64(c), uf, vf);
         uW = cross(uf, Wf);
         vW = cross(vf, Wf);
+        Rf = (float)R;
+        nW = sqrtf(dot(Wf, Wf));
+        rho = -1.0f;
+        sa = 0.0f;
+        ca = 1.0f;
     }
-    const float Rf = (float)R, nW = sqrtf(dot(Wf, Wf));
-    float rho = -1.0f, sa = 0.0f, ca = 1.0f, samax = 0.0f, a1 = INFINITY, a2 = INFINITY;
-    auto ranked = [&](int k) {   // |e_k|^2; the patterns' sub-rays come ring by ring
-        if (c_sub.rho[off + k] != rho) {
-            rho = c_sub.rho[off + k];
+    __device__ __forceinline__ float operator()(int i) {   // entry i of the table; sub-rays come ring by ring
+        if (c_sub.rho[i] != rho) {
+            rho = c_sub.rho[i];
             sincos_sub32(rho * Rf, sa, ca);
         }
-        const float3 e = e0 * ca + (uW * c_sub.cphi[off + k] + vW * c_sub.sphi[off + k]) * sa;
+        const float3 e = e0 * ca + (uW * c_sub.cphi[i] + vW * c_sub.sphi[i]) * sa;
         return dot(e, e);
-    };
+    }
+    // a sub-ray beyond it cannot win (never so for a NaN); a1: the smallest, samax: the largest sine
+    __device__ __forceinline__ float limit(float a1, float samax) const {
+        const float delta = 1e-5f * (samax * nW + sqrtf(dot(e0, e0))) + 4e-15f * nW + 1e-18f;
+        const float lim = sqrtf(a1) + 2.0f * delta;
+        return lim * lim * 1.00001f;
+    }
+};
+
+// The best sub-ray evaluated so far; lowest k on ties, as in the plain rule.
+struct Best64 {
+    double key, dw;
+    dvec3 d;
+    int k;
+    __device__ __forceinline__ Best64(dvec3 c) : key(INFINITY), dw(0.0), d(c), k(0x7fffffff) {}
+    // sub-ray i, evaluated exactly; false: invalid.  (Keys are >= 0 or +inf: their bits order like the values.)
+    __device__ __forceinline__ bool try_ray(const UnfD &ud, int nk, const SubTab64 &tab, int off, int i, double R, dvec3 c,
+                                            dvec3 u, dvec3 v) {
+        double s, co, w = 0.0;
+        sincos_sub(tab.rho[off + i] * R, s, co);
+        const dvec3 di = c * co + (u * tab.cphi[off + i] + v * tab.sphi[off + i]) * s;
+        const double x = key64(ud, nk, di, w);
+        const long long bx = __double_as_longlong(x), b = __double_as_longlong(key);
+        if (bx >= __double_as_longlong((double)INFINITY)) return false;
+        if (bx < b || (bx == b && i < k)) {
+            key = x;
+            dw = w;
+            k = i;
+            d = di;
+        }
+        return true;
+    }
+};
+
+__device__ __forceinline__ int iterate64(const UnfD &ud, int nk, int K, int off, const SubTab64 &tab, double R,
+                                         dvec3 &c, double &key_c, double &dw_c) {
+    dvec3 u, v;
+    frame64(c, u, v);
+    Rank64 rank(ud, c, R);
+    Best64 best(c);
+    float samax = 0.0f, a1 = INFINITY, a2 = INFINITY;
     int k1 = 0;
     for (int k = 0; k < K; ++k) {
-        const float a = ranked(k);
-        samax = fmaxf(samax, sa);
+        const float a = rank(off + k);
+        samax = fmaxf(samax, rank.sa);
         a2 = fminf(a2, fmaxf(a, a1));
         if (a < a1) {
             a1 = a;
             k1 = k;
         }
     }
-    const float delta = 1e-5f * (samax * nW + sqrtf(dot(e0, e0))) + 4e-15f * nW + 1e-18f;
-    const float lim = sqrtf(a1) + 2.0f * delta;
-    const float thr = lim * lim * 1.00001f;   // a sub-ray beyond it cannot win (never so for a NaN)
-    unsigned left = 1u << k1;                 // the sub-rays to evaluate
+    const float thr = rank.limit(a1, samax);
+    unsigned left = 1u << k1;   // the sub-rays that may win
     if (!(a2 > thr)) {
-        rho = -1.0f;
+        rank.rho = -1.0f;
         for (int k = 0; k < K; ++k)
-            if (!(ranked(k) > thr)) left |= 1u << k;
+            if (!(rank(off + k) > thr)) left |= 1u << k;
     }
-    double best = INFINITY, bdw = 0.0;
-    int bk = -1;
-    dvec3 bd = c;
-    for (bool first = true; left;) {   // lowest k first: the plain rule on ties
-        const int k = __ffs(left) - 1;
-        left &= left - 1;
-        double s, co;
-        sincos_sub(tab.rho[off + k] * R, s, co);
-        const dvec3 dk = c * co + (u * tab.cphi[off + k] + v * tab.sphi[off + k]) * s;
-        double dw = 0.0;
-        const double key = key64(ud, nk, dk, dw);
-        // key < best, both >= 0 (or +inf): their bits order like the values
-        if (__double_as_longlong(key) < __double_as_longlong(best)) {
-            best = key;
-            bdw = dw;
-            bk = k;
-            bd = dk;
+    for (;;) {
+        bool ok = false;
+        for (; left; left &= left - 1) {
+            const int k = __ffs(left) - 1;
+            const bool valid = best.try_ray(ud, nk, tab, off, k, R, c, u, v);
+            ok |= k == k1 && valid;
         }
-        if (first && k == k1 && !(__double_as_longlong(key) < __double_as_longlong((double)INFINITY))) {
-            // the nearest is invalid, so the margin says nothing: take all, from the start
-            first = false;
-            left = (1u << K) - 1u;
-            best = INFINITY;
-            bk = -1;
+        if (k1 < 0 || ok) break;
+        k1 = -1;   // the nearest is invalid, so the margin says nothing: take all
+        left = (1u << K) - 1u;
+    }
+    if (best.k >= K) return -1;
+    c = best.d * (1.0 / dnorm(best.d));
+    key_c = best.key;
+    dw_c = best.dw;
+    return best.k;
+}
+
+// The same iteration by G lanes that share a path (1 < G <= 32, a power of two; gl: the lane's
+// place among them, gmask: they), for lists too short to fill the chip with a thread a path: lane gl
+// takes the sub-rays gl, gl + G, ...  With G >= K every sub-ray has a lane, and one exact evaluation a
+// lane costs what a single one does, so there is no ranking; with fewer lanes each ranks its own, and
+// only those that may win are evaluated, side by side (all lanes the same one where one is left; all K
+// should the nearest be invalid).  The winner's direction, key and d . W come from its lane by shuffles.  Near the double
+// floor, where the ranking cannot tell the sub-rays apart, a thread evaluates all K in turn and a
+// path's lanes K / G.
+__device__ __forceinline__ int iterate64_lanes(const UnfD &ud, int nk, int K, int off, const SubTab64 &tab, double R,
+                                               dvec3 &c, double &key_c, double &dw_c, int G, int gl, unsigned gmask) {
+    dvec3 u, v;
+    frame64(c, u, v);
+    unsigned own = 0;   // the lane's sub-rays
+    for (int k = gl; k < K; k += G) own |= 1u << k;
+    unsigned left = own;
+    int k1 = -1;
+    bool one = false;   // all lanes evaluate the same sub-ray
+    if (G < K) {
+        Rank64 rank(ud, c, R);
+        float samax = 0.0f, a = INFINITY;
+        int ka = gl;
+        for (int k = gl; k < K; k += G) {
+            const float x = rank(off + k);
+            samax = fmaxf(samax, rank.sa);
+            if (x < a) {
+                a = x;
+                ka = k;
+            }
         }
+        float a1 = a;
+        for (int o = G >> 1; o; o >>= 1) {
+            a1 = fminf(a1, __shfl_xor_sync(gmask, a1, o));
+            samax = fmaxf(samax, __shfl_xor_sync(gmask, samax, o));
+        }
+        k1 = __shfl_sync(gmask, ka, __ffs(__ballot_sync(gmask, a == a1)) - 1);
+        const float thr = rank.limit(a1, samax);
+        rank.rho = -1.0f;
+        left = 0;
+        for (int k = gl; k < K; k += G)
+            if (k == k1 || !(rank(off + k) > thr)) left |= 1u << k;
+        const unsigned have = __ballot_sync(gmask, left != 0);
+        const unsigned first = __shfl_sync(gmask, left, __ffs(have) - 1);
+        one = (have & (have - 1)) == 0 && (first & (first - 1)) == 0;
+        if (one) left = first;
     }
-    if (bk >= 0) {
-        c = bd * (1.0 / dnorm(bd));
-        key_c = best;
-        dw_c = bdw;
+    Best64 best(c);
+    for (;;) {
+        bool ok = false;
+        for (; left; left &= left - 1) {
+            const int k = __ffs(left) - 1;
+            const bool valid = best.try_ray(ud, nk, tab, off, k, R, c, u, v);
+            ok |= k == k1 && valid;
+        }
+        if (k1 < 0 || __any_sync(gmask, ok)) break;
+        k1 = -1;
+        one = false;
+        left = own;
     }
-    return bk;
+    if (!one) {
+        double key = best.key;
+        int bk = best.k;
+        for (int o = G >> 1; o; o >>= 1) {
+            const double x = __shfl_xor_sync(gmask, key, o);
+            const int k = __shfl_xor_sync(gmask, bk, o);
+            const long long bx = __double_as_longlong(x), b = __double_as_longlong(key);
+            if (bx < b || (bx == b && k < bk)) {
+                key = x;
+                bk = k;
+            }
+        }
+        if (bk >= K) return -1;
+        const int src = (threadIdx.x & 31) - gl + (bk & (G - 1));
+        best.d = dv(__shfl_sync(gmask, best.d.x, src), __shfl_sync(gmask, best.d.y, src), __shfl_sync(gmask, best.d.z, src));
+        best.dw = __shfl_sync(gmask, best.dw, src);
+        best.key = key;
+        best.k = bk;
+    }
+    c = best.d * (1.0 / dnorm(best.d));
+    key_c = best.key;
+    dw_c = best.dw;
+    return best.k;
 }
 
 // ----------------------------------------------------------------------------- a7/a8
@@ -1084,11 +1189,12 @@ __device__ __forceinline__ void fp32_phase(const RefineArgs &A, const PathGeo &g
 }
 
 // FP64 phase, from the FP32 phase's centre with its |d x W|^2 and d . W, or, with no iteration
-// done, from the FP64 rough direction.  A thread a path; several may run it in step (log: one of
-// them writes the choice log).
+// done, from the FP64 rough direction.  A thread a path, or (kShared) G lanes that share it, the state
+// the same in all of them.
+template <bool kShared>
 __device__ __forceinline__ void fp64_phase(const RefineArgs &A, const PathGeo &g, const UnfD &ud, int off,
                                            const SubTab64 &tab, const sbr_path_record &p, double shrink, double stall,
-                                           long long pi, bool log, Iterated &x) {
+                                           long long pi, int G, int gl, unsigned gmask, Iterated &x) {
     x.R = cone_radius64(A, p.rough_err, x.it, shrink);
     if (x.fp64) {
         x.c = dv(p.dir[0], p.dir[1], p.dir[2]);
@@ -1109,14 +1215,15 @@ __device__ __forceinline__ void fp64_phase(const RefineArgs &A, const PathGeo &g
             break;
         }
         const int ax = A.choice_log ? frame_axis64(x.c) : 0;
-        const int bk = iterate64(ud, g.k, A.K, off, tab, x.R, x.c, x.key, x.dw);
+        const int bk = kShared ? iterate64_lanes(ud, g.k, A.K, off, tab, x.R, x.c, x.key, x.dw, G, gl, gmask)
+                               : iterate64(ud, g.k, A.K, off, tab, x.R, x.c, x.key, x.dw);
         if (bk < 0) {
             x.fail = true;
             break;
         }
         x.flags |= SBR_PATH_FP64;
         x.fp64 = true;
-        if (log) A.choice_log[pi * A.max_iters + x.it] = choice_entry(bk, ax);
+        if (A.choice_log && gl == 0) A.choice_log[pi * A.max_iters + x.it] = choice_entry(bk, ax);
         x.R *= shrink;
         ++x.it;
     }
@@ -1201,7 +1308,7 @@ __global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
                 for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
                 ud.w = unfold_rx(A.scene, g);
             }
-            fp64_phase(A, g, ud, off, tab, p, shrink, stall, pi, A.choice_log && (!wide || lane == 0), x);
+            fp64_phase<false>(A, g, ud, off, tab, p, shrink, stall, pi, 1, wide ? lane : 0, 0, x);
             c = x.c;
         }
         put_iterated(x, c, p);
@@ -1341,19 +1448,24 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
     }
 }
 
-// Batched form, FP64 tail, one thread per path: the paths whose cone fell below fp64_below in
-// batch_refine_kernel continue here with the plain form's FP64 iterations (iterate64), so that
-// each instruction of GB300's narrow FP64 pipe serves 32 paths, where a lane group would serve
-// one.  The state carried over: a path that started in FP64 (no iteration done) takes its FP64
-// rough direction; otherwise the FP32 phase's centre with its |d x W|^2 and d . W.  With many
-// paths the path is then listed in its order group for batch_walk_kernel.  One warp a
-// block: the FP64 pipe belongs to the SM, so a short list (the large city's 17k paths are 535
-// warps) has to spread over as many SMs as it has warps.  A list of at most kTailWide paths an
-// SM takes a warp a path instead: its lanes unfold the planes side by side and then iterate
-// in step, which spares the waits of one thread's chain of mirrors (canyon, 631 paths with one
-// FP64 iteration each: 14 against 20 us a launch) and the divergence of its iterations;
-// with more paths the pipe is full of redundant lanes (8 paths an SM cost what a thread a path does).
-constexpr int kTailBlock = 32, kTailWide = 6;
+// Batched form, FP64 tail: the paths whose cone fell below fp64_below in batch_refine_kernel continue
+// here with the plain form's FP64 iterations.  The state carried over: a path that started in FP64 (no
+// iteration done) takes its FP64 rough direction; otherwise the FP32 phase's centre with its |d x W|^2
+// and d . W.  With many paths the path is then listed in its order group for batch_walk_kernel.  One
+// warp a block: the FP64 pipe belongs to the SM, so a list has to spread over as many SMs as it has
+// warps.  A thread a path (iterate64) makes each instruction of that narrow pipe serve 32 paths; a
+// shorter list would leave SMs without a warp and every warp waiting for its chain, so G lanes share a
+// path (iterate64_lanes, the planes unfolded side by side too): the most lanes that keep the list at
+// kTailWarps warps an SM, where the pipe is full.  Eight and four lanes only where the iterations run
+// to the double floor, where a thread has all K sub-rays to evaluate in turn: above it they have one,
+// and a thread a path costs the same or less (2,015 paths, K = 16, 16 iterations: 118 us, with eight
+// lanes 120; 4,031: 121, with four 132).  Below four lanes never (5,479 paths, two lanes: 156 us against
+// 130 above the floor).  Calls, 60 iterations and K = 16, before (a lane group of 16 a path
+// for the FP64 iterations too) -> one warp or one thread a path, all lanes alike -> now: 63 paths
+// 816 -> 1461 -> 307 us, 881 paths 773 -> 2246 -> 323, 4,031 paths 2162 -> 1492 -> 709; K = 6: 728 -> 426
+// -> 286, 1010 -> 612 -> 295, 1916 -> 480 -> 427.  kTailWarps 1 / 2 / 4 / 6 / 8: 1,133 paths, K = 16,
+// 843 / 604 / 389 / 389 / 637 us; 2,015 paths, K = 6, 635 / 538 / 381 / 385 / 567.
+constexpr int kTailBlock = 32, kTailWarps = 4;
 __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A) {
     wait_predecessor();
     const bool many = path_count(A) >= A.split_min;
@@ -1366,11 +1478,15 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
     const int off = c_sub.off[A.K];
     const double shrink = c_sub.shrink[A.K];
     const double stall = 1.0 / (1.0 - shrink) + 2.0 * shrink;
-    __shared__ UnfD s_ud;
     const int lane = threadIdx.x;
-    const bool wide = n <= kTailWide * (long long)A.num_sms;
-    const long long per = wide ? 1 : kTailBlock;   // paths a warp
-    for (long long t = blockIdx.x * per + (wide ? 0 : lane); t < n; t += gridDim.x * per) {
+    const long long room = (long long)kTailBlock * kTailWarps * A.num_sms;
+    int G = kTailBlock;   // lanes a path
+    while (G > (A.deep ? 4 : 16) && n * G > room) G >>= 1;
+    if (n * G > room) G = 1;
+    const int gl = lane & (G - 1);
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - gl);
+    const long long per = kTailBlock / G;   // paths a warp
+    for (long long t = blockIdx.x * per + lane / G; t < n; t += gridDim.x * per) {
         long long slot = t, base = 0;
         for (int b = 0; b < 10; ++b) {
             const long long nb = (long long)A.order_cnt[32 + b];
@@ -1383,19 +1499,23 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
         PathGeo g;
         load_path(A, p, g);
         UnfD ud;
-        const float4 *u = A.unf + kUnfStride * pi;
-        if (wide) {
-            __syncwarp();
-            if (lane < g.k) s_ud.p[lane] = unfold_plane(A.scene, g, lane);
-            if (lane == kTailBlock - 1) s_ud.w = unfold_rx(A.scene, g);
-            __syncwarp();
-            for (int j = 0; j < g.k; ++j) ud.p[j] = s_ud.p[j];
-            ud.w = s_ud.w;
+        if (G > 1) {   // a lane per plane and one for the receiver, passed on by shuffles
+            for (int j0 = 0; j0 <= g.k; j0 += G) {
+                D4 mine = {0.0, 0.0, 0.0, 0.0};
+                if (j0 + gl < g.k) mine = unfold_plane(A.scene, g, j0 + gl);
+                else if (j0 + gl == g.k) mine = unfold_rx(A.scene, g);
+                for (int i = 0; i < G && j0 + i <= g.k; ++i) {
+                    const int src = lane - gl + i;
+                    const D4 q = {__shfl_sync(gmask, mine.x, src), __shfl_sync(gmask, mine.y, src),
+                                  __shfl_sync(gmask, mine.z, src), __shfl_sync(gmask, mine.w, src)};
+                    (j0 + i < g.k ? ud.p[j0 + i] : ud.w) = q;
+                }
+            }
         } else {
             for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
             ud.w = unfold_rx(A.scene, g);
         }
-        const float4 cu = u[kMaxOrder + 1];
+        const float4 cu = A.unf[kUnfStride * pi + kMaxOrder + 1];
         Iterated x;
         x.cf = f3(cu);
         x.keyf = cu.w;
@@ -1404,8 +1524,9 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
         x.flags = 0;
         x.fp64 = x.it == 0;
         x.fail = false;
-        fp64_phase(A, g, ud, off, tab, p, shrink, stall, pi, A.choice_log && (!wide || lane == 0), x);
-        if (wide && lane != 0) continue;   // the lanes agree
+        if (G > 1) fp64_phase<true>(A, g, ud, off, tab, p, shrink, stall, pi, G, gl, gmask, x);
+        else fp64_phase<false>(A, g, ud, off, tab, p, shrink, stall, pi, 1, 0, 0, x);
+        if (gl != 0) continue;   // the lanes agree
         put_iterated(x, x.fp64 ? x.c : dv(x.cf.x, x.cf.y, x.cf.z), p);
         if (many) list_for_finalize(A, g, pi, p.err, x.R);
         sbr_path_record *dst = A.paths + pi;

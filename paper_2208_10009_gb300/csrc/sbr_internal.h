@@ -409,6 +409,7 @@ struct RefineArgs {
     long long split_min;      // batched form: from this many paths on, planes are unfolded and
                               // paths walked one thread per path, legs queried one thread each
     int num_sms;
+    int deep;                 // the iterations run to the double floor (no target, last cone below 1e-14 rad)
     int ntx, nrx, nf, nw;     // bounds of the ids a path record may hold
 };
 cudaError_t launch_refine(const RefineArgs &a, int grid, int block, cudaStream_t s);
