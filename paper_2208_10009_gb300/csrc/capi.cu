@@ -1133,6 +1133,10 @@ static sbr_status refine_args(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *p
     // 683 -> 608 us.
     A.split_min = 16LL * std::max(ctx->num_sms, 1);
     A.deep = !A.target_on && A.theta_launch * std::pow(sh, prm->max_iters) < 1e-14;
+    // Plain form, a warp a path up to here (one wave: twelve warps an SM), then a thread a path.  With
+    // a warp / a thread a path: 1,448 paths, 8 iterations (K = 6, none in FP64) 33 / 70 us, 10 in FP64
+    // 163 / 156, 60 in FP64 771 / 930 (K = 16: 781 / 2,911); 4,031 paths 76 / 44, 369 / 105, 1,787 / 539.
+    A.wide_max = 12LL * std::max(ctx->num_sms, 1);
     A.ntx = paths->ntx;
     A.nrx = paths->nrx;
     A.nf = scene->dev.nf;
@@ -1199,8 +1203,7 @@ sbr_status sbr_refine_pair(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *path
     A.index = paths->pair_off + npairs + 1;
     {
         Range r("sbr_refine_pair: iterations + validity + outputs");
-        // a warp a path up to twelve paths an SM, then a thread a path
-        const int per_block = count <= 12 * ctx->num_sms ? 4 : 128;
+        const int per_block = count <= A.wide_max ? 4 : 128;
         SBR_CUDA(launch_refine(A, (count + per_block - 1) / per_block, 128, ctx->stream));
     }
     return SBR_OK;

@@ -1243,11 +1243,10 @@ __device__ __forceinline__ void put_iterated(const Iterated &x, dvec3 c, sbr_pat
 }
 
 // a6-a8 in one launch with nothing shared between paths (static schedule): the plain and per-pair
-// forms.  A thread a path, or, while there are at most kPlainWide paths a warp of the grid, a warp
-// a path: few paths leave the chip idle and a thread's own chain of mirrors, K sub-rays, bounce
-// points and occlusion queries is what the launch waits for, so its lanes take them side by
-// side, as in the batched form's groups (110 paths of a cluttered room: 193 -> 45 us).
-constexpr int kPlainWide = 3;
+// forms.  A thread a path, or, up to RefineArgs::wide_max paths, a warp a path: few paths leave the
+// chip idle and a thread's own chain of mirrors, K sub-rays, bounce points and occlusion queries is
+// what the launch waits for, so its lanes take them side by side, as in the batched form's groups (110
+// paths of a cluttered room: 193 -> 45 us).
 __global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
     wait_predecessor();
     __shared__ SubTab64 tab;
@@ -1256,7 +1255,7 @@ __global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
     const long long total = A.range ? (long long)(A.range[1] - A.range[0]) : path_count(A);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    const bool wide = total <= kPlainWide * warps;
+    const bool wide = total <= A.wide_max;
     const int off = c_sub.off[A.K];
     const double shrink = c_sub.shrink[A.K];
     const float shrinkf = c_sub.shrink_f[A.K];
@@ -1308,7 +1307,8 @@ __global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
                 for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
                 ud.w = unfold_rx(A.scene, g);
             }
-            fp64_phase<false>(A, g, ud, off, tab, p, shrink, stall, pi, 1, wide ? lane : 0, 0, x);
+            if (wide) fp64_phase<true>(A, g, ud, off, tab, p, shrink, stall, pi, 32, lane, 0xffffffffu, x);
+            else fp64_phase<false>(A, g, ud, off, tab, p, shrink, stall, pi, 1, 0, 0, x);
             c = x.c;
         }
         put_iterated(x, c, p);

@@ -30,7 +30,10 @@ def _rough(ctx, nrx):
 def _refined(ctx, scene, tx, rxs, rough, paths, K, iters, lanes):
     ctx.paths_import(paths, rough, tx, rxs, 16)
     log = torch.full((paths.path_cap, iters), -1, dtype=torch.int8, device="cuda")
-    ctx.batch_refine(scene, paths, iters, K, fp64_below=10.0, choice_log=log, lanes_per_path=lanes)
+    if lanes:
+        ctx.batch_refine(scene, paths, iters, K, fp64_below=10.0, choice_log=log, lanes_per_path=lanes)
+    else:
+        ctx.refine(scene, paths, iters, K, fp64_below=10.0, choice_log=log)
     return ctx.query(paths), log.cpu().numpy()[: len(rough)]
 
 
@@ -41,8 +44,8 @@ def test_lengths_alike(gpu_ctx, K, iters):
     lines = [PER_SM * sms // g for g in (32, 16, 8, 4)]   # the longest list of each number of lanes
     assert len(rough) > lines[-1] + 33
     want, choice = _refined(gpu_ctx, scene, tx, rxs, rough, paths, K, iters, 16)
-    for n in [1, 33] + lines + [x + 1 for x in lines]:
-        for lanes in (16, 1):
+    for n in [1, 33, 12 * sms, 12 * sms + 1] + lines + [x + 1 for x in lines]:
+        for lanes in (16, 1, 0):   # 0: the plain form
             got, log = _refined(gpu_ctx, scene, tx, rxs, rough[:n], paths, K, iters, lanes)
             assert np.array_equal(log, choice[:n]), (n, lanes)
             for f in ("iters", "valid", "flags", "dir", "err", "delay"):
@@ -51,14 +54,17 @@ def test_lengths_alike(gpu_ctx, K, iters):
         h.close()
 
 
-def _time(ctx, scene, tx, rxs, rough, paths, K):
+def _time(ctx, scene, tx, rxs, rough, paths, K, lanes):
     best = np.inf
     for _ in range(5):
         ctx.paths_import(paths, rough, tx, rxs, 16)
         torch.cuda.synchronize()
         a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
         a.record()
-        ctx.batch_refine(scene, paths, 60, K)
+        if lanes:
+            ctx.batch_refine(scene, paths, 60, K, lanes_per_path=lanes)
+        else:
+            ctx.refine(scene, paths, 60, K)
         b.record()
         torch.cuda.synchronize()
         best = min(best, a.elapsed_time(b))
@@ -66,12 +72,15 @@ def _time(ctx, scene, tx, rxs, rough, paths, K):
 
 
 @pytest.mark.parametrize("K", [6, 16])
-def test_short_list_takes_no_longer(gpu_ctx, K):
+@pytest.mark.parametrize("form", ["batch", "plain"])
+def test_short_list_takes_no_longer(gpu_ctx, form, K):
     """900 and 4,000 paths against the whole list, run to the double floor.  (All lanes of a warp on the
-    same path and sub-ray: 900 paths 1.3 times as long as 10,000.)"""
+    same path and sub-ray: 900 paths 1.3 times as long as 10,000 in the batched form, 4,000 four times
+    in the plain one.)"""
     scene, tx, rxs, rough, paths = _rough(gpu_ctx, 150)
     assert len(rough) > 9000
-    whole, mid, short = (_time(gpu_ctx, scene, tx, rxs, rough[:n], paths, K) for n in (len(rough), 4000, 900))
+    lanes = 16 if form == "batch" else 0
+    whole, mid, short = (_time(gpu_ctx, scene, tx, rxs, rough[:n], paths, K, lanes) for n in (len(rough), 4000, 900))
     assert mid < 1.15 * whole and short < 1.15 * whole, (short, mid, whole)
     for h in (paths, rxs, scene):
         h.close()
