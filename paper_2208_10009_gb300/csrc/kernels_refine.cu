@@ -487,7 +487,9 @@ __device__ __forceinline__ int iterate32(const UnfF &uf, int nk, int K, int off,
 // key64's own rounding (of d_k and of the cross product) stays below 2e-15 |W|.  A sub-ray whose
 // |e_k| exceeds the smallest by more than 2 delta has the larger key64, valid or not, so only
 // the others are evaluated, exactly as before: one as a rule, more within about 1e-14 of the
-// double floor.  Should the smallest be invalid (a face met out of order), all K are.
+// double floor.  Should the smallest be invalid (a face met out of order), the next one left and
+// those that may win beside it follow: one such path in a warp of 32 would hold it for K evaluations
+// (a list of 4,031 paths, one iteration with K = 16: 96 -> 72 us).
 // Office tail (942,656 paths, K = 16): 935 -> 302 us, the FP64 pipe 71 % busy and still the bound; large
 // city (17.7k paths, 12 FP64 iterations, K = 9): 590 -> 387 us.
 struct Rank64 {   // |e_k|^2 of the sub-rays of one iteration
@@ -566,23 +568,35 @@ __device__ __forceinline__ int iterate64(const UnfD &ud, int nk, int K, int off,
             k1 = k;
         }
     }
-    const float thr = rank.limit(a1, samax);
-    unsigned left = 1u << k1;   // the sub-rays that may win
+    float thr = rank.limit(a1, samax);
+    unsigned left = 1u << k1, rest = (1u << K) - 1u;   // the sub-rays that may win; those not known to be invalid
     if (!(a2 > thr)) {
         rank.rho = -1.0f;
         for (int k = 0; k < K; ++k)
             if (!(rank(off + k) > thr)) left |= 1u << k;
     }
     for (;;) {
-        bool ok = false;
         for (; left; left &= left - 1) {
             const int k = __ffs(left) - 1;
-            const bool valid = best.try_ray(ud, nk, tab, off, k, R, c, u, v);
-            ok |= k == k1 && valid;
+            if (!best.try_ray(ud, nk, tab, off, k, R, c, u, v)) rest &= ~(1u << k);
         }
-        if (k1 < 0 || ok) break;
-        k1 = -1;   // the nearest is invalid, so the margin says nothing: take all
-        left = (1u << K) - 1u;
+        if ((rest >> k1 & 1u) || !rest) break;
+        // the nearest was invalid: the next one left, and those that may win beside it
+        a1 = INFINITY;
+        k1 = __ffs(rest) - 1;
+        rank.rho = -1.0f;
+        for (int k = 0; k < K; ++k) {
+            const float a = rank(off + k);
+            if ((rest >> k & 1u) && a < a1) {
+                a1 = a;
+                k1 = k;
+            }
+        }
+        thr = rank.limit(a1, samax);
+        rank.rho = -1.0f;
+        for (int k = 0; k < K; ++k)
+            if (!(rank(off + k) > thr)) left |= 1u << k;
+        left = (left | 1u << k1) & rest;
     }
     if (best.k >= K) return -1;
     c = best.d * (1.0 / dnorm(best.d));
@@ -596,7 +610,8 @@ __device__ __forceinline__ int iterate64(const UnfD &ud, int nk, int K, int off,
 // takes the sub-rays gl, gl + G, ...  With G >= K every sub-ray has a lane, and one exact evaluation a
 // lane costs what a single one does, so there is no ranking; with fewer lanes each ranks its own, and
 // only those that may win are evaluated, side by side (all lanes the same one where one is left; all K
-// should the nearest be invalid).  The winner's direction, key and d . W come from its lane by shuffles.  Near the double
+// should the nearest be invalid: ranking the others again took 25 % longer a call, in the lists that never
+// need it).  The winner's direction, key and d . W come from its lane by shuffles.  Near the double
 // floor, where the ranking cannot tell the sub-rays apart, a thread evaluates all K in turn and a
 // path's lanes K / G.
 __device__ __forceinline__ int iterate64_lanes(const UnfD &ud, int nk, int K, int off, const SubTab64 &tab, double R,
