@@ -206,7 +206,8 @@ typedef struct {
 #define SBR_LAUNCH_ID_ORDER 32 /* trace the rays in lattice id order.  By default a launch of
                                   the equiangular lattice takes them in compact tiles of
                                   each face's triangular grid (neighbouring directions together
-                                  in a warp); the results are the same either way (§III.A:
+                                  in a warp), a range of less than half of its faces' rays
+                                  excepted; the results are the same either way (§III.A:
                                   rays are independent) */
 
 typedef struct {

@@ -869,7 +869,6 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     a.ntx = ntx;
     a.ray_begin = (int)ray_begin;
     a.ray_end = (int)(ray_begin + ray_count);
-    a.id_order_n = prm->launcher == 0 && (prm->flags & SBR_LAUNCH_ID_ORDER) ? prm->n_div : 0;
     a.first = ray_begin;
     a.count = ray_count;
     int64_t place0 = ray_begin, places = ray_count;   // the places of dirs that hold the range's rays
@@ -881,6 +880,12 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
         const int64_t last = a.ray_end - 1;
         places = (last < E ? a.ray_end : E + ((last - E) / per + 1) * per) - place0;
     }
+    // Fewer ids than half of those places are taken in id order: passing over the others costs more than
+    // the tiles give.  Large city, n = 2200 (2.4M places a face), four transmitters, schedule / id order:
+    // 1,000 ids in one face 536 / 326 us, 600,000 560 / 444, 1.2M 626 / 573, 1.5M 644 / 645; 3M over two
+    // faces 1,273 / 1,470.
+    const bool narrow = 2 * ray_count < places;
+    a.id_order_n = prm->launcher == 0 && (narrow || (prm->flags & SBR_LAUNCH_ID_ORDER)) ? prm->n_div : 0;
     if (!a.id_order_n) {
         a.first = place0;
         a.count = places;
@@ -900,7 +905,7 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     a.refill_min = prm->refill_min > 0 ? std::min(prm->refill_min, 32) : 24;
     a.front = nullptr;
     a.group0 = a.groups = 0;
-    if (scene->dev.nnodes >= kFrontMinNodes && ntx * places >= kFrontMinRays && places > 0 &&
+    if (scene->dev.nnodes >= kFrontMinNodes && ntx * ray_count >= kFrontMinRays && !narrow &&
         scene->max_stack4 + kFrontEntries <= kStack4) {
         const int64_t group0 = place0 / kFrontRays, groups = (place0 + places + kFrontRays - 1) / kFrontRays - group0;
         const size_t need = (size_t)ntx * groups * kFrontEntries * sizeof(int2);
