@@ -197,6 +197,13 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) 
     return SBR_OK;
 }
 
+bool capturing(sbr_ctx *ctx) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(ctx->stream, &capture);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e != cudaSuccess || capture != cudaStreamCaptureStatusNone;
+}
+
 // The first segments' frontier (frontier_kernel) pays from about two million rays: it takes 45 us
 // of latency whatever their number, and saves 20 us of a trace of 0.9M rays (street receivers,
 // 10k triangles), 105 of 4.9M, 5.1 ms of 194M (1.07M triangles); and on trees worth skipping (a
@@ -214,11 +221,7 @@ void *front_room(sbr_ctx *ctx, sbr_paths *p, size_t need) {
     if (need > kFrontMaxBytes) return nullptr;
     const size_t have = p->front.empty() ? 0 : p->front.back().second;
     if (have >= need) return p->front.back().first;
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return nullptr;
-    }
+    if (capturing(ctx)) return nullptr;
     const size_t bytes = std::max(need, std::min(2 * have, kFrontMaxBytes));
     void *block = dev_alloc(ctx, bytes);
     if (block) p->front.push_back({block, bytes});
@@ -1236,7 +1239,14 @@ sbr_status sbr_batch_refine(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *pat
     if (lanes == 1) A.split_min = 0;   // the one-lane form runs with the unfold and FP64 tail kernels
     {
         Range r("sbr_batch_refine: unfold, iterations, FP64 tail, validity + outputs");
+        // order_cnt is left zero by a call's last kernel; one that never got there is made up for here.
+        // (A clear that is only captured has not run yet: the next call outside makes its own.)
+        if (paths->order_dirty)
+            SBR_CUDA(cudaMemsetAsync(paths->order_cnt, 0, kOrderCounts * sizeof(unsigned long long), ctx->stream));
+        const bool still = paths->order_dirty && capturing(ctx);
+        paths->order_dirty = true;
         SBR_CUDA(launch_batch_refine(A, ctx->num_sms * nb, block, ctx->stream));
+        paths->order_dirty = still;
     }
     return SBR_OK;
 }

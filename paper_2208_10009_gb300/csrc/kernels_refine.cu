@@ -10,6 +10,8 @@
 // traces each through the path's fixed face planes, evaluates Eq. 3 at Rx, keeps the
 // smallest (lowest k on ties) and shrinks R by the pattern's factor.  Iterations run in
 // FP32 while R >= fp64_below and in FP64 after that.
+#include <cstdlib>
+
 #include "dfloat.cuh"
 #include "nvtx_ranges.h"
 #include "sbr_device.cuh"
@@ -1734,34 +1736,41 @@ cudaError_t launch_batch_refine(const RefineArgs &a, int grid, int block, cudaSt
     static const int walk_blocks = resident(batch_walk_kernel, 128);
     static const int occ_blocks = resident(batch_occlusion_kernel, 128);
     const int sms = a.num_sms;
+    // SBR_CHECKED builds: the launch that SBR_CHECKED_FAIL_LAUNCH counts to (1 is the first) is not
+    // made and reports an error, as a failing driver call would
+    const char *fail = SBR_CHECKED_ON ? std::getenv("SBR_CHECKED_FAIL_LAUNCH") : nullptr;
+    int to_fail = fail ? std::atoi(fail) : 0;
+    auto run = [&](void (*kernel)(RefineArgs), int blocks, int threads) {
+        return --to_fail == 0 ? cudaErrorUnknown : launch_chained(kernel, blocks, threads, 0, s, a);
+    };
     // the two kernels of the many-path form (from split_min paths on) have nothing to do when the
     // container cannot hold that many (a room's call 225 -> 219 us)
     const bool many = a.path_cap >= a.split_min;
     cudaError_t e = cudaSuccess;
     if (many) {
         Range r("batch refine: plane unfolding");
-        e = launch_chained(batch_unfold_kernel, sms * unf_blocks, 128, 0, s, a);
+        e = run(batch_unfold_kernel, sms * unf_blocks, 128);
     }
     if (e != cudaSuccess) return e;
     {
         Range r("batch refine: iterations (work queue)");
         switch (a.chunk) {
-            case 1: e = launch_chained(batch_refine_kernel<1>, grid, block, 0, s, a); break;
-            case 8: e = launch_chained(batch_refine_kernel<8>, grid, block, 0, s, a); break;
-            case 32: e = launch_chained(batch_refine_kernel<32>, grid, block, 0, s, a); break;
-            default: e = launch_chained(batch_refine_kernel<16>, grid, block, 0, s, a); break;
+            case 1: e = run(batch_refine_kernel<1>, grid, block); break;
+            case 8: e = run(batch_refine_kernel<8>, grid, block); break;
+            case 32: e = run(batch_refine_kernel<32>, grid, block); break;
+            default: e = run(batch_refine_kernel<16>, grid, block); break;
         }
     }
     if (e != cudaSuccess) return e;
     {
         Range r("batch refine: FP64 tail");
-        e = launch_chained(batch_refine64_kernel, sms * tail_blocks, kTailBlock, 0, s, a);
+        e = run(batch_refine64_kernel, sms * tail_blocks, kTailBlock);
     }
     if (e != cudaSuccess) return e;
     {
         Range r("batch refine: validity + outputs");
-        if (many) e = launch_chained(batch_walk_kernel, sms * walk_blocks, 128, 0, s, a);
-        if (e == cudaSuccess) e = launch_chained(batch_occlusion_kernel, sms * occ_blocks, 128, 0, s, a);
+        if (many) e = run(batch_walk_kernel, sms * walk_blocks, 128);
+        if (e == cudaSuccess) e = run(batch_occlusion_kernel, sms * occ_blocks, 128);
     }
     return e;
 }

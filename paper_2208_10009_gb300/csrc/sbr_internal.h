@@ -217,6 +217,7 @@ struct sbr_paths {
                                                // 62: queue head, 63: blocks that have read them; [64, 74)
                                                // paths per group with legs to test.  Zero between calls
                                                // (the last kernel of a call clears them)
+    bool order_dirty = false;              // order_cnt may not be zero: a call's launches failed half way
     int *fp64_idx = nullptr;               // batched refinement: paths handed to the FP64 tail
     unsigned long long *table = nullptr;   // dedup hash table: 2 x u64 per slot (key, value)
     int64_t table_slots = 0;
