@@ -20,6 +20,11 @@
  *   - Device memory owned by handles is obtained through the context's allocator
  *     callbacks (or cudaMallocAsync when none are given) and released by the matching
  *     destroy call.
+ *   - Launches of a context share its ray directions, so its calls (graph replays included)
+ *     run one after the other, except launches of one division level and launcher into
+ *     different containers, which may overlap.  What captured calls use stays as it is until
+ *     its handle is destroyed: later calls that need larger blocks, or directions of another
+ *     division level, get blocks of their own.
  *   - Coordinates are metres in a right-handed frame; angles are radians; azimuth =
  *     atan2(y, x) in (-pi, pi], elevation = atan2(z, hypot(x, y)).
  *   - A "face" is a planar polygon given as triangles sharing a face id; path face

@@ -96,8 +96,33 @@ float bits_as_float(int i) {
     return f;
 }
 
+bool capturing(sbr_ctx *ctx) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(ctx->stream, &capture);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e != cudaSuccess || capture != cudaStreamCaptureStatusNone;
+}
+
 sbr_status ensure_lattice(sbr_ctx *ctx, int n) {
     if (ctx->lattice_n == n && ctx->lattice_mem) return SBR_OK;
+    if (ctx->lattice_held) {   // a captured launch's tables stay as they are
+        ctx->held_lattices.push_back({ctx->lattice_mem, ctx->lattice_bytes, ctx->lattice});
+        ctx->lattice_mem = nullptr;
+        ctx->lattice_bytes = 0;
+        ctx->lattice_held = false;
+    }
+    for (size_t i = 0; i < ctx->held_lattices.size(); ++i) {
+        const sbr_ctx::HeldLattice h = ctx->held_lattices[i];
+        if (h.tables.n != n) continue;
+        dev_free(ctx, ctx->lattice_mem, ctx->lattice_bytes);
+        ctx->held_lattices.erase(ctx->held_lattices.begin() + i);
+        ctx->lattice_mem = h.mem;
+        ctx->lattice_bytes = h.bytes;
+        ctx->lattice = h.tables;
+        ctx->lattice_n = n;
+        ctx->lattice_held = true;
+        return SBR_OK;
+    }
     std::vector<float4> ico, centre, layers;
     std::vector<int2> edges;
     int nl = 0;
@@ -109,6 +134,7 @@ sbr_status ensure_lattice(sbr_ctx *ctx, int n) {
     cv.add(&d_edges, edges.size());
     cv.add(&d_centre, centre.size());
     cv.add(&d_layers, layers.size());
+    ctx->lattice_n = 0;   // until the tables are there
     if (ctx->lattice_bytes < cv.total) {
         dev_free(ctx, ctx->lattice_mem, ctx->lattice_bytes);
         ctx->lattice_mem = dev_alloc(ctx, cv.total);
@@ -136,7 +162,9 @@ sbr_status ensure_lattice(sbr_ctx *ctx, int n) {
 }
 
 sbr_status ensure_poly(sbr_ctx *ctx, int poly, int n) {
-    if (ctx->poly_kind != poly || !ctx->poly_mem) {
+    const int slot = poly == 20;
+    PolyDev &P = ctx->poly[slot];
+    if (!ctx->poly_mem[slot]) {
         std::vector<float4> v;
         std::vector<int2> e;
         std::vector<int4> f;
@@ -148,26 +176,27 @@ sbr_status ensure_poly(sbr_ctx *ctx, int poly, int n) {
         cv.add(&dv, v.size());
         cv.add(&de, e.size());
         cv.add(&df, f.size());
-        if (ctx->poly_bytes < cv.total) {
-            dev_free(ctx, ctx->poly_mem, ctx->poly_bytes);
-            ctx->poly_mem = dev_alloc(ctx, cv.total);
-            ctx->poly_bytes = ctx->poly_mem ? cv.total : 0;
-            if (!ctx->poly_mem) return fail(ctx, SBR_ENOMEM, "equidistant tables: allocation failed");
-        }
-        cv.bind(ctx->poly_mem);
-        SBR_CUDA(cudaMemcpyAsync(dv, v.data(), v.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
-        SBR_CUDA(cudaMemcpyAsync(de, e.data(), e.size() * sizeof(int2), cudaMemcpyHostToDevice, ctx->stream));
-        SBR_CUDA(cudaMemcpyAsync(df, f.data(), f.size() * sizeof(int4), cudaMemcpyHostToDevice, ctx->stream));
-        SBR_CUDA(cudaStreamSynchronize(ctx->stream));
-        ctx->poly.v = dv;
-        ctx->poly.edges = de;
-        ctx->poly.faces = df;
-        ctx->poly.nv = (int)v.size();
-        ctx->poly.ne = (int)e.size();
-        ctx->poly.nf = (int)f.size();
-        ctx->poly_kind = poly;
+        void *mem = dev_alloc(ctx, cv.total);
+        if (!mem) return fail(ctx, SBR_ENOMEM, "equidistant tables: allocation failed");
+        cv.bind(mem);
+        cudaError_t err = cudaMemcpyAsync(dv, v.data(), v.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream);
+        if (err == cudaSuccess)
+            err = cudaMemcpyAsync(de, e.data(), e.size() * sizeof(int2), cudaMemcpyHostToDevice, ctx->stream);
+        if (err == cudaSuccess)
+            err = cudaMemcpyAsync(df, f.data(), f.size() * sizeof(int4), cudaMemcpyHostToDevice, ctx->stream);
+        if (err == cudaSuccess) err = cudaStreamSynchronize(ctx->stream);
+        if (err != cudaSuccess) dev_free(ctx, mem, cv.total);
+        SBR_CUDA(err);
+        ctx->poly_mem[slot] = mem;
+        ctx->poly_bytes[slot] = cv.total;
+        P.v = dv;
+        P.edges = de;
+        P.faces = df;
+        P.nv = (int)v.size();
+        P.ne = (int)e.size();
+        P.nf = (int)f.size();
     }
-    ctx->poly.n = n;
+    P.n = n;
     return SBR_OK;
 }
 
@@ -175,6 +204,26 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) 
     int64_t N = rays_for_launcher(n, launcher);
     if (N < 0) return fail(ctx, SBR_EINVAL, "launcher must be 0 (equiangular), 20 or 8 (equidistant)");
     size_t need = (size_t)N * sizeof(float4);
+    if (ctx->dirs_n != n || ctx->dirs_launcher != launcher) {
+        if (ctx->dirs_held) {   // replays of a captured launch write their own directions there
+            ctx->held_dirs.push_back({ctx->dirs, ctx->dirs_bytes, ctx->dirs_n, ctx->dirs_launcher});
+            ctx->dirs = nullptr;
+            ctx->dirs_bytes = 0;
+            ctx->dirs_held = ctx->dirs_valid = false;
+        }
+        for (size_t i = 0; i < ctx->held_dirs.size(); ++i) {
+            const sbr_ctx::HeldDirs h = ctx->held_dirs[i];
+            if (h.n != n || h.launcher != launcher) continue;
+            dev_free(ctx, ctx->dirs, ctx->dirs_bytes);
+            ctx->held_dirs.erase(ctx->held_dirs.begin() + i);
+            ctx->dirs = h.mem;
+            ctx->dirs_bytes = h.bytes;
+            ctx->dirs_n = n;
+            ctx->dirs_launcher = launcher;
+            ctx->dirs_held = true;
+            break;
+        }
+    }
     if (ctx->dirs_bytes < need) {
         dev_free(ctx, ctx->dirs, ctx->dirs_bytes);
         ctx->dirs = dev_alloc(ctx, need);
@@ -189,19 +238,17 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) 
     } else {
         sbr_status st = ensure_poly(ctx, launcher, n);
         if (st != SBR_OK) return st;
-        SBR_CUDA(launch_raygen_equidistant(ctx->poly, static_cast<float4 *>(ctx->dirs), N, true, prep, ctx->stream));
+        SBR_CUDA(launch_raygen_equidistant(ctx->poly[launcher == 20], static_cast<float4 *>(ctx->dirs), N, true, prep,
+                                           ctx->stream));
     }
     ctx->dirs_n = n;
     ctx->dirs_launcher = launcher;
     ctx->dirs_valid = true;
+    if (capturing(ctx)) {
+        ctx->dirs_held = true;
+        if (launcher == 0) ctx->lattice_held = true;
+    }
     return SBR_OK;
-}
-
-bool capturing(sbr_ctx *ctx) {
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    const cudaError_t e = cudaStreamIsCapturing(ctx->stream, &capture);
-    if (e != cudaSuccess) cudaGetLastError();
-    return e != cudaSuccess || capture != cudaStreamCaptureStatusNone;
 }
 
 // The first segments' frontier (frontier_kernel) pays from about two million rays: it takes 45 us
@@ -212,8 +259,9 @@ bool capturing(sbr_ctx *ctx) {
 constexpr int64_t kFrontMinRays = 3000000, kFrontMinNodes = 1024;
 constexpr size_t kFrontMaxBytes = (size_t)4 << 30;
 
-// The container's room for a frontier of `need` bytes, or null (the walks start at the root).  What a
-// launch writes belongs to its container, so that launches into other containers may overlap it.  A
+// The container's room for a frontier of `need` bytes, or null (the walks start at the root).  The lists
+// belong to the container, so launches of one division level and launcher into different containers
+// may overlap (the directions, which they share, are then written with the same values).  A
 // block outgrown stays until the container goes, since a captured launch may hold its address; sizes
 // at least double, so all of them together take at most twice the largest.  No room is made while the
 // stream captures: memory from inside a capture would live and die with the graph.
@@ -303,7 +351,8 @@ sbr_status sbr_raygen_equidistant(sbr_ctx *ctx, int32_t n, int32_t poly, float *
     DeviceGuard g(ctx->device);
     sbr_status st = ensure_poly(ctx, poly, n);
     if (st != SBR_OK) return st;
-    SBR_CUDA(launch_raygen_equidistant(ctx->poly, reinterpret_cast<float4 *>(dirs), N, false, PrepArgs(), ctx->stream));
+    SBR_CUDA(launch_raygen_equidistant(ctx->poly[poly == 20], reinterpret_cast<float4 *>(dirs), N, false, PrepArgs(),
+                                       ctx->stream));
     return SBR_OK;
 }
 
@@ -349,7 +398,9 @@ sbr_status sbr_ctx_destroy(sbr_ctx *ctx) {
     DeviceGuard g(ctx->device);
     dev_free(ctx, ctx->dirs, ctx->dirs_bytes);
     dev_free(ctx, ctx->lattice_mem, ctx->lattice_bytes);
-    dev_free(ctx, ctx->poly_mem, ctx->poly_bytes);
+    for (int i = 0; i < 2; ++i) dev_free(ctx, ctx->poly_mem[i], ctx->poly_bytes[i]);
+    for (auto &h : ctx->held_dirs) dev_free(ctx, h.mem, h.bytes);
+    for (auto &h : ctx->held_lattices) dev_free(ctx, h.mem, h.bytes);
     cudaStreamSynchronize(ctx->stream);
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
@@ -779,15 +830,23 @@ sbr_status sbr_paths_destroy(sbr_ctx *ctx, sbr_paths *p) {
     dev_free(ctx, p->mem, p->bytes);
     dev_free(ctx, p->tx_mem, p->tx_bytes);
     dev_free(ctx, p->pair_mem, p->pair_bytes);
+    for (auto &b : p->held) dev_free(ctx, b.first, b.second);
     for (auto &b : p->front) dev_free(ctx, b.first, b.second);
     delete p;
     return SBR_OK;
 }
 
+// The end of a container's block that a larger one replaces: kept if a captured call uses it.
+static void outgrown(sbr_ctx *ctx, sbr_paths *p, void *mem, size_t bytes, bool &held) {
+    if (held) p->held.push_back({mem, bytes});
+    else dev_free(ctx, mem, bytes);
+    held = false;
+}
+
 // room for ntx transmitters, and a copy of them (tx null: the room only)
 static sbr_status ensure_tx(sbr_ctx *ctx, sbr_paths *p, const float *tx, int32_t ntx) {
     if (ntx > p->tx_cap) {
-        dev_free(ctx, p->tx_mem, p->tx_bytes);
+        outgrown(ctx, p, p->tx_mem, p->tx_bytes, p->tx_held);
         size_t b = (size_t)ntx * sizeof(float4);
         p->tx_mem = dev_alloc(ctx, b);
         p->tx_bytes = p->tx_mem ? b : 0;
@@ -848,6 +907,7 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     const bool tx_on_device = is_local_ptr(ctx, tx);
     sbr_status st = ensure_tx(ctx, paths, tx_on_device ? nullptr : tx, ntx);
     if (st != SBR_OK) return st;
+    if (capturing(ctx)) paths->tx_held = true;
     if (tx_on_device) {
         prep.tx_src = tx;
         prep.tx = paths->tx;
@@ -1081,6 +1141,7 @@ sbr_status sbr_records_dedup(sbr_ctx *ctx, sbr_paths *paths, const sbr_reception
         sbr_status st = ensure_dirs(ctx, paths->n_div, paths->launcher, PrepArgs());   // rough launch directions
         if (st != SBR_OK) return st;
     }
+    if (capturing(ctx)) ctx->dirs_held = true;
     if (count > 0) {
         cudaMemcpyKind kind = is_device_ptr(in) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
         SBR_CUDA(cudaMemcpyAsync(paths->recs, in, (size_t)count * sizeof(RecDev), kind, ctx->stream));
@@ -1105,6 +1166,7 @@ static sbr_status refine_args(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *p
         return fail(ctx, SBR_EINVAL, "refine: subrays must be 6, 7, 9 or 16");
     if (prm->max_iters < 0 || prm->max_iters > 200) return fail(ctx, SBR_EINVAL, "refine: max_iters out of [0, 200]");
     if (!paths->rx || paths->ntx < 1) return fail(ctx, SBR_EINVAL, "refine: container holds no launch");
+    if (capturing(ctx)) paths->tx_held = true;
     A.scene = scene->dev;
     A.scene.status = reinterpret_cast<unsigned long long *>(paths->counters + kErrorFlags);
     A.tx = paths->tx;
@@ -1181,7 +1243,7 @@ sbr_status sbr_refine_pair(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *path
     if (paths->pair_cap != paths->path_cap) {
         size_t need = sizeof(int) * ((size_t)npairs + 1 + (size_t)paths->path_cap + (size_t)npairs);
         if (paths->pair_bytes < need) {
-            dev_free(ctx, paths->pair_mem, paths->pair_bytes);
+            outgrown(ctx, paths, paths->pair_mem, paths->pair_bytes, paths->pair_held);
             paths->pair_mem = dev_alloc(ctx, need);
             paths->pair_bytes = paths->pair_mem ? need : 0;
             if (!paths->pair_mem) return fail(ctx, SBR_ENOMEM, "sbr_refine_pair: allocation failed");
@@ -1204,6 +1266,7 @@ sbr_status sbr_refine_pair(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *path
         SBR_CUDA(cudaStreamSynchronize(ctx->stream));
         paths->pair_cap = paths->path_cap;
     }
+    if (capturing(ctx)) paths->pair_held = true;
     int p = tx * paths->nrx + rx;
     int count = paths->pair_host[p + 1] - paths->pair_host[p];
     if (count <= 0) return SBR_OK;

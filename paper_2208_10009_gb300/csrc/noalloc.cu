@@ -198,6 +198,7 @@ extern "C" sbr_status sbr_dedup_noalloc(sbr_ctx *ctx, const sbr_paths *src, sbr_
             cudaGetLastError();
             cs = cudaStreamCaptureStatusNone;
         }
+        if (cs != cudaStreamCaptureStatusNone) ctx->dirs_held = true;   // read again by the replays
         std::lock_guard<std::mutex> lk(g_mu);
         if (!g_addr[ctx->device] || cs == cudaStreamCaptureStatusNone) {
             cudaError_t e = cudaGetSymbolAddress(&g_addr[ctx->device], g_dedup_scratch);

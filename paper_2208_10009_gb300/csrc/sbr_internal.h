@@ -163,6 +163,22 @@ struct sbr_ctx {
     std::string last_error;
     int num_sms = 0;
     int max_threads_per_sm = 0;
+    // Blocks that captured launches use (the flags: the current one is such a block).  A replay writes
+    // and reads them again, so they are neither freed nor given other contents before the context goes;
+    // a launch at the same division level takes them up again, so there is one at most for each.
+    struct HeldDirs {
+        void *mem;
+        size_t bytes;
+        int n, launcher;
+    };
+    struct HeldLattice {
+        void *mem;
+        size_t bytes;
+        sbr::LatticeDev tables;
+    };
+    std::vector<HeldDirs> held_dirs;
+    std::vector<HeldLattice> held_lattices;
+    bool dirs_held = false, lattice_held = false;
     // ray-generation workspace (directions of the last division level: the equiangular
     // lattice's at their places of the schedule, an equidistant launcher's at their ray ids;
     // the ray id's bits in w)
@@ -176,11 +192,10 @@ struct sbr_ctx {
     int lattice_n = 0;
     sbr::LatticeDev lattice{};
     int dirs_launcher = 0;
-    // equidistant launcher tables
-    void *poly_mem = nullptr;
-    size_t poly_bytes = 0;
-    int poly_kind = 0;
-    sbr::PolyDev poly{};
+    // equidistant launcher tables: octahedron, icosahedron (made once)
+    void *poly_mem[2] = {nullptr, nullptr};
+    size_t poly_bytes[2] = {0, 0};
+    sbr::PolyDev poly[2]{};
     // resident blocks per SM, looked up once: trace kernel by block size / 32, batched refinement
     // by lanes (1, 8, 16, 32) and block size / 32
     int trace_nb[5] = {0}, refine_nb = 0, batch_nb[4][9] = {{0}};
@@ -234,6 +249,9 @@ struct sbr_paths {
     size_t tx_bytes = 0;
     int32_t ntx = 0, nrx = 0, n_div = 0, max_order = 0, launcher = 0;
     const sbr_rxset *rx = nullptr;
+    // transmitter and pair blocks that captured calls use, outgrown since (the flags: the current ones)
+    std::vector<std::pair<void *, size_t>> held;
+    bool tx_held = false, pair_held = false;
     // first segments' frontier: blocks of growing size, the last in use (front_room in capi.cu)
     std::vector<std::pair<void *, size_t>> front;
     float alpha = 1.0f;
