@@ -169,8 +169,9 @@ sbr_status sbr_rx_destroy(sbr_ctx *ctx, sbr_rxset *rx);
 /* Device container for reception records and paths.  record_cap bounds the records one
  * launch may emit (before double-count removal), path_cap the unique paths.  A launch of three
  * million rays and more on a scene of 1,024 nodes and more adds room for the entries its first
- * segments start from (about a byte per ray, at most 4 GB, kept until sbr_paths_destroy; none is
- * made while the stream captures, and where there is none the segments start at the root). */
+ * segments start from (about a byte per ray, at most 4 GB, kept for the largest such launch until
+ * sbr_paths_destroy; a launch that needs more, one that finds no memory for it, and one whose stream
+ * captures with too little room start at the root). */
 sbr_status sbr_paths_create(sbr_ctx *ctx, int64_t record_cap, int64_t path_cap, sbr_paths **out);
 sbr_status sbr_paths_destroy(sbr_ctx *ctx, sbr_paths *paths);
 

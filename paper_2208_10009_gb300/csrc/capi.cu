@@ -251,6 +251,13 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) 
     return SBR_OK;
 }
 
+// The end of a container's block that a larger one replaces: kept if a captured call uses it.
+void outgrown(sbr_ctx *ctx, sbr_paths *p, void *mem, size_t bytes, bool &held) {
+    if (held) p->held.push_back({mem, bytes});
+    else dev_free(ctx, mem, bytes);
+    held = false;
+}
+
 // The first segments' frontier (frontier_kernel) pays from about two million rays: it takes 45 us
 // of latency whatever their number, and saves 20 us of a trace of 0.9M rays (street receivers,
 // 10k triangles), 105 of 4.9M, 5.1 ms of 194M (1.07M triangles); and on trees worth skipping (a
@@ -261,19 +268,19 @@ constexpr size_t kFrontMaxBytes = (size_t)4 << 30;
 
 // The container's room for a frontier of `need` bytes, or null (the walks start at the root).  The lists
 // belong to the container, so launches of one division level and launcher into different containers
-// may overlap (the directions, which they share, are then written with the same values).  A
-// block outgrown stays until the container goes, since a captured launch may hold its address; sizes
-// at least double, so all of them together take at most twice the largest.  No room is made while the
-// stream captures: memory from inside a capture would live and die with the graph.
+// may overlap (the directions, which they share, are then written with the same values).  No room is
+// made while the stream captures: memory from inside a capture would live and die with the graph.
 void *front_room(sbr_ctx *ctx, sbr_paths *p, size_t need) {
     if (need > kFrontMaxBytes) return nullptr;
-    const size_t have = p->front.empty() ? 0 : p->front.back().second;
-    if (have >= need) return p->front.back().first;
-    if (capturing(ctx)) return nullptr;
-    const size_t bytes = std::max(need, std::min(2 * have, kFrontMaxBytes));
-    void *block = dev_alloc(ctx, bytes);
-    if (block) p->front.push_back({block, bytes});
-    return block;
+    const bool capture = capturing(ctx);
+    if (p->front_bytes < need) {
+        if (capture) return nullptr;
+        outgrown(ctx, p, p->front, p->front_bytes, p->front_held);
+        p->front = dev_alloc(ctx, need);
+        p->front_bytes = p->front ? need : 0;
+    }
+    p->front_held |= capture && p->front;
+    return p->front;
 }
 
 // a value looked up once (0: not yet)
@@ -831,16 +838,9 @@ sbr_status sbr_paths_destroy(sbr_ctx *ctx, sbr_paths *p) {
     dev_free(ctx, p->tx_mem, p->tx_bytes);
     dev_free(ctx, p->pair_mem, p->pair_bytes);
     for (auto &b : p->held) dev_free(ctx, b.first, b.second);
-    for (auto &b : p->front) dev_free(ctx, b.first, b.second);
+    dev_free(ctx, p->front, p->front_bytes);
     delete p;
     return SBR_OK;
-}
-
-// The end of a container's block that a larger one replaces: kept if a captured call uses it.
-static void outgrown(sbr_ctx *ctx, sbr_paths *p, void *mem, size_t bytes, bool &held) {
-    if (held) p->held.push_back({mem, bytes});
-    else dev_free(ctx, mem, bytes);
-    held = false;
 }
 
 // room for ntx transmitters, and a copy of them (tx null: the room only)

@@ -249,11 +249,13 @@ struct sbr_paths {
     size_t tx_bytes = 0;
     int32_t ntx = 0, nrx = 0, n_div = 0, max_order = 0, launcher = 0;
     const sbr_rxset *rx = nullptr;
-    // transmitter and pair blocks that captured calls use, outgrown since (the flags: the current ones)
+    // first segments' frontier (front_room in capi.cu)
+    void *front = nullptr;
+    size_t front_bytes = 0;
+    // transmitter, pair and frontier blocks that captured calls use, outgrown since (the flags: the
+    // current ones)
     std::vector<std::pair<void *, size_t>> held;
-    bool tx_held = false, pair_held = false;
-    // first segments' frontier: blocks of growing size, the last in use (front_room in capi.cu)
-    std::vector<std::pair<void *, size_t>> front;
+    bool tx_held = false, pair_held = false, front_held = false;
     float alpha = 1.0f;
     int64_t ray_begin = 0, ray_count = 0;  // ray ids traced per transmitter by the last launch
     bool timed = false;                    // last launch recorded kernel events
