@@ -161,7 +161,8 @@ sbr_status sbr_scene_wedges(const sbr_scene *scene, float *ab, int32_t *faces, i
 /* ---------------------------------------------------------------- receivers */
 /* Upload nrx receiver positions (host, nrx x 3 floats) and build their BVH (used by the
  * reception judgment to find candidate Rx near a ray segment): on the device for 64 to
- * 131,072 receivers, with 96 bytes per receiver of device memory held during the call. */
+ * 131,072 receivers, with 96 bytes per receiver of device memory held during the call (on the host,
+ * slower, where that cannot be had). */
 sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset **out);
 sbr_status sbr_rx_destroy(sbr_ctx *ctx, sbr_rxset *rx);
 

@@ -719,8 +719,12 @@ sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset *
     // the host less than the launches, and beyond the upper one the device's ranks by counting (n^2
     // comparisons) overtake the host's search.  Whole call, host -> device: 1 receiver 18 -> 23 us,
     // 64 37 -> 35, 256 99 -> 51, 1,024 343 -> 67, 4,096 910 -> 111, 16,384 3,440 -> 476, 65,536
-    // 13,500 -> 4,490, 131,072 27,200 -> 16,300, 262,144 both 57,000.
-    const bool on_device = nrx >= kRxDeviceMin && nrx <= kRxDeviceMax;
+    // 13,500 -> 4,490, 131,072 27,200 -> 16,300, 262,144 both 57,000.  The host also builds it where
+    // there is no device memory for the other way's scratch.
+    bool on_device = nrx >= kRxDeviceMin && nrx <= kRxDeviceMax;
+    const size_t scratch_bytes = on_device ? (size_t)rx_tree_scratch(nrx) * sizeof(float4) : 0;
+    float4 *scratch = scratch_bytes ? static_cast<float4 *>(dev_alloc(ctx, scratch_bytes)) : nullptr;
+    if (scratch_bytes && !scratch) on_device = false;
     BvhOut bvh;
     std::string err;
     if (!on_device) {
@@ -730,7 +734,10 @@ sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset *
     const size_t room = (size_t)std::max(nrx, 1);
     std::vector<float4> by_id(room), pts(on_device ? 0 : room);
     sbr_rxset *rs = new (std::nothrow) sbr_rxset();
-    if (!rs) return fail(ctx, SBR_ENOMEM, "rx: host allocation failed");
+    if (!rs) {
+        dev_free(ctx, scratch, scratch_bytes);
+        return fail(ctx, SBR_ENOMEM, "rx: host allocation failed");
+    }
     for (int a = 0; a < 3; ++a) {
         rs->dev.lo[a] = INFINITY;
         rs->dev.hi[a] = -INFINITY;
@@ -752,29 +759,27 @@ sbr_status sbr_rx_upload(sbr_ctx *ctx, const float *rx, int32_t nrx, sbr_rxset *
     cv.add(&d_by, room);
     rs->mem = dev_alloc(ctx, cv.total);
     if (!rs->mem) {
+        dev_free(ctx, scratch, scratch_bytes);
         delete rs;
         return fail(ctx, SBR_ENOMEM, "rx: device allocation failed");
     }
     rs->bytes = cv.total;
     cv.bind(rs->mem);
-    SBR_CUDA(cudaMemcpyAsync(d_by, by_id.data(), by_id.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
-    if (on_device) {
-        const size_t bytes = (size_t)rx_tree_scratch(nrx) * sizeof(float4);
-        float4 *scratch = bytes ? static_cast<float4 *>(dev_alloc(ctx, bytes)) : nullptr;
-        if (bytes && !scratch) {
-            dev_free(ctx, rs->mem, rs->bytes);
-            delete rs;
-            return fail(ctx, SBR_ENOMEM, "rx: device allocation failed");
-        }
-        cudaError_t e = launch_rx_tree(d_by, nrx, d_pts, scratch, d_nodes4, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        dev_free(ctx, scratch, bytes);
+    cudaError_t e = cudaMemcpyAsync(d_by, by_id.data(), by_id.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess && on_device) {
+        e = launch_rx_tree(d_by, nrx, d_pts, scratch, d_nodes4, ctx->stream);
+    } else if (e == cudaSuccess) {
+        e = cudaMemcpyAsync(d_nodes4, bvh.nodes4.data(), bvh.nodes4.size() * sizeof(float4), cudaMemcpyHostToDevice,
+                            ctx->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(d_pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    dev_free(ctx, scratch, scratch_bytes);
+    if (e != cudaSuccess) {
+        dev_free(ctx, rs->mem, rs->bytes);
+        delete rs;
         SBR_CUDA(e);
-    } else {
-        SBR_CUDA(cudaMemcpyAsync(d_nodes4, bvh.nodes4.data(), bvh.nodes4.size() * sizeof(float4),
-                                 cudaMemcpyHostToDevice, ctx->stream));
-        SBR_CUDA(cudaMemcpyAsync(d_pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
-        SBR_CUDA(cudaStreamSynchronize(ctx->stream));
     }
     rs->dev.nodes4 = d_nodes4;
     rs->dev.pts = d_pts;
