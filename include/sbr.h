@@ -260,6 +260,7 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
 #define SBR_CHECK_RX_STACK 4         /* receiver walk of the reception judgment */
 #define SBR_CHECK_FACE_ID 8          /* a face id outside [0, num_faces) met on the device */
 #define SBR_CHECK_BVH2_STACK 16      /* binary-BVH walks (point in face, wedge search) */
+#define SBR_CHECK_RX_FILTER 32       /* a diffraction reception that the filter before its test let go */
 
 /* Synchronises the stream and reads the counters of the container's last launch. */
 sbr_status sbr_launch_get_stats(sbr_ctx *ctx, const sbr_paths *paths, sbr_launch_stats *out);

@@ -1101,9 +1101,10 @@ sbr_status sbr_launch_get_stats(sbr_ctx *ctx, const sbr_paths *paths, sbr_launch
 // SBR_ECHECK with the failed checks named, when a container's status word has bits set
 static sbr_status report_checks(sbr_ctx *ctx, long long flags, const char *where) {
     if (!flags) return SBR_OK;
-    static const char *names[] = {"trace stack", "occlusion stack", "receiver stack", "face id", "binary-BVH stack"};
+    static const char *names[] = {"trace stack", "occlusion stack", "receiver stack", "face id", "binary-BVH stack",
+                                  "diffraction receiver filter"};
     std::string m = std::string(where) + ": device bounds checks failed:";
-    for (int b = 0; b < 5; ++b)
+    for (int b = 0; b < 6; ++b)
         if (flags & (1LL << b)) m += std::string(" ") + names[b];
     return fail(ctx, SBR_ECHECK, m);
 }

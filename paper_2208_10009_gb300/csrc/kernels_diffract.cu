@@ -486,7 +486,12 @@ __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
         const float3 a0 = w.a - o;
         const float t2 = A.tan_cone * A.tan_cone * 1.0001f;   // pre-test, the exact test follows
         // the same test in the edge's frame, as a conservative filter: W = A e - B b1 with A = z -
-        // z_Tx, B = rho + rho_Tx, so |d x W|^2 = (d_e B + d_b1 A)^2 + d_b2^2 |W|^2
+        // z_Tx, B = rho + rho_Tx, so |d x W|^2 = (d_e B + d_b1 A)^2 + d_b2^2 |W|^2.  Beside 1 % of the cone it
+        // allows for FP32: b1 is off by up to 2e-7 |Tx - a| / rho_Tx (Tx close to the edge's line), A by
+        // 2e-7 (|z| + |z_Tx|), and both enter times |A| + B at most.  (With 2e-6 (|A| + B) alone, receptions
+        // within a metre of the line were lost, 1 in 700 at 1 km from the origin and 2 mrad; with twice these
+        // bounds none of 1.7e7 is.)
+        const float off = 2e-6f + 1e-6f * sqrtf(dot(a0, a0)) / rt, off_z = 1e-6f * fabsf(dot(a0, e));
         const float de = dot(d, e), db = dot(d, b1), dn2 = dot(d, b2) * dot(d, b2), ze = dot(o - w.a, e);
         const float tc = A.tan_cone * 1.01f;
         for (int rx = lane; rx < A.rx.nrx; rx += 32) {
@@ -496,8 +501,9 @@ __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
             float rho;
             asm("sqrt.approx.f32 %0, %1;" : "=f"(rho) : "f"(x * x + y * y));
             const float fa = z - ze, fb = rho + rt, u = fmaf(de, fb, db * fa);
-            const float lim = fmaf(fabsf(fmaf(de, fa, -db * fb)), tc, 2e-6f * (fabsf(fa) + fb));
-            if (fmaf(u, u, dn2 * fmaf(fa, fa, fb * fb)) > lim * lim) continue;
+            const float lim = fmaf(fabsf(fmaf(de, fa, -db * fb)), tc, fmaf(off, fabsf(fa) + fb, off_z));
+            const bool far = fmaf(u, u, dn2 * fmaf(fa, fa, fb * fb)) > lim * lim;
+            if (far && !SBR_CHECKED_ON) continue;
             const float c1 = w1x * y - w1y * x, c2 = x * w2y - y * w2x;
             if (c1 * s12 > 0.0f && c2 * s12 > 0.0f) continue;   // Rx inside the solid's sector
             const float3 W = a0 + e * z - b1 * sqrtf(x * x + y * y);
@@ -506,6 +512,10 @@ __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
             if (!(dw > 0.0f) || cc > dw * dw * t2) continue;
             const float err = atan2f(sqrtf(cc), dw);
             if (!(err <= A.cone)) continue;
+            if (far) {   // SBR_CHECKED builds: the filter let go of a reception
+                check_fail(S, SBR_CHECK_RX_FILTER);
+                continue;
+            }
             // the segment X -> Rx is tested by diffract_occlusion, a query per thread in
             // full warps (here it would run in one lane while the warp waits); the
             // reception is parked with X in its unused face slots 1-3
