@@ -300,7 +300,7 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
     const float gx = rad * aix, gy = rad * aiy, gz = rad * aiz;
     const float cnx = oix + gx, cny = oiy + gy, cnz = oiz + gz;
     const float cfx = oix - gx, cfy = oiy - gy, cfz = oiz - gz;
-    const float tfar = tcap * 1.0000005f + 1e-6f;
+    const float tfar = tcap * kSlabMargin + 1e-6f;
     {
         // the receivers' bounding box, grown like the node boxes: one slab test before the
         // walk (most segments, e.g. those rising above every receiver, end here; 2-3 %
@@ -311,7 +311,7 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
         const float nz = bz ? R.hi[2] : R.lo[2], fz = bz ? R.lo[2] : R.hi[2];
         const float tn = max3f(fmaf(nx, r.inv.x, -cnx), fmaf(ny, r.inv.y, -cny), fmaxf(fmaf(nz, r.inv.z, -cnz), 0.0f));
         const float tf = min3f(fmaf(fx, r.inv.x, -cfx), fmaf(fy, r.inv.y, -cfy), fminf(fmaf(fz, r.inv.z, -cfz), tfar));
-        if (!(tn <= tf * 1.0000005f)) return;
+        if (!(tn <= tf * kSlabMargin)) return;
     }
     int stack[kStack4];
     int sp = 0;
@@ -332,7 +332,7 @@ __device__ __forceinline__ void reception(const TraceArgs &a, const RayPre &r, c
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 float tn = max3f(sx.n[c], sy.n[c], fmaxf(sz.n[c], 0.0f));
-                float tf = min3f(sx.f[c], sy.f[c], fminf(sz.f[c], tfar)) * 1.0000005f;
+                float tf = min3f(sx.f[c], sy.f[c], fminf(sz.f[c], tfar)) * kSlabMargin;
                 if (tn <= tf) {
                     if (next == 0x7fffffff) next = rf[c];
                     else stack[sp++] = rf[c];
