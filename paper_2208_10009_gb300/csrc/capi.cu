@@ -1075,6 +1075,9 @@ sbr_status sbr_launch_get_stats(sbr_ctx *ctx, const sbr_paths *paths, sbr_launch
     out->tri_tests = c[kTriTests];
     out->rx_tests = c[kRxTests];
     out->records = c[kRecords];
+    // diffraction receptions that found no room to wait for their occlusion query (diffract_receive)
+    if (c[kDiffPending] > std::max((paths->record_cap - c[kDiffBase]) / 2, (long long)0))
+        out->records = std::max((long long)out->records, (long long)paths->record_cap + 1);
     out->paths = c[kPaths];
     out->collisions = c[kCollisions];
     out->ntx = paths->ntx;

@@ -446,8 +446,9 @@ __global__ void __launch_bounds__(128) diffract_visible(DiffractArgs A) {
 // Receptions waiting for their occlusion query (diffract_occlusion) are parked at the top of
 // the record array, slot rec_cap - 1 - q for the q-th, while the final records grow from
 // the trace's count n0 at the bottom; parking q < (rec_cap - n0) / 2 of them leaves room for
-// all of them as final records, so the two ends never meet.  Past that bound the launch
-// reports record overflow (the record count is raised above the capacity).
+// all of them as final records, so the two ends never meet.  Those past that bound are only
+// counted, and the host reports a record overflow (sbr_launch_get_stats): the record count on the
+// device stays that of the records written, which is what later kernels read.
 __device__ __forceinline__ long long park_limit(const DiffractArgs &A, long long n0) { return (A.rec_cap - n0) / 2; }
 
 __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
@@ -520,11 +521,7 @@ __global__ void __launch_bounds__(256) diffract_receive(DiffractArgs A) {
             // full warps (here it would run in one lane while the warp waits); the
             // reception is parked with X in its unused face slots 1-3
             const long long pq = (long long)atomicAdd(reinterpret_cast<unsigned long long *>(A.counters + kDiffPending), 1ULL);
-            if (pq >= limit) {
-                atomicMax(reinterpret_cast<unsigned long long *>(A.counters + kRecords),
-                          (unsigned long long)A.rec_cap + 1ULL);
-                continue;
-            }
+            if (pq >= limit) continue;
             RecDev rec;
             rec.tx = txi;
             rec.rx = rx;

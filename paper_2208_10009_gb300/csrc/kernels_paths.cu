@@ -175,6 +175,7 @@ __global__ void records_reset(long long *counters, long long n) {
     counters[kRecords] = n;
     counters[kPaths] = 0;
     counters[kCollisions] = 0;
+    counters[kDiffPending] = 0;
 }
 
 cudaError_t launch_records_reset(long long *counters, long long n, cudaStream_t s) {

@@ -389,7 +389,8 @@ struct DedupArgs {
     int shard_rank, shard_world;   // == shard_rank
 };
 cudaError_t launch_dedup(const DedupArgs &a, int num_sms, cudaStream_t s);
-// counters of a container whose records were replaced: kRecords = n, kPaths = kCollisions = 0
+// counters of a container whose records were replaced: kRecords = n, kPaths = kCollisions =
+// kDiffPending = 0
 cudaError_t launch_records_reset(long long *counters, long long n, cudaStream_t s);
 // counters[kNonFinite] = valid paths with a non-finite output
 cudaError_t launch_nonfinite_scan(const sbr_path_record *paths, long long *counters, int64_t path_cap, int num_sms,
