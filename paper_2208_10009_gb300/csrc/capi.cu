@@ -909,11 +909,11 @@ sbr_status sbr_launch(sbr_ctx *ctx, const sbr_scene *scene, const float *tx, int
     DeviceGuard g(ctx->device);
     PrepArgs prep;   // the ray generation also zeroes the counters and takes device-side transmitters
     prep.counters = paths->counters;
-    const bool tx_on_device = is_local_ptr(ctx, tx);
-    sbr_status st = ensure_tx(ctx, paths, tx_on_device ? nullptr : tx, ntx);
+    const bool read_tx = reinterpret_cast<uintptr_t>(tx) % alignof(float) == 0 && is_local_ptr(ctx, tx);
+    sbr_status st = ensure_tx(ctx, paths, read_tx ? nullptr : tx, ntx);
     if (st != SBR_OK) return st;
     if (capturing(ctx)) paths->tx_held = true;
-    if (tx_on_device) {
+    if (read_tx) {
         prep.tx_src = tx;
         prep.tx = paths->tx;
         prep.ntx = ntx;
