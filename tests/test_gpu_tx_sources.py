@@ -32,3 +32,18 @@ def test_any_address(gpu_ctx, shift):
     assert _sorted(gpu_ctx.records(paths)) == want
     for h in (paths, rxs, scene):
         h.close()
+
+
+def test_many_transmitters(gpu_ctx):
+    """16,384 are read by the ray generation, more are copied."""
+    sc, _, rx = scenes.shoebox_config()
+    scene, rxs, paths = gpu_ctx.scene_from(sc), gpu_ctx.rx_upload(rx), gpu_ctx.paths_create(1 << 20, 1 << 10)
+    t = torch.rand(40_000, 3, device="cuda") * 2 + 0.5
+    for n in (16384, 16385, 40000):
+        got = []
+        for x in (t[:n], t[:n].cpu().numpy()):
+            gpu_ctx.launch(scene, x, rxs, paths, 2, 1, rx_angle_scale=3.0 ** 0.5, records_only=True, sync=True)
+            got.append(_sorted(gpu_ctx.records(paths)))
+        assert got[0] == got[1] and len(got[0]) > 64 * 1000
+    for h in (paths, rxs, scene):
+        h.close()
