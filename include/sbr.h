@@ -340,8 +340,8 @@ typedef struct {
  * sub-rays of an iteration in parallel (one lane: all K in turn, the form for many
  * paths); a group that finishes a path (iteration cap, target reached, stalled) takes the
  * next one from a device work queue (atomic head), so uneven iteration counts do not idle
- * the GPU.  A launch after it runs the FP64 iterations, one path per thread (one per warp while
- * few have them).  From 16 paths an SM on (and always with one lane per path) a launch before it
+ * the GPU.  A launch after it runs the FP64 iterations, one path per thread (shared by
+ * up to 32 lanes while few have them).  From 16 paths an SM on (and always with one lane per path) a launch before it
  * unfolds every path's planes one path per thread, and two last launches walk the paths for the
  * outputs and the points' faces, one path per thread, and test their legs for occlusion, one leg
  * per thread; with fewer, one last launch does both with a warp per path.  Results equal
@@ -402,17 +402,19 @@ sbr_status sbr_paths_import(sbr_ctx *ctx, sbr_paths *paths, const sbr_path_recor
  * of (az, el).  Outputs per path (8 floats): miss[3] = real-space vector from the foot of
  * Rx on the last leg to Rx, delay = |w| / c0, AOD (az, el) of w, AOA (az, el) of the last
  * Tx image minus Rx.  All pointers DEVICE: tx, rx [P][3]; az_el [P][2]; faces [P][8];
- * order [P]; out [P][8]. */
+ * order [P]; out [P][8].  A path with a face id outside [0, nf) gets NaN outputs, and so do paths
+ * whose inputs did not arrive (staged inputs: see sbr_unfold_bwd). */
 sbr_status sbr_unfold_fwd(sbr_ctx *ctx, const sbr_scene *scene, int64_t npaths, const float *tx,
                           const float *rx, const float *az_el, const int32_t *faces, const int32_t *order,
                           float *out);
 /* Vector-Jacobian product of sbr_unfold_fwd: given grad_out [P][8], writes grad_tx,
  * grad_rx [P][3] and grad_az_el [P][2] (DEVICE).  Bounce state is recomputed, not read
- * from the forward pass.  A path with a face id outside [0, nf) gets NaN gradients.  When
- * every input array is 16-byte aligned and there are at least two 256-path tiles per SM,
- * the kernel stages whole tiles of the inputs in shared memory with bulk copies (same
- * results, bit for bit, as the unstaged form); should a tile's copies not arrive within
- * one second, the paths that block had left get NaN gradients instead of a hang. */
+ * from the forward pass.  A path with a face id outside [0, nf) gets NaN gradients.
+ *
+ * Both directions: when every input array is 16-byte aligned and there are at least 16 chunks of
+ * 32 paths per SM, each warp stages chunks of the inputs in shared memory with bulk copies (same
+ * results, bit for bit, as the unstaged form); should a chunk's copies not arrive within one
+ * second, the paths that warp had left get NaN outputs or gradients instead of a hang. */
 sbr_status sbr_unfold_bwd(sbr_ctx *ctx, const sbr_scene *scene, int64_t npaths, const float *tx,
                           const float *rx, const float *az_el, const int32_t *faces, const int32_t *order,
                           const float *grad_out, float *grad_tx, float *grad_rx, float *grad_az_el);

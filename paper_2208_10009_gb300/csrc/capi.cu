@@ -258,10 +258,10 @@ void outgrown(sbr_ctx *ctx, sbr_paths *p, void *mem, size_t bytes, bool &held) {
     held = false;
 }
 
-// The first segments' frontier (frontier_kernel) pays from about two million rays: it takes 45 us
+// The first segments' frontier (frontier_kernel) is made from three million rays traced: it takes 45 us
 // of latency whatever their number, and saves 20 us of a trace of 0.9M rays (street receivers,
-// 10k triangles), 105 of 4.9M, 5.1 ms of 194M (1.07M triangles); and on trees worth skipping (a
-// room of a dozen boxes has four levels).  Past 4 GB of lists (64 places a transmitter take 64
+// 10k triangles; even at about two million), 105 of 4.9M, 5.1 ms of 194M (1.07M triangles); and on
+// trees worth skipping (a room of a dozen boxes has four levels).  Past 4 GB of lists (64 places a transmitter take 64
 // bytes: 4.3e9 first segments) the walks start at the root.
 constexpr int64_t kFrontMinRays = 3000000, kFrontMinNodes = 1024;
 constexpr size_t kFrontMaxBytes = (size_t)4 << 30;

@@ -1435,7 +1435,7 @@ __global__ void __launch_bounds__(256, 3) batch_refine_kernel(RefineArgs A) {
         if (gl != 0) continue;
         sbr_path_record *dst = A.paths + pi;
         if (!x.fail && x.Rf < A.fp64_below_f) {
-            // the FP64 iterations run in batch_refine64_kernel, one thread per path.  The
+            // the FP64 iterations run in batch_refine64_kernel.  The
             // record keeps the iterations done; the path's unf slot keeps the cone centre and
             // |d x W|^2 of the FP32 phase, the record's err field d . W.  With many paths listed
             // by order group (group offsets from batch_unfold_kernel's counts), so that the

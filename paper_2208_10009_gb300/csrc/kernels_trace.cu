@@ -390,7 +390,11 @@ __device__ __forceinline__ BeamAxis beam_axis(float o, float dl, float dh) {
     return b;
 }
 
-// Bounds over the beam of where its rays enter (not before) and leave (not after) a slab.
+// Bounds over the beam of where its rays enter (not before) and leave (not after) a slab.  The intervals
+// of the directions (1e-6 wider on either side) and of their reciprocals (1e-6) cover their own rounding.
+// p - h rounds by 6e-8 of |centre - o| and so bounds the entry to that, the size of what a ray's own slab
+// test loses when it rounds o / d.  (Tx within 1 mm to 1 m of walls, roofs and the ground, 1.3e9 first
+// segments: all segments as from the root.)
 __device__ __forceinline__ void beam_slab(const BeamAxis &b, float c, float h, float &tn, float &tf) {
     const float x = c - b.o, p = b.s == 0.0f ? fabsf(x) : x * b.s;
     const float np = p - h, fp = p + h;
