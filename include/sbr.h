@@ -320,7 +320,7 @@ typedef struct {
  * AOA errors both meet it (§III.B: iterate until the error satisfies the requirement;
  * the AOA error is measured exactly in the unfolded space).  Then the validity test
  * (bounce points inside their faces, no segment occluded) and the outputs (delay, AOD,
- * AOA, power).  One launch, static schedule: a thread per path, or a warp per path while
+ * AOA, power).  One launch, static schedule: a thread per path, or 32 or 8 lanes per path while
  * there are few. */
 sbr_status sbr_refine(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *paths, const sbr_refine_params *params);
 /* Same as sbr_refine restricted to the paths of one (tx, rx) pair: the per-pair form.  The

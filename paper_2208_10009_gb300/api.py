@@ -236,7 +236,7 @@ class Context:
 
     def refine(self, scene: Scene, paths: Paths, max_iters: int, subrays: int = 9, target: float = 0.0,
                fp64_below: float = 1e-5, freq: float = 2.4e9, ptx_dbm: float = 0.0, choice_log=None):
-        """a6-a8, plain form: one launch, a warp per path while there are few, else a thread."""
+        """a6-a8, plain form: one launch, 32 or 8 lanes per path while there are few, else a thread."""
         prm = self._refine_params(max_iters, subrays, target, fp64_below, freq, ptx_dbm, choice_log)
         self._check(self.lib.sbr_refine(self.handle, scene.handle, paths.handle, ctypes.byref(prm)))
 

@@ -1217,10 +1217,13 @@ static sbr_status refine_args(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *p
     // 683 -> 608 us.
     A.split_min = 16LL * std::max(ctx->num_sms, 1);
     A.deep = !A.target_on && A.theta_launch * std::pow(sh, prm->max_iters) < 1e-14;
-    // Plain form, a warp a path up to here (one wave: twelve warps an SM), then a thread a path.  With
-    // a warp / a thread a path: 1,448 paths, 8 iterations (K = 6, none in FP64) 33 / 70 us, 10 in FP64
-    // 163 / 156, 60 in FP64 771 / 930 (K = 16: 781 / 2,911); 4,031 paths 76 / 44, 369 / 105, 1,787 / 539.
+    // Plain form: a warp a path up to one wave of them (twelve warps an SM), 8 lanes a path up to one
+    // wave of those, then a thread.  With 32 / 8 / 1 lanes, 16 iterations, K = 6 (half of them in FP64):
+    // 1,800 paths of a city 199 / 177 / 435 us (6 iterations, none in FP64: 89 / 128 / 359), 2,700 365 / 212
+    // / 442, 7,000 982 / 298 / 488, 10,000 1,457 / 507 / 486; 2,700 paths of a canyon 318 / 177 / 324.  Room
+    // paths run to the double floor (60 iterations): 1,700 625 / 294 / 675, 5,479 1,975 / 607 / 681.
     A.wide_max = 12LL * std::max(ctx->num_sms, 1);
+    A.shared_max = 48LL * std::max(ctx->num_sms, 1);
     A.ntx = paths->ntx;
     A.nrx = paths->nrx;
     A.nf = scene->dev.nf;
@@ -1288,7 +1291,7 @@ sbr_status sbr_refine_pair(sbr_ctx *ctx, const sbr_scene *scene, sbr_paths *path
     A.index = paths->pair_off + npairs + 1;
     {
         Range r("sbr_refine_pair: iterations + validity + outputs");
-        const int per_block = count <= A.wide_max ? 4 : 128;
+        const int per_block = count <= A.wide_max ? 4 : (count <= A.shared_max ? 16 : 128);
         SBR_CUDA(launch_refine(A, (count + per_block - 1) / per_block, 128, ctx->stream));
     }
     return SBR_OK;

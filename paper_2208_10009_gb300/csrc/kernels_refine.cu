@@ -365,6 +365,27 @@ __device__ __forceinline__ bool stalled32(float key, float dw, float Rf, float s
     return atan2f(sqrtf(key), dw) > Rf * stall + 1e-6f;
 }
 
+// The FP64 planes and W of a path by G lanes: a lane per plane and one for the receiver, passed on by
+// shuffles.
+__device__ __forceinline__ void unfold64(const SceneDev &S, const PathGeo &g, UnfD &ud, int G, int gl, unsigned gmask) {
+    if (G == 1) {
+        for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(S, g, j);
+        ud.w = unfold_rx(S, g);
+        return;
+    }
+    const int lane0 = (threadIdx.x & 31) - gl;
+    for (int j0 = 0; j0 <= g.k; j0 += G) {
+        D4 mine = {0.0, 0.0, 0.0, 0.0};
+        if (j0 + gl < g.k) mine = unfold_plane(S, g, j0 + gl);
+        else if (j0 + gl == g.k) mine = unfold_rx(S, g);
+        for (int i = 0; i < G && j0 + i <= g.k; ++i) {
+            const D4 q = {__shfl_sync(gmask, mine.x, lane0 + i), __shfl_sync(gmask, mine.y, lane0 + i),
+                          __shfl_sync(gmask, mine.z, lane0 + i), __shfl_sync(gmask, mine.w, lane0 + i)};
+            (j0 + i < g.k ? ud.p[j0 + i] : ud.w) = q;
+        }
+    }
+}
+
 // Why an iteration loop ended before its cap: the accuracy target met, or the error left
 // the stall bound (a redundant path); recorded where the loop exits, so that the path's
 // flags name the test that stopped it, in the precision it was taken in.
@@ -1260,82 +1281,78 @@ __device__ __forceinline__ void put_iterated(const Iterated &x, dvec3 c, sbr_pat
 }
 
 // a6-a8 in one launch with nothing shared between paths (static schedule): the plain and per-pair
-// forms.  A thread a path, or, up to RefineArgs::wide_max paths, a warp a path: few paths leave the
-// chip idle and a thread's own chain of mirrors, K sub-rays, bounce points and occlusion queries is
-// what the launch waits for, so its lanes take them side by side, as in the batched form's groups (110
-// paths of a cluttered room: 193 -> 45 us).
-__global__ void __launch_bounds__(128) refine_kernel(RefineArgs A) {
-    wait_predecessor();
-    __shared__ SubTab64 tab;
-    __shared__ UnfF s_uf[4];
-    __shared__ UnfD s_ud[4];
-    const long long total = A.range ? (long long)(A.range[1] - A.range[0]) : path_count(A);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    const bool wide = total <= A.wide_max;
+// forms.  A thread a path, or, up to RefineArgs::shared_max paths, 8 lanes a path, and up to wide_max a
+// warp: few paths leave the chip idle and a thread's own chain of mirrors, K sub-rays, bounce points
+// and occlusion queries is what the launch waits for, so lanes take them side by side, as in the
+// batched form's groups (110 paths of a cluttered room: 193 -> 45 us).
+// One path by G lanes (G = 1, 8 or 32; gl, gmask as in iterate64_lanes).
+template <int G>
+__device__ __forceinline__ void refine_path(const RefineArgs &A, long long pi, const SubTab64 &tab, UnfF &uf, int gl,
+                                            unsigned gmask) {
     const int off = c_sub.off[A.K];
     const double shrink = c_sub.shrink[A.K];
     const float shrinkf = c_sub.shrink_f[A.K];
     const double stall = 1.0 / (1.0 - shrink) + 2.0 * shrink;
-    const float stallf = (float)stall;
-    load_sub64(tab);
-    const long long first = wide ? (long long)blockIdx.x * (blockDim.x >> 5) + wid
-                                 : blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long stride = wide ? warps : (long long)gridDim.x * blockDim.x;
-    for (long long i = first; i < total; i += stride) {
-        const long long pi = A.range ? (long long)A.index[A.range[0] + i] : i;
-        sbr_path_record p = A.paths[pi];
-        if (!path_ids_ok(A, p)) {
-            if (!wide || lane == 0) {
-                A.paths[pi].valid = 0;
-                A.paths[pi].flags = SBR_PATH_TRACE_FAIL;
-            }
-            continue;
+    sbr_path_record p = A.paths[pi];
+    if (!path_ids_ok(A, p)) {
+        if (gl == 0) {
+            A.paths[pi].valid = 0;
+            A.paths[pi].flags = SBR_PATH_TRACE_FAIL;
         }
-        PathGeo g;
-        load_path(A, p, g);
-        Iterated x;
-        x.cf = make_float3((float)p.dir[0], (float)p.dir[1], (float)p.dir[2]);
-        x.key = INFINITY;
-        x.dw = 0.0;
+        return;
+    }
+    PathGeo g;
+    load_path(A, p, g);
+    Iterated x;
+    x.cf = make_float3((float)p.dir[0], (float)p.dir[1], (float)p.dir[2]);
+    x.key = INFINITY;
+    x.dw = 0.0;
+    if (G > 1) __syncwarp(gmask);   // the lanes are done with the path before
+    for (int j = gl; j < g.k; j += G) uf.p[j] = unfold_plane32(A.scene, g, j);
+    if (gl == G - 1) uf.w = unfold_rx32(A.scene, g);
+    if (G > 1) __syncwarp(gmask);
+    fp32_phase<G>(A, g, uf, off, p.rough_err, shrinkf, (float)stall, pi, gl, gmask, x);
+    dvec3 c = dv(x.cf.x, x.cf.y, x.cf.z);
+    if (!x.fail && x.Rf < A.fp64_below_f) {
         UnfD ud;
-        if (wide) {
-            UnfF &uf = s_uf[wid];
-            __syncwarp();
-            if (lane < g.k) uf.p[lane] = unfold_plane32(A.scene, g, lane);
-            if (lane == 31) uf.w = unfold_rx32(A.scene, g);
-            __syncwarp();
-            fp32_phase<32>(A, g, uf, off, p.rough_err, shrinkf, stallf, pi, lane, 0xffffffffu, x);
+        unfold64(A.scene, g, ud, G, gl, gmask);
+        fp64_phase<(G > 1)>(A, g, ud, off, tab, p, shrink, stall, pi, G, gl, gmask, x);
+        c = x.c;
+    }
+    put_iterated(x, c, p);
+    const double bound = converged_bound(x.it, cone_radius64(A, p.rough_err, x.it, shrink));
+    if (G > 1) group_finalize<G>(A, g, c, p, gl, gmask, bound);
+    else finalize_path(A, g, c, p, bound);
+    if (gl == 0) store_result(A.paths + pi, p);
+}
+
+// The same as a function of its own.  Inlined beside the others, the 8-lane and thread forms ran 1.4 to 2
+// times as long with the same registers (2,700 canyon paths, 16 iterations, 410 -> 177 us, a thread each
+// 808 -> 310; a warp a path is faster inlined, 49 -> 45 us).
+template <int G>
+__device__ __noinline__ void refine_path_apart(const RefineArgs &A, long long pi, const SubTab64 &tab, UnfF &uf, int gl,
+                                               unsigned gmask) {
+    refine_path<G>(A, pi, tab, uf, gl, gmask);
+}
+
+__global__ void __launch_bounds__(128, 3) refine_kernel(const __grid_constant__ RefineArgs A) {
+    wait_predecessor();
+    __shared__ SubTab64 tab;
+    __shared__ UnfF s_uf[16];
+    const long long total = A.range ? (long long)(A.range[1] - A.range[0]) : path_count(A);
+    load_sub64(tab);
+    const int G = total <= A.wide_max ? 32 : (total <= A.shared_max ? 8 : 1);   // lanes a path
+    const int lane = threadIdx.x & 31, gl = lane & (G - 1), slot = threadIdx.x / G;
+    const long long stride = (long long)gridDim.x * blockDim.x / G;
+    for (long long i = (long long)blockIdx.x * (blockDim.x / G) + slot; i < total; i += stride) {
+        const long long pi = A.range ? (long long)A.index[A.range[0] + i] : i;
+        if (G == 32) {
+            refine_path<32>(A, pi, tab, s_uf[slot], gl, 0xffffffffu);
+        } else if (G == 8) {
+            refine_path_apart<8>(A, pi, tab, s_uf[slot], gl, 0xffu << (lane - gl));
         } else {
             UnfF uf;
-            for (int j = 0; j < g.k; ++j) uf.p[j] = unfold_plane32(A.scene, g, j);
-            uf.w = unfold_rx32(A.scene, g);
-            fp32_phase<1>(A, g, uf, off, p.rough_err, shrinkf, stallf, pi, 0, 0, x);
-        }
-        dvec3 c = dv(x.cf.x, x.cf.y, x.cf.z);
-        if (!x.fail && x.Rf < A.fp64_below_f) {
-            if (wide) {
-                if (lane < g.k) s_ud[wid].p[lane] = unfold_plane(A.scene, g, lane);
-                if (lane == 31) s_ud[wid].w = unfold_rx(A.scene, g);
-                __syncwarp();
-                for (int j = 0; j < g.k; ++j) ud.p[j] = s_ud[wid].p[j];
-                ud.w = s_ud[wid].w;
-            } else {
-                for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
-                ud.w = unfold_rx(A.scene, g);
-            }
-            if (wide) fp64_phase<true>(A, g, ud, off, tab, p, shrink, stall, pi, 32, lane, 0xffffffffu, x);
-            else fp64_phase<false>(A, g, ud, off, tab, p, shrink, stall, pi, 1, 0, 0, x);
-            c = x.c;
-        }
-        put_iterated(x, c, p);
-        const double bound = converged_bound(x.it, cone_radius64(A, p.rough_err, x.it, shrink));
-        if (wide) {
-            group_finalize<32>(A, g, c, p, lane, 0xffffffffu, bound);
-            if (lane == 0) store_result(A.paths + pi, p);
-        } else {
-            finalize_path(A, g, c, p, bound);
-            store_result(A.paths + pi, p);
+            refine_path_apart<1>(A, pi, tab, uf, 0, 0);
         }
     }
 }
@@ -1516,22 +1533,7 @@ __global__ void __launch_bounds__(kTailBlock) batch_refine64_kernel(RefineArgs A
         PathGeo g;
         load_path(A, p, g);
         UnfD ud;
-        if (G > 1) {   // a lane per plane and one for the receiver, passed on by shuffles
-            for (int j0 = 0; j0 <= g.k; j0 += G) {
-                D4 mine = {0.0, 0.0, 0.0, 0.0};
-                if (j0 + gl < g.k) mine = unfold_plane(A.scene, g, j0 + gl);
-                else if (j0 + gl == g.k) mine = unfold_rx(A.scene, g);
-                for (int i = 0; i < G && j0 + i <= g.k; ++i) {
-                    const int src = lane - gl + i;
-                    const D4 q = {__shfl_sync(gmask, mine.x, src), __shfl_sync(gmask, mine.y, src),
-                                  __shfl_sync(gmask, mine.z, src), __shfl_sync(gmask, mine.w, src)};
-                    (j0 + i < g.k ? ud.p[j0 + i] : ud.w) = q;
-                }
-            }
-        } else {
-            for (int j = 0; j < g.k; ++j) ud.p[j] = unfold_plane(A.scene, g, j);
-            ud.w = unfold_rx(A.scene, g);
-        }
+        unfold64(A.scene, g, ud, G, gl, gmask);
         const float4 cu = A.unf[kUnfStride * pi + kMaxOrder + 1];
         Iterated x;
         x.cf = f3(cu);

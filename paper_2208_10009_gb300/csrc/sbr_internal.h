@@ -432,7 +432,8 @@ struct RefineArgs {
                               // paths walked one thread per path, legs queried one thread each
     int num_sms;
     int deep;                 // the iterations run to the double floor (no target, last cone below 1e-14 rad)
-    long long wide_max;       // plain and per-pair form: up to this many paths a warp each, then a thread
+    // plain and per-pair form: up to so many paths 32 lanes each, up to so many 8, then a thread
+    long long wide_max, shared_max;
     int ntx, nrx, nf, nw;     // bounds of the ids a path record may hold
 };
 cudaError_t launch_refine(const RefineArgs &a, int grid, int block, cudaStream_t s);

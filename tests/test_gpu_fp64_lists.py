@@ -1,7 +1,7 @@
 """FP64 iterations of short lists: the tail of the batched refinement shares a path among 32 to 4
-lanes, by the list's length and the iterations to come, and longer lists take a thread a path.  Every
-length makes the decisions and results of the longest list's form, bit for bit, and a list takes no
-longer than one many times as long."""
+lanes, by the list's length and the iterations to come, the plain form among 32 or 8, and longer
+lists take a thread a path.  Every length makes the decisions and results of the longest list's form,
+bit for bit, and a list takes no longer than one many times as long."""
 import numpy as np
 import pytest
 import torch
@@ -16,7 +16,7 @@ PER_SM = 4 * 32   # lanes of the warps that a list in shared lanes may have an S
 
 
 def _rough(ctx, nrx):
-    """Scene, transmitter, receivers, their rough paths of a room (over 60 a receiver) and a container."""
+    """Scene, transmitter, receivers, their rough paths of a room (about 63 a receiver) and a container."""
     sc, tx, _ = scenes.shoebox_config()
     rng = np.random.default_rng(nrx)
     rx = scenes.f32_exact(rng.uniform([0.4, 0.4, 0.4], [9.6, 7.6, 2.6], (nrx, 3)))
@@ -39,12 +39,12 @@ def _refined(ctx, scene, tx, rxs, rough, paths, K, iters, lanes):
 
 @pytest.mark.parametrize("K,iters", [(6, 60), (7, 12), (9, 44), (16, 60), (16, 1)])
 def test_lengths_alike(gpu_ctx, K, iters):
-    scene, tx, rxs, rough, paths = _rough(gpu_ctx, 90)
+    scene, tx, rxs, rough, paths = _rough(gpu_ctx, 130)
     sms = gpu_ctx.num_sms
     lines = [PER_SM * sms // g for g in (32, 16, 8, 4)]   # the longest list of each number of lanes
-    assert len(rough) > lines[-1] + 33
+    assert len(rough) > 48 * sms + 33
     want, choice = _refined(gpu_ctx, scene, tx, rxs, rough, paths, K, iters, 16)
-    for n in [1, 33, 12 * sms, 12 * sms + 1] + lines + [x + 1 for x in lines]:
+    for n in [1, 33, 12 * sms, 12 * sms + 1, 48 * sms, 48 * sms + 1] + lines + [x + 1 for x in lines]:
         for lanes in (16, 1, 0):   # 0: the plain form
             got, log = _refined(gpu_ctx, scene, tx, rxs, rough[:n], paths, K, iters, lanes)
             assert np.array_equal(log, choice[:n]), (n, lanes)
