@@ -1285,6 +1285,13 @@ __device__ __forceinline__ void put_iterated(const Iterated &x, dvec3 c, sbr_pat
 // warp: few paths leave the chip idle and a thread's own chain of mirrors, K sub-rays, bounce points
 // and occlusion queries is what the launch waits for, so lanes take them side by side, as in the
 // batched form's groups (110 paths of a cluttered room: 193 -> 45 us).
+// (Called, so that its traversal stacks and those of refine_path_apart share their place: 1,840 bytes a
+// thread where inlined 2,256, for which a context sets 120 MB more aside.)
+__device__ __noinline__ void finalize_apart(const RefineArgs &A, const PathGeo &g, dvec3 c, sbr_path_record &p, int gl,
+                                            double bound) {
+    group_finalize<32>(A, g, c, p, gl, 0xffffffffu, bound);
+}
+
 // One path by G lanes (G = 1, 8 or 32; gl, gmask as in iterate64_lanes).
 template <int G>
 __device__ __forceinline__ void refine_path(const RefineArgs &A, long long pi, const SubTab64 &tab, UnfF &uf, int gl,
@@ -1321,7 +1328,8 @@ __device__ __forceinline__ void refine_path(const RefineArgs &A, long long pi, c
     }
     put_iterated(x, c, p);
     const double bound = converged_bound(x.it, cone_radius64(A, p.rough_err, x.it, shrink));
-    if (G > 1) group_finalize<G>(A, g, c, p, gl, gmask, bound);
+    if (G == 32) finalize_apart(A, g, c, p, gl, bound);
+    else if (G > 1) group_finalize<G>(A, g, c, p, gl, gmask, bound);
     else finalize_path(A, g, c, p, bound);
     if (gl == 0) store_result(A.paths + pi, p);
 }
