@@ -111,13 +111,23 @@ sbr_status ensure_lattice(sbr_ctx *ctx, int n) {
         ctx->lattice_bytes = 0;
         ctx->lattice_held = false;
     }
-    for (size_t i = 0; i < ctx->held_lattices.size(); ++i) {
+    // this division level's held tables if there are some, their place taken by the block in use (n = 0:
+    // held by no launch); else that spare
+    for (int level : {n, 0}) {
+        if (level == 0 && ctx->lattice_mem) break;
+        size_t i = 0;
+        while (i < ctx->held_lattices.size() && ctx->held_lattices[i].tables.n != level) ++i;
+        if (i == ctx->held_lattices.size()) continue;
         const sbr_ctx::HeldLattice h = ctx->held_lattices[i];
-        if (h.tables.n != n) continue;
-        dev_free(ctx, ctx->lattice_mem, ctx->lattice_bytes);
-        ctx->held_lattices.erase(ctx->held_lattices.begin() + i);
+        if (ctx->lattice_mem) {
+            ctx->held_lattices[i] = {ctx->lattice_mem, ctx->lattice_bytes, ctx->lattice};
+            ctx->held_lattices[i].tables.n = 0;
+        } else {
+            ctx->held_lattices.erase(ctx->held_lattices.begin() + i);
+        }
         ctx->lattice_mem = h.mem;
         ctx->lattice_bytes = h.bytes;
+        if (level == 0) break;
         ctx->lattice = h.tables;
         ctx->lattice_n = n;
         ctx->lattice_held = true;
@@ -211,16 +221,23 @@ sbr_status ensure_dirs(sbr_ctx *ctx, int n, int launcher, const PrepArgs &prep) 
             ctx->dirs_bytes = 0;
             ctx->dirs_held = ctx->dirs_valid = false;
         }
-        for (size_t i = 0; i < ctx->held_dirs.size(); ++i) {
+        // this division level's held block if there is one, its place taken by the block in use (n = 0: held by
+        // no launch); else that spare
+        for (int level : {n, 0}) {
+            if (level == 0 && ctx->dirs) break;
+            size_t i = 0;
+            while (i < ctx->held_dirs.size() &&
+                   (ctx->held_dirs[i].n != level || (level && ctx->held_dirs[i].launcher != launcher)))
+                ++i;
+            if (i == ctx->held_dirs.size()) continue;
             const sbr_ctx::HeldDirs h = ctx->held_dirs[i];
-            if (h.n != n || h.launcher != launcher) continue;
-            dev_free(ctx, ctx->dirs, ctx->dirs_bytes);
-            ctx->held_dirs.erase(ctx->held_dirs.begin() + i);
+            if (ctx->dirs) ctx->held_dirs[i] = {ctx->dirs, ctx->dirs_bytes, 0, 0};
+            else ctx->held_dirs.erase(ctx->held_dirs.begin() + i);
             ctx->dirs = h.mem;
             ctx->dirs_bytes = h.bytes;
             ctx->dirs_n = n;
             ctx->dirs_launcher = launcher;
-            ctx->dirs_held = true;
+            ctx->dirs_held = level != 0;
             break;
         }
     }

@@ -18,12 +18,13 @@ class Blocks:
     """The device blocks that the library holds."""
 
     def __init__(self, monkeypatch):
-        self.live, self.freed = set(), []
+        self.live, self.freed, self.allocs = set(), [], 0
         alloc, free = torch.cuda.caching_allocator_alloc, torch.cuda.caching_allocator_delete
 
         def _alloc(*a):
             p = alloc(*a)
             self.live.add(p)
+            self.allocs += 1
             return p
 
         def _free(p):
@@ -86,10 +87,11 @@ def test_blocks_stay_for_replays(monkeypatch, launcher):
         # records of the replay's launch removed of double counts on this context: its own directions
         count = ctx.launch_stats(mine)["records"]
         step(one, mine, 24)
-        held = len(blocks.live)
-        for n in (33, 24, 57, 24):
+        step(one, mine, 57)
+        held = len(blocks.live), blocks.allocs
+        for n in (33, 24, 57, 24, 33, 57, 24):   # back and forth: no block made or given back
             step(one, mine, n)
-        assert len(blocks.live) == held and count == ctx.launch_stats(mine)["records"]
+        assert (len(blocks.live), blocks.allocs) == held and count == ctx.launch_stats(mine)["records"]
         assert _rows(ctx, mine).tobytes() == want.tobytes()
         graph.replay()
         torch.cuda.synchronize()
