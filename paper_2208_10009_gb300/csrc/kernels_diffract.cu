@@ -98,7 +98,7 @@ __device__ __forceinline__ bool cone_box(float lx, float ly, float lz, float hx,
 // and only the pairs left run the exact test, a ray per lane.  Where the group does not bundle
 // (a beam past kMaxBeam: vertex rays, the ends of the icosahedron's edges, coarse lattices), each
 // 32 places make a beam, and where those do not either, each lane walks the tree for its own ray.  Per-ray walks took 3,300 warp instructions for 32 rays of the canyon
-// (n = 700, 2,000 faces' wedges, 4.9M rays: 687 us); beams take 670 and the exact tests 170 (170 + 41
+// (n = 700, 2,000 faces' wedges, 4.9M rays: 687 us); beams take 670 and the exact tests 170 (179 + 42
 // us; groups of 64 / 256 places: 226 / 239 us).
 constexpr int kGroup = 128, kSub = 32, kSubs = kGroup / kSub;
 constexpr int kBeamStack = 512, kBeamList = 128;   // nodes to visit, wedges to test of a warp
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(128) diffract_visible(DiffractArgs A) {
 // compared with it in the frame of the edge, where the test is two products and needs no sector,
 // arc tangent or exact root (60 -> 30 instructions a receiver).  A warp used to take 32
 // candidates, whose unlike loops left 21 % of the warp slots in use: with the
-// visibility queries inside 186 us, now 42 (diffract_visible) + 77 us (canyon, 240k candidates, 256
+// visibility queries inside 186 us, now 42 (diffract_visible) + 71 us (canyon, 240k candidates, 256
 // receivers).
 // Receptions waiting for their occlusion query (diffract_occlusion) are parked at the top of
 // the record array, slot rec_cap - 1 - q for the q-th, while the final records grow from
